@@ -245,13 +245,13 @@ static KArgs base_args(const tdse_ctx* c) {
     a.k1d_lo = opt<float2>(c, c->off.k1lo);
     a.k1d_hi = opt<float2>(c, c->off.k1hi);
     a.a1d = opt<float2>(c, c->off.a1d);
-    a.tw64_0 = c->P<double2>(c->off.tw64_0);
+    a.tw64_0 = c->P<int4>(c->off.tw64_0);
     a.tw32_0 = c->P<float2>(c->off.tw32_0);
-    a.tw64_1 = c->P<double2>(c->off.tw64_1);
+    a.tw64_1 = c->P<int4>(c->off.tw64_1);
     a.tw32_1 = c->P<float2>(c->off.tw32_1);
     a.tw32lo_0 = c->P<float2>(c->off.tw32lo_0);
     a.tw32lo_1 = c->P<float2>(c->off.tw32lo_1);
-    a.tw64_2 = c->P<double2>(c->off.tw64_2);
+    a.tw64_2 = c->P<int4>(c->off.tw64_2);
     a.tw32_2 = c->P<float2>(c->off.tw32_2);
     a.tw32lo_2 = c->P<float2>(c->off.tw32lo_2);
     if (c->four1d) {   // 1D through the 2D passes: geometry fs0 x fs1, tables of the N-point grid
@@ -317,6 +317,22 @@ static tdse_status build_phase_tables(tdse_ctx* c, int b, cudaStream_t s) {
             TDSE_CK(c, launch_e2d(c->P<float2>(c->off.e2d) + b * nsp1 * c->ntab, phi, c->ntf, c->cfg.nsteps, c->n0,
                                   c->n1, n2t, c->cfg.dt, s));
     }
+    return TDSE_OK;
+}
+
+// The twiddle tables of a periodic context (functions of the grid alone).
+static tdse_status build_twiddles(tdse_ctx* c, cudaStream_t s) {
+    auto axis = [&](size_t t64, size_t t32, size_t t32lo, int n) {
+        return launch_twiddles(c->P<int4>(t64), c->P<float2>(t32), c->P<float2>(t32lo), n, s);
+    };
+    TDSE_CK(c, axis(c->off.tw64_0, c->off.tw32_0, c->off.tw32lo_0, c->four1d ? c->fs0 : c->n0));
+    if (c->four1d) {
+        TDSE_CK(c, axis(c->off.tw64_1, c->off.tw32_1, c->off.tw32lo_1, c->fs1));
+        TDSE_CK(c, launch_roots(c->P<double2>(c->off.tw1d64), c->P<float2>(c->off.tw1d32), c->n0, s));
+    }
+    if (c->d >= 2) TDSE_CK(c, axis(c->off.tw64_1, c->off.tw32_1, c->off.tw32lo_1, c->n1));
+    if (c->d == 3) TDSE_CK(c, axis(c->off.tw64_2, c->off.tw32_2, c->off.tw32lo_2, c->n2));
+    if (c->off.tw128) TDSE_CK(c, launch_four_step_tables(c->P<int4>(c->off.tw128), s));
     return TDSE_OK;
 }
 
@@ -473,25 +489,12 @@ tdse_status tdse_bind_workspace(tdse_ctx* c, void* dev, size_t bytes, void* stre
         tdse_status st = fs_bind(c, s);
         if (st != TDSE_OK) return st;
     } else {
-    TDSE_CK(c, launch_twiddles(c->P<double2>(c->off.tw64_0), c->P<float2>(c->off.tw32_0),
-                               c->P<float2>(c->off.tw32lo_0), c->four1d ? c->fs0 : c->n0, s));
-    if (c->four1d) {
-        TDSE_CK(c, launch_twiddles(c->P<double2>(c->off.tw64_1), c->P<float2>(c->off.tw32_1),
-                                   c->P<float2>(c->off.tw32lo_1), c->fs1, s));
-        TDSE_CK(c, launch_twiddles(c->P<double2>(c->off.tw1d64), c->P<float2>(c->off.tw1d32),
-                                   c->P<float2>(c->off.tw1d32lo), c->n0, s));
-    }
-    if (c->d == 3)
-        TDSE_CK(c, launch_twiddles(c->P<double2>(c->off.tw64_2), c->P<float2>(c->off.tw32_2),
-                                   c->P<float2>(c->off.tw32lo_2), c->n2, s));
-    if (c->d >= 2)
-        TDSE_CK(c, launch_twiddles(c->P<double2>(c->off.tw64_1), c->P<float2>(c->off.tw32_1),
-                                   c->P<float2>(c->off.tw32lo_1), c->n1, s));
-    else
+    tdse_status ts = build_twiddles(c, s);
+    if (ts != TDSE_OK) return ts;
+    if (c->d == 1)
         TDSE_CK(c, launch_kin1d(opt<double2>(c, c->off.kin64), opt<float4>(c, c->off.kinff), c->n0, c->L, c->cfg.dt, s));
     if (c->d == 1 && c->mixed)
         TDSE_CK(c, launch_k1d(c->P<float2>(c->off.k1lo), c->P<float2>(c->off.k1hi), c->nhi, c->n0, c->cfg.dt, s));
-    if (c->off.tw128) TDSE_CK(c, launch_four_step_tables(c->P<double2>(c->off.tw128), s));
     TDSE_CK(c, cudaMemsetAsync(c->P<int>(c->off.err), 0, sizeof(int), s));
     c->cl_ok = false;
     if (c->off.cl_tab) {
@@ -740,7 +743,7 @@ static tdse_status do_init(tdse_ctx* c, cudaStream_t s) {
     a.out_slot = slot_of(c, 0);
     set_time(c, a, 0);
     if (c->off.tw128)
-        TDSE_CK(c, launch_four_step_init(a, c->P<double2>(c->off.tw128), s));
+        TDSE_CK(c, launch_four_step_init(a, c->P<int4>(c->off.tw128), s));
     else
         TDSE_CK(c, run(c, a, f64_combo(c), s));
     c->inited = true;
@@ -1059,7 +1062,7 @@ tdse_status tdse_read_u(tdse_ctx* c, int instance, double* u_out, int where, voi
         a.ip = c->ip ? 1 : 0;
         a.e_step = c->step;
         if (c->off.tw128)
-            TDSE_CK(c, launch_four_step_read(a, c->P<double2>(c->off.tw128), s));
+            TDSE_CK(c, launch_four_step_read(a, c->P<int4>(c->off.tw128), s));
         else
             TDSE_CK(c, run(c, a, f64_combo(c), s));
         src = a.aux2;
@@ -1214,6 +1217,10 @@ tdse_status tdse_load(tdse_ctx* c, const void* blob, size_t size, void* stream) 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const char* in = static_cast<const char*>(blob);
     TDSE_CK(c, cudaMemcpyAsync(c->ws, in + sizeof(h) + 2 * (size_t)c->B, c->ws_need, cudaMemcpyHostToDevice, s));
+    // the transform tables depend on the configuration alone and are built by
+    // this library: those of the checkpoint may be another version's
+    const tdse_status ts = c->fs ? fs_upload_twiddles(c, s) : build_twiddles(c, s);
+    if (ts != TDSE_OK) return ts;
     TDSE_CK(c, cudaStreamSynchronize(s));
     for (int b = 0; b < c->B; ++b) {
         c->have_V[b] = in[sizeof(h) + 2 * b];

@@ -23,11 +23,16 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "fx.cuh"
+
 namespace tdse {
 
+// Real type, and the type of a twiddle table's entries: FP64 transforms run
+// in 64-bit fixed point (fx.cuh).
 template <class C> struct cx_traits;
-template <> struct cx_traits<double2> { using real = double; };
-template <> struct cx_traits<float2> { using real = float; };
+template <> struct cx_traits<double2> { using real = double; using tw = int4; };
+template <> struct cx_traits<float2> { using real = float; using tw = float2; };
+template <class C> using tw_t = typename cx_traits<C>::tw;
 
 __device__ __forceinline__ double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 operator-(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
@@ -55,7 +60,7 @@ template <> __device__ __forceinline__ double2 czero<double2>() { return make_do
 template <> __device__ __forceinline__ float2 czero<float2>() { return make_float2(0.f, 0.f); }
 
 // multiply by -i (forward) or +i (inverse)
-template <bool INV, class C> __device__ __forceinline__ C rot90(C a) {
+template <bool INV, class C> FX_HD C rot90(C a) {
     C r;
     if (INV) { r.x = -a.y; r.y = a.x; } else { r.x = a.y; r.y = -a.x; }
     return r;
@@ -64,12 +69,9 @@ template <bool INV, class C> __device__ __forceinline__ C rot90(C a) {
 // multiply by e^{-+ i pi/4} = (1 -+ i)/sqrt(2).  In FP32 the constant is
 // applied as hi + lo so that the butterfly has no fixed rounding of 1/sqrt(2)
 // (a rounding repeated identically at every step would bias the transform).
-template <bool INV> __device__ __forceinline__ double2 rot45(double2 a) {
-    const double s = 0.70710678118654752440;
-    double2 r;
-    if (INV) { r.x = (a.x - a.y) * s; r.y = (a.x + a.y) * s; }
-    else     { r.x = (a.x + a.y) * s; r.y = (a.y - a.x) * s; }
-    return r;
+template <bool INV> FX_HD longlong2 rot45(longlong2 a) {
+    const long long u = INV ? a.x - a.y : a.x + a.y, v = INV ? a.x + a.y : a.y - a.x;
+    return make_longlong2(fx_times_rsqrt2(u), fx_times_rsqrt2(v));
 }
 template <bool INV> __device__ __forceinline__ float2 rot45(float2 a) {
     const float sh = 0.707106769084930419921875f;          // float(1/sqrt 2)
@@ -79,16 +81,16 @@ template <bool INV> __device__ __forceinline__ float2 rot45(float2 a) {
     return make_float2(fmaf(u, sh, u * sl), fmaf(v, sh, v * sl));
 }
 
-template <bool INV, class C> __device__ __forceinline__ void dft2(C* v) {
+template <bool INV, class C> FX_HD void dft2(C* v) {
     C t = v[0] - v[1]; v[0] = v[0] + v[1]; v[1] = t;
 }
 
-template <bool INV, class C> __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3) {
+template <bool INV, class C> FX_HD void dft4(C& a0, C& a1, C& a2, C& a3) {
     C t0 = a0 + a2, t1 = a0 - a2, t2 = a1 + a3, t3 = rot90<INV>(a1 - a3);
     a0 = t0 + t2; a2 = t0 - t2; a1 = t1 + t3; a3 = t1 - t3;
 }
 
-template <bool INV, class C> __device__ __forceinline__ void dft8(C* v) {
+template <bool INV, class C> FX_HD void dft8(C* v) {
     C e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
     C o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
     dft4<INV>(e0, e1, e2, e3);
@@ -102,7 +104,7 @@ template <bool INV, class C> __device__ __forceinline__ void dft8(C* v) {
     v[3] = e3 + o3; v[7] = e3 - o3;
 }
 
-template <int R, bool INV, class C> __device__ __forceinline__ void dft_r(C* v) {
+template <int R, bool INV, class C> FX_HD void dft_r(C* v) {
     if constexpr (R == 2) dft2<INV>(v);
     else if constexpr (R == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
     else dft8<INV>(v);
@@ -124,13 +126,7 @@ template <int N, bool INV> struct FftPlan {
     static constexpr int ns(int s) { return s == 0 ? 1 : ns(s - 1) * radix(s - 1); }
 };
 
-// v * w (w from tw, conjugated for the inverse); FP32 adds the residual table.
-template <bool INV> __device__ __forceinline__ double2 twiddle(double2 v, const double2* __restrict__ tw,
-                                                               const double2*, int idx) {
-    double2 w = __ldg(&tw[idx]);
-    if (INV) w.y = -w.y;
-    return cmul(v, w);
-}
+// v * w (w from tw, conjugated for the inverse).
 // TDSE_TWIDDLE_LO = 1 applies the FP32 twiddle as hi + lo.  Off by default:
 // on the 512^2 mixed workload it lowers the 2000-step error from 5.1e-7 to
 // 4.4e-7 at a 7% cost in step time.
@@ -169,8 +165,8 @@ struct GroupSync {
 // L interleaved length-N transforms by T threads (thread index tid in 0..T-1
 // of the group, barrier `sync`); element (pos, line) at buf[pos * PS + line].
 // Item it of a pass with NB butterflies is butterfly j = it / L of line it % L.
-template <class C, int N, int L, int PS, int T, bool INV>
-struct Fft {
+template <int N, int L, int T, bool INV>
+struct FftShape {
     using Plan = FftPlan<N, INV>;
     static constexpr int NPASS = Plan::NPASS;
     static constexpr int RF = Plan::radix(0);
@@ -186,6 +182,20 @@ struct Fft {
         j = it / L;
         return ((NB * L) % T == 0) || it < NB * L;
     }
+};
+
+template <class C, int N, int L, int PS, int T, bool INV>
+struct Fft : FftShape<N, L, T, INV> {
+    using Shape = FftShape<N, L, T, INV>;
+    using Plan = FftPlan<N, INV>;
+    using Shape::item;
+    using Shape::NBF;
+    using Shape::NBL;
+    using Shape::NPASS;
+    using Shape::PF;
+    using Shape::PL;
+    using Shape::RF;
+    using Shape::RL;
 
     template <int S, class Sync>
     __device__ static __forceinline__ void mid_pass(C* buf, const C* __restrict__ tw, const C* __restrict__ twl,
@@ -355,6 +365,234 @@ struct CtaFft {
     }
     __device__ static __forceinline__ void run(C* buf, const C* __restrict__ tw, const C* __restrict__ twl) {
         pass<0>(buf, tw, twl);
+    }
+};
+
+// ---------------------------------------------------------------------------
+// The same two transforms for FP64 values, in 64-bit fixed point (fx.cuh): tw
+// holds int4 table factors, buf holds FP64 values outside a transform and
+// integers inside.  The results are multiplied by 2^lg on the way out (exact).
+//
+// Pass S of radix R with its butterflies' values in v: twiddle and 1/R for
+// S > 0, then the R-point DFT.
+template <int N, bool INV>
+struct FxPass {
+    using Plan = FftPlan<N, INV>;
+    static constexpr int S0 = 62 - ilog2(Plan::radix(0));       // input scale
+    static constexpr int GAIN = ilog2(N / Plan::radix(0));      // the passes' 1/R
+    template <int S>
+    FX_HD static void butterfly(longlong2* v, int j, const int4* __restrict__ tw) {
+        constexpr int R = Plan::radix(S);
+        if constexpr (S > 0) {
+            constexpr int Ns = Plan::ns(S), LR = ilog2(R), stride = N / (Ns * R);
+            const int k = j & (Ns - 1);
+            v[0].x = (v[0].x + (1ll << (LR - 1))) >> LR;
+            v[0].y = (v[0].y + (1ll << (LR - 1))) >> LR;
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = fx_mul<INV, 3 - LR>(v[r], fx_ldg(&tw[k * r * stride]));
+        }
+        dft_r<R, INV>(v);
+    }
+    // exponent of the results for block exponent E (of the largest high word mx)
+    FX_HD static int out_exp(unsigned mx, int E, int lg) {
+        return mx >= 0x7ff00000u ? FX_NAN : E - 1022 - S0 + GAIN + lg;
+    }
+};
+
+template <int N, int L, int LS, int T, bool INV>
+struct CtaFft<double2, N, L, LS, T, INV> {
+    using Fx = FxPass<N, INV>;
+    using Plan = FftPlan<N, INV>;
+    template <int S>
+    __device__ static __forceinline__ void pass(longlong2* buf, const int4* __restrict__ tw, int X) {
+        if constexpr (S < Plan::NPASS) {
+            constexpr int R = Plan::radix(S), Ns = Plan::ns(S), NB = N / R, ITEMS = NB * L, PER = (ITEMS + T - 1) / T;
+            longlong2 v[PER][R];
+#pragma unroll
+            for (int p = 0; p < PER; ++p) {
+                const int it = threadIdx.x + p * T;
+                if (ITEMS % T == 0 || it < ITEMS) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) v[p][r] = buf[(it / L + r * NB) * LS + it % L];
+                }
+            }
+            __syncthreads();
+            store<S, PER, R, Ns>(buf, tw, v, X);
+            __syncthreads();
+            pass<S + 1>(buf, tw, X);
+        }
+    }
+    template <int S, int PER, int R, int Ns>
+    __device__ static __forceinline__ void store(longlong2* buf, const int4* __restrict__ tw, longlong2 (&v)[PER][R],
+                                                 int X) {
+        constexpr int ITEMS = N / R * L;
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            const int it = threadIdx.x + p * T;
+            if (ITEMS % T == 0 || it < ITEMS) {
+                const int line = it % L, j = it / L, k = j & (Ns - 1);
+                Fx::template butterfly<S>(v[p], j, tw);
+                longlong2* out = buf + ((j - k) * R + k) * LS + line;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if constexpr (S == Plan::NPASS - 1) reinterpret_cast<double2*>(out)[r * Ns * LS] = fx_to(v[p][r], X);
+                    else out[r * Ns * LS] = v[p][r];
+                }
+            }
+        }
+    }
+    __device__ static __forceinline__ void run(double2* dbuf, const int4* __restrict__ tw, const int4*, int lg = 0) {
+        constexpr int R = Plan::radix(0), NB = N / R, ITEMS = NB * L, PER = (ITEMS + T - 1) / T;
+        longlong2* buf = reinterpret_cast<longlong2*>(dbuf);
+        double2 x[PER][R];
+        unsigned mx = 0;
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            const int it = threadIdx.x + p * T;
+            if (ITEMS % T == 0 || it < ITEMS) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    x[p][r] = dbuf[(it / L + r * NB) * LS + it % L];
+                    mx = max(mx, fx_hi(x[p][r]));
+                }
+            }
+        }
+        mx = fx_cta_max<T>(mx);                 // its barrier also orders the loads above before the stores below
+        if constexpr (T <= 32) __syncwarp();
+        const int E = fx_exponent(mx), X = Fx::out_exp(mx, E, lg);
+        longlong2 v[PER][R];
+#pragma unroll
+        for (int p = 0; p < PER; ++p)
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[p][r] = fx_from(x[p][r], Fx::S0, E);
+        store<0, PER, R, 1>(buf, tw, v, X);
+        __syncthreads();
+        pass<1>(buf, tw, X);
+    }
+};
+
+template <int N, int L, int PS, int T, bool INV>
+struct Fft<double2, N, L, PS, T, INV> : FftShape<N, L, T, INV> {
+    using Shape = FftShape<N, L, T, INV>;
+    using Fx = FxPass<N, INV>;
+    using Plan = FftPlan<N, INV>;
+    using Shape::item;
+    using Shape::NBF;
+    using Shape::NBL;
+    using Shape::NPASS;
+    using Shape::PF;
+    using Shape::PL;
+    using Shape::RF;
+    using Shape::RL;
+
+    template <int S, class Sync>
+    __device__ static __forceinline__ void mids(longlong2* buf, const int4* __restrict__ tw, int tid, const Sync& sync) {
+        if constexpr (S <= NPASS - 2) {
+            constexpr int R = Plan::radix(S), Ns = Plan::ns(S), NB = N / R, PER = (NB * L + T - 1) / T;
+            longlong2 v[PER][R];
+#pragma unroll
+            for (int p = 0; p < PER; ++p) {
+                int j, line;
+                if (item(p, NB, j, line, tid)) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) v[p][r] = buf[(j + r * NB) * PS + line];
+                }
+            }
+            sync();
+#pragma unroll
+            for (int p = 0; p < PER; ++p) {
+                int j, line;
+                if (item(p, NB, j, line, tid)) {
+                    Fx::template butterfly<S>(v[p], j, tw);
+                    const int k = j & (Ns - 1), base = (j - k) * R + k;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) buf[(base + r * Ns) * PS + line] = v[p][r];
+                }
+            }
+            sync();
+            mids<S + 1>(buf, tw, tid, sync);
+        }
+    }
+    // Block exponent of a transform from this thread's largest high word; every
+    // thread of the group calls it.
+    struct Scale {
+        int E, X;
+    };
+    __device__ static __forceinline__ Scale scale_of(unsigned mx, int lg) {
+        mx = fx_cta_max<T>(mx);
+        const int E = fx_exponent(mx);
+        return Scale{E, Fx::out_exp(mx, E, lg)};
+    }
+    __device__ static __forceinline__ void first_item(int p, double2 (&x)[RF], double2* dbuf, int tid, const Scale& sc) {
+        longlong2* buf = reinterpret_cast<longlong2*>(dbuf);
+        int j, line;
+        if (item(p, NBF, j, line, tid)) {
+            longlong2 v[RF];
+#pragma unroll
+            for (int r = 0; r < RF; ++r) v[r] = fx_from(x[r], Fx::S0, sc.E);
+            dft_r<RF, INV>(v);
+#pragma unroll
+            for (int r = 0; r < RF; ++r) buf[(j * RF + r) * PS + line] = v[r];
+        }
+    }
+    template <class Sync>
+    __device__ static __forceinline__ void middle(double2* buf, const int4* __restrict__ tw, const int4*, int tid,
+                                                  const Sync& sync) {
+        sync();
+        mids<1>(reinterpret_cast<longlong2*>(buf), tw, tid, sync);
+    }
+    __device__ static __forceinline__ bool last_item(int p, double2 (&x)[RL], const double2* dbuf,
+                                                     const int4* __restrict__ tw, const int4*, int tid, int& j,
+                                                     const Scale& sc) {
+        const longlong2* buf = reinterpret_cast<const longlong2*>(dbuf);
+        int line;
+        if (!item(p, NBL, j, line, tid)) return false;
+        longlong2 v[RL];
+#pragma unroll
+        for (int r = 0; r < RL; ++r) v[r] = buf[(j + r * NBL) * PS + line];
+        Fx::template butterfly<NPASS - 1>(v, j, tw);
+#pragma unroll
+        for (int r = 0; r < RL; ++r) x[r] = fx_to(v[r], sc.X);
+        return true;
+    }
+    template <class Sync>
+    __device__ static __forceinline__ void finish(const Sync& sync) { sync(); }
+
+    template <class Sync>
+    __device__ static __forceinline__ void run(double2 (&in)[PF][RF], double2 (&out)[PL][RL], double2* buf,
+                                               const int4* __restrict__ tw, const int4* twl, int tid,
+                                               const Sync& sync, int lg = 0) {
+        unsigned mx = 0;
+#pragma unroll
+        for (int p = 0; p < PF; ++p) {
+            int j, line;
+            if (item(p, NBF, j, line, tid)) {
+#pragma unroll
+                for (int r = 0; r < RF; ++r) mx = max(mx, fx_hi(in[p][r]));
+            }
+        }
+        const Scale sc = scale_of(mx, lg);
+        if constexpr (NPASS == 1) {
+#pragma unroll
+            for (int p = 0; p < PF; ++p) {
+                longlong2 v[RF];
+#pragma unroll
+                for (int r = 0; r < RF; ++r) v[r] = fx_from(in[p][r], Fx::S0, sc.E);
+                dft_r<RF, INV>(v);
+#pragma unroll
+                for (int r = 0; r < RF; ++r) out[p][r] = fx_to(v[r], sc.X);
+            }
+        } else {
+#pragma unroll
+            for (int p = 0; p < PF; ++p) first_item(p, in[p], buf, tid, sc);
+            middle(buf, tw, twl, tid, sync);
+#pragma unroll
+            for (int p = 0; p < PL; ++p) {
+                int j;
+                last_item(p, out[p], buf, tw, twl, tid, j, sc);
+            }
+            sync();
+        }
     }
 };
 

@@ -153,6 +153,7 @@ inline size_t vrow(const tdse_ctx* c, int tf) {
 // once the common fields of the context are set.
 tdse_status fs_create(tdse_ctx* c);
 tdse_status fs_bind(tdse_ctx* c, cudaStream_t s);
+tdse_status fs_upload_twiddles(tdse_ctx* c, cudaStream_t s);
 tdse_status fs_build_phase_tables(tdse_ctx* c, int b, cudaStream_t s);
 tdse_status fs_set_initial(tdse_ctx* c, int b, const double* u0, cudaMemcpyKind kind, cudaStream_t s);
 tdse_status fs_steps(tdse_ctx* c, int nsteps, cudaStream_t s);

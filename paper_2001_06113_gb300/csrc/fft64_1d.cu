@@ -21,7 +21,7 @@ enum F4Dst : int { F4_DST_STATE = 0, F4_DST_RING = 1, F4_DST_OUT = 2 };
 
 // Pass A: Y[b][k1 N2 + n2] = w^{n2 k1} sum_n1 x[n1 N2 + n2] w_N1^{n1 k1}
 template <bool INV>
-__global__ void __launch_bounds__(F4_T) k_f4_cols(const KArgs a, const double2* tw128, double2* Y, int src) {
+__global__ void __launch_bounds__(F4_T) k_f4_cols(const KArgs a, const int4* tw128, double2* Y, int src) {
     __shared__ double2 buf[F4_N1 * F4_L];
     const int cg = blockIdx.x, b = blockIdx.y;
     const size_t off = (size_t)b * F4_N;
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(F4_T) k_f4_cols(const KArgs a, const double2* 
     for (int it = threadIdx.x; it < F4_N1 * F4_L; it += F4_T) {
         const int k1 = it / F4_L, c = it % F4_L;
         const int n2 = cg * F4_L + c;
-        double2 w = __ldg(&a.tw64_0[(n2 * k1) % F4_N]);
+        double2 w = fx_factor_to_d(__ldg(&a.tw64_0[(n2 * k1) % F4_N]));
         if (INV) w.y = -w.y;
         Y[off + (size_t)k1 * F4_N2 + n2] = cmul(buf[k1 * F4_L + c], w);
     }
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(F4_T) k_f4_cols(const KArgs a, const double2* 
 // Pass B: X[k1 + N1 k2] = sum_n2 Y[k1 N2 + n2] w_N2^{n2 k2}, written to the
 // state (scaled 1/N), a ring slot (scaled 1/N) or the read-out array.
 template <bool INV>
-__global__ void __launch_bounds__(F4_T) k_f4_rows(const KArgs a, const double2* tw128, const double2* Y, int dst) {
+__global__ void __launch_bounds__(F4_T) k_f4_rows(const KArgs a, const int4* tw128, const double2* Y, int dst) {
     __shared__ double2 buf[F4_N2 * F4_L];
     const int rg = blockIdx.x, b = blockIdx.y;
     const size_t off = (size_t)b * F4_N;
@@ -80,25 +80,25 @@ __global__ void __launch_bounds__(F4_T) k_f4_rows(const KArgs a, const double2* 
     }
 }
 
-__global__ void k_tw128(double2* tw) {
+__global__ void k_tw128(int4* tw) {
     const int m = threadIdx.x;
     double s, c;
     sincospi(-2.0 * m / F4_N1, &s, &c);
-    tw[m] = make_double2(c, s);
+    tw[m] = fx_factor(c, s);
 }
 
 }  // namespace
 
 int four_step_n() { return F4_N; }
 
-cudaError_t launch_four_step_tables(double2* tw128, cudaStream_t s) {
+cudaError_t launch_four_step_tables(int4* tw128, cudaStream_t s) {
     k_tw128<<<1, F4_N1, 0, s>>>(tw128);
     return cudaGetLastError();
 }
 
 // Start of a mixed 1D instance set of length 128^2 (MODE_INIT): ring[out_slot]
 // = DFT(V(t_tf) u0) / N and state = DFT(u0) / N, u0 parked in the state slots.
-cudaError_t launch_four_step_init(const KArgs& a, const double2* tw128, cudaStream_t s) {
+cudaError_t launch_four_step_init(const KArgs& a, const int4* tw128, cudaStream_t s) {
     const dim3 grid(F4_N2 / F4_L, a.B);
     k_f4_cols<false><<<grid, F4_T, 0, s>>>(a, tw128, a.aux, F4_SRC_VU0);
     k_f4_cols<false><<<grid, F4_T, 0, s>>>(a, tw128, a.aux2, F4_SRC_U0);
@@ -108,7 +108,7 @@ cudaError_t launch_four_step_init(const KArgs& a, const double2* tw128, cudaStre
 }
 
 // Read-out (MODE_READ): aux2 = IDFT(E_n v^) (or IDFT(u^) in the lab frame), FP64.
-cudaError_t launch_four_step_read(const KArgs& a, const double2* tw128, cudaStream_t s) {
+cudaError_t launch_four_step_read(const KArgs& a, const int4* tw128, cudaStream_t s) {
     const dim3 grid(F4_N2 / F4_L, a.B);
     k_f4_cols<true><<<grid, F4_T, 0, s>>>(a, tw128, a.aux, F4_SRC_STATE);
     k_f4_rows<true><<<grid, F4_T, 0, s>>>(a, tw128, a.aux, F4_DST_OUT);

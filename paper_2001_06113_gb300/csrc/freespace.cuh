@@ -106,7 +106,7 @@ template <> struct Tab<double2> {
     static __device__ __forceinline__ const double2* postF(const FsAxis& a) { return a.postF; }
     static __device__ __forceinline__ const double2* Gd(const FsAxis& a) { return a.Gd; }
     static __device__ __forceinline__ const double2* Fd(const FsAxis& a) { return a.Fd; }
-    static __device__ __forceinline__ const double2* tw(const FsAxis& a) { return a.tw; }
+    static __device__ __forceinline__ const int4* tw(const FsAxis& a) { return a.tw; }
     static __device__ __forceinline__ const double2* P(const FsAxis& a) { return a.P; }
     static __device__ __forceinline__ const double2* Lf(const FsAxis& a) { return a.Lf; }
     static __device__ __forceinline__ const double2* Li(const FsAxis& a) { return a.Li; }

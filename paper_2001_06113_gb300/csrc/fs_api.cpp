@@ -10,6 +10,7 @@
 #include "alpert_rules.h"
 #include "ctx.h"
 #include "fsargs.h"
+#include "fx.cuh"
 #include "kargs.h"
 
 using namespace tdse;
@@ -301,7 +302,7 @@ FsArgs fs_base(const tdse_ctx* c) {
         X.postF = c->P<double2>(F.off.postF[x]);
         X.Gd = c->P<double2>(F.off.Gd[x]);
         X.Fd = c->P<double2>(F.off.Fd[x]);
-        X.tw = c->P<double2>(F.off.tw[x]);
+        X.tw = c->P<int4>(F.off.tw[x]);
         X.P = c->P<double2>(F.off.P[x]);
         X.p = A.p;
         X.NC = A.NC;
@@ -666,7 +667,6 @@ tdse_status fs_bind(tdse_ctx* c, cudaStream_t s) {
         TDSE_CK(c, up(F.off.postF[x], T.postF));
         TDSE_CK(c, up(F.off.Gd[x], T.Gd));
         TDSE_CK(c, up(F.off.Fd[x], T.Fd));
-        TDSE_CK(c, up(F.off.tw[x], T.tw));
         if (F.ax[x].NT > 0) {
             TDSE_CK(c, up(F.off.Lf[x], T.Lf));
             TDSE_CK(c, up(F.off.Li[x], T.Li));
@@ -696,6 +696,23 @@ tdse_status fs_bind(tdse_ctx* c, cudaStream_t s) {
             }
         }
         TDSE_CK(c, cudaStreamSynchronize(s));    // T goes out of scope
+    }
+    return fs_upload_twiddles(c, s);
+}
+
+// The fixed-point twiddles of every axis (functions of the grid alone).
+tdse_status fs_upload_twiddles(tdse_ctx* c, cudaStream_t s) {
+    const FsState& F = c->F;
+    for (int x = 0; x < c->d; ++x) {
+        const int M = F.ax[x].M;
+        std::vector<int4> w(M);
+        for (int m = 0; m < M; ++m) {
+            const long double th = -2.0L * kPiL * m / M;
+            fx_limbs(llroundl(cosl(th) * 0x1p61L), w[m].x, w[m].y);
+            fx_limbs(llroundl(sinl(th) * 0x1p61L), w[m].z, w[m].w);
+        }
+        TDSE_CK(c, cudaMemcpyAsync(c->P<int4>(F.off.tw[x]), w.data(), w.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+        TDSE_CK(c, cudaStreamSynchronize(s));    // w goes out of scope
     }
     return TDSE_OK;
 }

@@ -42,7 +42,7 @@ struct FsAxis {
     const double2* postF;  // [2][NE]    forward: e^{+i i h}
     const double2* Gd;     // [ND][M]    inverse dense: (w_d / 2pi) e^{i zeta_d x_j}
     const double2* Fd;     // [ND][M]    forward dense: (2/M) e^{-i zeta_d x_j}
-    const double2* tw;     // [M]        e^{-2 pi i m / M}
+    const int4* tw;        // [M]        e^{-2 pi i m / M}, fixed-point factors (fx.cuh)
     const double2* P;      // [B][n_int][N] one-step phases e^{-i zeta^2 s + i zeta (phi(t1) - phi(t0))}
     // FP32 copies for the FP32-transform variant (TDSE_MIXED), same layouts
     const float2* preI_f;

@@ -91,14 +91,15 @@ struct KArgs {
     const float2* k1d_lo;     // [E1D_NLO][N]               (1D: e^{-i k^2 n dt}, n < 32)
     const float2* k1d_hi;     // [nhi][N]                   (1D: e^{-i k^2 32 q dt})
     const float2* a1d;        // [B][nsteps + 1][nh + nl]   (1D: e^{i k phi(t_n)})
-    // twiddles e^{-2 pi i m / n} for each axis length
-    const double2* tw64_0;
-    const double2* tw64_1;
+    // twiddles e^{-2 pi i m / n} for each axis length: fixed-point table factors
+    // (fx.cuh) for the FP64 transforms, FP32 for the others
+    const int4* tw64_0;
+    const int4* tw64_1;
     const float2* tw32_0;
     const float2* tw32_1;
     const float2* tw32lo_0;   // e^{-2 pi i m / n} - tw32 (rounding residual)
     const float2* tw32lo_1;
-    const double2* tw64_2;    // axis 2 (3D)
+    const int4* tw64_2;       // axis 2 (3D)
     const float2* tw32_2;
     const float2* tw32lo_2;
 };
@@ -190,12 +191,15 @@ int step2d_cluster_smem();
 // limit: FP64 init / read-out of such sizes go through launch_fft64_four_step).
 constexpr int P1D_MAX_F32 = 16384;
 int four_step_n();                                   // 128 * 128
-cudaError_t launch_four_step_tables(double2* tw128, cudaStream_t s);
-cudaError_t launch_four_step_init(const KArgs& a, const double2* tw128, cudaStream_t s);
-cudaError_t launch_four_step_read(const KArgs& a, const double2* tw128, cudaStream_t s);
+cudaError_t launch_four_step_tables(int4* tw128, cudaStream_t s);
+cudaError_t launch_four_step_init(const KArgs& a, const int4* tw128, cudaStream_t s);
+cudaError_t launch_four_step_read(const KArgs& a, const int4* tw128, cudaStream_t s);
 
 // Table builders (tables.cu).
-cudaError_t launch_twiddles(double2* tw64, float2* tw32, float2* tw32lo, int n, cudaStream_t s);
+// e^{-2 pi i m / n}, m < n: as fixed-point factors tw64 (FP64 transforms) and
+// in FP32 with its rounding residual; launch_roots: in FP64 (and FP32).
+cudaError_t launch_twiddles(int4* tw64, float2* tw32, float2* tw32lo, int n, cudaStream_t s);
+cudaError_t launch_roots(double2* w64, float2* w32, int n, cudaStream_t s);
 cudaError_t launch_kin1d(double2* kin64, float4* kinff, int n, int L, double dt, cudaStream_t s);
 cudaError_t launch_adv1d(double2* adv64, float4* advff, const int2* intervals, int n_int, const double* phi,
                          int ntf, int n, int nh, int nl, cudaStream_t s);

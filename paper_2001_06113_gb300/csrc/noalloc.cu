@@ -111,8 +111,8 @@ extern "C" tdse_status tdse_modes_to_grid_2d_noalloc(const double* uhat, double*
     if (scratch_address(&base) != cudaSuccess) return TDSE_ECUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char* b = static_cast<char*>(base);
-    double2* tw64_0 = reinterpret_cast<double2*>(b + NOALLOC_TW_OFF);
-    double2* tw64_1 = tw64_0 + 1024;
+    int4* tw64_0 = reinterpret_cast<int4*>(b + NOALLOC_TW_OFF);
+    int4* tw64_1 = tw64_0 + 1024;
     float2* tw32_0 = reinterpret_cast<float2*>(tw64_1 + 1024);
     float2* tw32_1 = tw32_0 + 1024;
     float2* tw32lo_0 = tw32_1 + 1024;

@@ -89,6 +89,16 @@ __device__ __forceinline__ void batched_copy(Load load, Store store) {
     }
 }
 
+// v / n for the n-point forward transforms: FP64 transforms apply it as an
+// exact power of two on their way out (lg of CtaFft::run).
+__device__ __forceinline__ float2 norm_of(float2 v, float scale) { return cscale(v, scale); }
+__device__ __forceinline__ double2 norm_of(double2 v, double) { return v; }
+template <class F, class C>
+__device__ __forceinline__ void run_fwd(C* buf, const tw_t<C>* tw, const tw_t<C>* twl, int lg) {
+    if constexpr (std::is_same<C, double2>::value) F::run(buf, tw, twl, -lg);
+    else F::run(buf, tw, twl);
+}
+
 // Hint the L2 to fetch `bytes` from p (one request per 128-byte line).
 __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
     const char* c = static_cast<const char*>(p);
@@ -168,8 +178,8 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_begin(const KAr
     const size_t NP = (size_t)N0 * n1;
     ST* st = reinterpret_cast<ST*>(a.uhat) + (size_t)b * NP;
     const RT* ringb = reinterpret_cast<const RT*>(a.ring) + (size_t)b * a.ring_slots * NP;
-    const C* tw;
-    const C* twl;
+    const tw_t<C>* tw;
+    const tw_t<C>* twl;
     if constexpr (is_f64<C>::value) { tw = a.tw64_0; twl = tw; } else { tw = a.tw32_0; twl = a.tw32lo_0; }
     const bool step = (a.mode == MODE_STEP);
 
@@ -223,8 +233,8 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
     const int r0 = blockIdx.x * L;
     const int n0 = a.n0;
     const size_t NP = (size_t)n0 * N1;
-    const C* tw;
-    const C* twl;
+    const tw_t<C>* tw;
+    const tw_t<C>* twl;
     if constexpr (F64) { tw = a.tw64_1; twl = tw; } else { tw = a.tw32_1; twl = a.tw32lo_1; }
     const double vfac = a.tfac[(size_t)b * a.ntf + a.tf];
     const double* V0 = a.V0 + (size_t)b * a.vstride;
@@ -246,13 +256,13 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
                 buf[j1 * LS + lane] = pass == 0 ? cscale(u, (R)(vfac * V0[idx])) : u;
             }
             __syncthreads();
-            FW::run(buf, tw, twl);
+            run_fwd<FW>(buf, tw, twl, ilog2(N1));
             C* dst = pass == 0 ? T2 : T1;
             for (int item = threadIdx.x; item < N1 * L; item += T2D) {
                 const int lane = item / N1, k1 = item % N1;
                 C v = buf[k1 * LS + lane];
                 if (a.flat1d) v = tw1d<false>(a, r0 + lane, k1, v);
-                dst[(size_t)(r0 + lane) * N1 + k1] = cscale(v, scale);
+                dst[(size_t)(r0 + lane) * N1 + k1] = norm_of(v, scale);
             }
             __syncthreads();
         }
@@ -314,13 +324,13 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
         }
     }
     __syncthreads();
-    FW::run(buf, tw, twl);
+    run_fwd<FW>(buf, tw, twl, ilog2(N1));
     C* T2 = reinterpret_cast<C*>(a.aux2) + (size_t)b * NP;
     for (int item = threadIdx.x; item < N1 * L; item += T2D) {
         const int lane = item / N1, k1 = item % N1;
         C v = buf[k1 * LS + lane];
         if (a.flat1d) v = tw1d<false>(a, r0 + lane, k1, v);
-        T2[(size_t)(r0 + lane) * N1 + k1] = cscale(v, scale);
+        T2[(size_t)(r0 + lane) * N1 + k1] = norm_of(v, scale);
     }
 }
 
@@ -340,8 +350,8 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs
     const size_t NP = (size_t)N0 * n1;
     ST* st = reinterpret_cast<ST*>(a.uhat) + (size_t)b * NP;
     RT* ringb = reinterpret_cast<RT*>(a.ring) + (size_t)b * a.ring_slots * NP;
-    const C* tw;
-    const C* twl;
+    const tw_t<C>* tw;
+    const tw_t<C>* twl;
     if constexpr (is_f64<C>::value) { tw = a.tw64_0; twl = tw; } else { tw = a.tw32_0; twl = a.tw32lo_0; }
     const R scale = (R)1 / (R)N0;
 
@@ -349,20 +359,20 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs
         batched_copy<C, N0 * L>([&](int item) { return src[(size_t)(item / L) * n1 + c0 + item % L]; },
                                 [&](int item, C v) { buf[item] = v; });
         __syncthreads();
-        FW::run(buf, tw, twl);
+        run_fwd<FW>(buf, tw, twl, ilog2(N0));
     };
     load_tile(reinterpret_cast<const C*>(a.aux2) + (size_t)b * NP);
 
     if (a.mode == MODE_INIT) {
         for (int item = threadIdx.x; item < N0 * L; item += T2D) {
             const int lane = item % L, m0 = item / L;
-            ringb[(size_t)a.out_slot * NP + (size_t)m0 * n1 + c0 + lane] = cvt<RT>(cscale(buf[m0 * L + lane], scale));
+            ringb[(size_t)a.out_slot * NP + (size_t)m0 * n1 + c0 + lane] = cvt<RT>(norm_of(buf[m0 * L + lane], scale));
         }
         __syncthreads();
         load_tile(reinterpret_cast<const C*>(a.aux) + (size_t)b * NP);
         for (int item = threadIdx.x; item < N0 * L; item += T2D) {
             const int lane = item % L, m0 = item / L;
-            st[(size_t)m0 * n1 + c0 + lane] = d_to_st<ST>(cvt<double2>(cscale(buf[m0 * L + lane], scale)));
+            st[(size_t)m0 * n1 + c0 + lane] = d_to_st<ST>(cvt<double2>(norm_of(buf[m0 * L + lane], scale)));
         }
         return;
     }
@@ -373,7 +383,7 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs
         const int lane = item % L, m0 = item / L;
         const int m1 = c0 + lane;
         const size_t idx = (size_t)m0 * n1 + m1;
-        end_elem<C, RT>(a, step, b, st, ringb, NP, idx, m0, m1, cscale(buf[m0 * L + lane], scale), a.e_step);
+        end_elem<C, RT>(a, step, b, st, ringb, NP, idx, m0, m1, norm_of(buf[m0 * L + lane], scale), a.e_step);
         if constexpr (FUSED) buf[m0 * L + lane] = begin_elem<C, RT>(a, true, b, st, ringb, NP, idx, m0, m1, a.e_next);
     }
     if constexpr (FUSED) {
@@ -686,13 +696,13 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_axis1(const KArgs a
     batched_copy<C, N1 * L>([&](int item) { return base[(size_t)(item / L) * n2 + item % L]; },
                             [&](int item, C v) { buf[item] = v; });
     __syncthreads();
-    const C* tw;
-    const C* twl;
+    const tw_t<C>* tw;
+    const tw_t<C>* twl;
     if constexpr (is_f64<C>::value) { tw = a.tw64_1; twl = tw; } else { tw = a.tw32_1; twl = a.tw32lo_1; }
-    F::run(buf, tw, twl);
+    run_fwd<F>(buf, tw, twl, INV ? 0 : ilog2(N1));
     const R scale = (R)1 / (R)N1;
     for (int item = threadIdx.x; item < N1 * L; item += T2D)
-        base[(size_t)(item / L) * n2 + item % L] = INV ? buf[item] : cscale(buf[item], scale);
+        base[(size_t)(item / L) * n2 + item % L] = INV ? buf[item] : norm_of(buf[item], scale);
 }
 
 template <class C, int N1>

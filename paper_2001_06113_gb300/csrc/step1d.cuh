@@ -32,13 +32,21 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
     const size_t NP = N;
     ST* st = reinterpret_cast<ST*>(a.uhat) + (size_t)b * NP;
     RT* ringb = reinterpret_cast<RT*>(a.ring) + (size_t)b * a.ring_slots * NP;
-    const C* tw;
-    const C* twl;
+    const tw_t<C>* tw;
+    const tw_t<C>* twl;
     if constexpr (F64) { tw = a.tw64_0; twl = tw; } else { tw = a.tw32_0; twl = a.tw32lo_0; }
     const double vfac = a.tfac[(size_t)b * a.ntf + a.tf];
     const double* V0 = a.V0 + (size_t)b * a.vstride;
     const float2* V0f = a.V0f + (size_t)b * a.vstride;
-    const R scale = (R)1 / (R)N;
+    const R scale = (R)1 / (R)N;             // forward transforms: 1/N (FP64: an exact power of two inside them)
+    auto norm = [&](C v) -> C {
+        if constexpr (F64) return v;
+        else return cscale(v, scale);
+    };
+    auto run_fw = [&](auto& in, auto& out) {
+        if constexpr (F64) FW::run(in, out, buf, tw, twl, tid, sync, -ilog2(N));
+        else FW::run(in, out, buf, tw, twl, tid, sync);
+    };
     const float fh = (float)vfac, fl = (float)(vfac - (double)fh);
 
     // V(x_j, t) as hi + lo in the compute precision
@@ -72,7 +80,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
                     }
                 }
             }
-            FW::run(in, out, buf, tw, twl, tid, sync);
+            run_fw(in, out);
 #pragma unroll
             for (int p = 0; p < FW::PL; ++p) {
                 int j, line;
@@ -80,7 +88,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
 #pragma unroll
                     for (int r = 0; r < FW::RL; ++r) {
                         const int k = j + r * FW::NBL;
-                        const C v = cscale(out[p][r], scale);
+                        const C v = norm(out[p][r]);
                         if (pass == 0) ringb[(size_t)a.out_slot * NP + k] = cvt<RT>(v);
                     }
                 }
@@ -94,7 +102,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
             if (FW::item(p, FW::NBL, j, line, tid)) {
 #pragma unroll
                 for (int r = 0; r < FW::RL; ++r)
-                    st[j + r * FW::NBL] = d_to_st<ST>(cvt<double2>(cscale(out[p][r], scale)));
+                    st[j + r * FW::NBL] = d_to_st<ST>(cvt<double2>(norm(out[p][r])));
             }
         }
         return;
@@ -151,7 +159,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
     };
     // End of the step at mode k from the forward-transform output o and W.
     auto output_of = [&](int k, C o, const ST& W) {
-        RT rv = cvt<RT>(cscale(o, scale));
+        RT rv = cvt<RT>(norm(o));
         if constexpr (FF) {
             if (step && a.ip) {
                 rv = cmul(make_float2(a.zr[0], a.zr[1]), cmul(conjf2(e_1d(a, b, a.e_step, k)), rv));
@@ -187,6 +195,66 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
     // kernel's code within the instruction cache.
     constexpr bool ROLLED = !KEEP && PB > 1 && FI::NPASS > 1 && FW::NPASS > 1;
     if constexpr (ROLLED) {
+        // FP64: the transform's block exponent needs every input first, so the
+        // inputs (which are the parked W) are formed in a loop of their own.
+        if constexpr (F64) {
+            unsigned mx = 0;
+#pragma unroll 1
+            for (int p = 0; p < PB; ++p) {
+                int j, line;
+                if (FI::item(p, FI::NBF, j, line, tid)) {
+#pragma unroll
+                    for (int r = 0; r < RB; ++r) {
+                        const int k = j + r * FI::NBF;
+                        ST W;
+                        mx = max(mx, fx_hi(cvt<double2>(input_of(k, W))));
+                        if (step) st[k] = W;
+                    }
+                }
+            }
+            const auto sc = FI::scale_of(mx, 0);
+#pragma unroll 1
+            for (int p = 0; p < PB; ++p) {
+                int j, line;
+                C x[RB];
+                if (FI::item(p, FI::NBF, j, line, tid)) {
+#pragma unroll
+                    for (int r = 0; r < RB; ++r) x[r] = st_to_c<C>(st[j + r * FI::NBF]);
+                }
+                FI::first_item(p, x, buf, tid, sc);
+            }
+            FI::middle(buf, tw, twl, tid, sync);
+            C mid[FI::PL][FI::RL];
+#pragma unroll
+            for (int p = 0; p < FI::PL; ++p) {
+                int j;
+                FI::last_item(p, mid[p], buf, tw, twl, tid, j, sc);
+            }
+            FI::finish(sync);
+            solve(mid);
+            mx = 0;
+#pragma unroll
+            for (int p = 0; p < FI::PL; ++p)
+#pragma unroll
+                for (int r = 0; r < FI::RL; ++r) mx = max(mx, fx_hi(mid[p][r]));
+            const auto sw = FW::scale_of(mx, -ilog2(N));
+#pragma unroll
+            for (int p = 0; p < FW::PF; ++p) FW::first_item(p, mid[p], buf, tid, sw);
+            FW::middle(buf, tw, twl, tid, sync);
+#pragma unroll 1
+            for (int p = 0; p < FW::PL; ++p) {
+                C o[FW::RL];
+                int j;
+                if (FW::last_item(p, o, buf, tw, twl, tid, j, sw)) {
+#pragma unroll
+                    for (int r = 0; r < FW::RL; ++r) {
+                        const int k = j + r * FW::NBL;
+                        output_of(k, o[r], st[k]);
+                    }
+                }
+            }
+            FW::finish(sync);
+        } else {
 #pragma unroll 1
         for (int p = 0; p < PB; ++p) {
             int j, line;
@@ -227,6 +295,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
             }
         }
         FW::finish(sync);
+        }
         return;
     } else {
         ST Wk[KEEP ? PB : 1][KEEP ? RB : 1];
@@ -248,7 +317,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
         }
         FI::run(in, mid, buf, tw, twl, tid, sync);
         solve(mid);
-        FW::run(mid, out, buf, tw, twl, tid, sync);
+        run_fw(mid, out);
 #pragma unroll
         for (int p = 0; p < FW::PL; ++p) {
             int j, line;

@@ -30,15 +30,24 @@ __device__ __forceinline__ double dither_angle(int n) {
 
 __device__ __forceinline__ float4 ff_from_cs(double c, double s) { return d_to_ffc(make_double2(c, s)); }
 
-__global__ void k_twiddles(double2* tw64, float2* tw32, float2* tw32lo, int n) {
+__global__ void k_twiddles(int4* tw64, float2* tw32, float2* tw32lo, int n) {
     int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= n) return;
     double s, c;
     sincospi(-2.0 * (double)m / (double)n, &s, &c);
-    tw64[m] = make_double2(c, s);
+    tw64[m] = fx_factor(c, s);
     const float ch = (float)c, sh = (float)s;
     tw32[m] = make_float2(ch, sh);
     tw32lo[m] = make_float2((float)(c - (double)ch), (float)(s - (double)sh));
+}
+
+__global__ void k_roots(double2* w64, float2* w32, int n) {
+    int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= n) return;
+    double s, c;
+    sincospi(-2.0 * (double)m / (double)n, &s, &c);
+    w64[m] = make_double2(c, s);
+    w32[m] = make_float2((float)c, (float)s);
 }
 
 __global__ void k_kin1d(double2* kin64, float4* kinff, int n, int L, double dt) {
@@ -259,7 +268,11 @@ cudaError_t launch_transpose_1d(void* dst, const void* src, int n0, int n1, int 
     return cudaGetLastError();
 }
 
-cudaError_t launch_twiddles(double2* tw64, float2* tw32, float2* tw32lo, int n, cudaStream_t s) {
+cudaError_t launch_roots(double2* w64, float2* w32, int n, cudaStream_t s) {
+    k_roots<<<(n + 255) / 256, 256, 0, s>>>(w64, w32, n);
+    return cudaGetLastError();
+}
+cudaError_t launch_twiddles(int4* tw64, float2* tw32, float2* tw32lo, int n, cudaStream_t s) {
     k_twiddles<<<(n + 255) / 256, 256, 0, s>>>(tw64, tw32, tw32lo, n);
     return cudaGetLastError();
 }
