@@ -387,21 +387,6 @@ tdse_status grid_part(tdse_ctx* c, const FsArgs& a, int f32, cudaStream_t s) {
     return TDSE_OK;
 }
 
-// One step with the description in a: 1D fused kernel; 2D / 3D row begin,
-// grid part, row end.
-tdse_status one_step(tdse_ctx* c, const FsArgs& a, cudaStream_t s) {
-    const int f32 = c->F.f32 ? 1 : 0;
-    if (c->d == 1) {
-        TDSE_CK(c, launch_fs_1d(a, FS_1D_STEP, f32, s));
-    } else {
-        TDSE_CK(c, launch_fs_row(a, FS_ROW_BEGIN, f32, s));
-        tdse_status st = grid_part(c, a, f32, s);
-        if (st != TDSE_OK) return st;
-        TDSE_CK(c, launch_fs_row(a, FS_ROW_END, f32, s));
-    }
-    return TDSE_OK;
-}
-
 tdse_status fs_init(tdse_ctx* c, cudaStream_t s) {
     const FsState& F = c->F;
     double2* u = c->P<double2>(F.off.u);
@@ -410,6 +395,28 @@ tdse_status fs_init(tdse_ctx* c, cudaStream_t s) {
     st = forward_to(c, u, 1, 0, ring_at(c, F.off.ring, (size_t)slot_of(c, 0) * F.NM), (size_t)c->RS * F.NM, 1, s);
     if (st != TDSE_OK) return st;
     c->inited = true;
+    return TDSE_OK;
+}
+
+// Steps first..last of a chain, step i described by args(i).  2D / 3D: row
+// begin, (grid part, row end + begin) x (last - first), grid part, row end;
+// the end of step i runs with the arguments of i + 1 and the ring slot of i.
+template <class Args>
+tdse_status fs_chain(tdse_ctx* c, Args args, int first, int last, cudaStream_t s) {
+    const int f32 = c->F.f32 ? 1 : 0;
+    if (c->d == 1) {
+        for (int i = first; i <= last; ++i) TDSE_CK(c, launch_fs_1d(args(i), FS_1D_STEP, f32, s));
+        return TDSE_OK;
+    }
+    TDSE_CK(c, launch_fs_row(args(first), FS_ROW_BEGIN, f32, s));
+    for (int i = first; i <= last; ++i) {
+        const FsArgs a = args(i);
+        tdse_status st = grid_part(c, a, f32, s);
+        if (st != TDSE_OK) return st;
+        FsArgs f = i < last ? args(i + 1) : a;
+        f.out_slot = a.out_slot;
+        TDSE_CK(c, launch_fs_row(f, i < last ? FS_ROW_END | FS_ROW_BEGIN : FS_ROW_END, f32, s));
+    }
     return TDSE_OK;
 }
 
@@ -424,8 +431,8 @@ tdse_status fs_startup_step(tdse_ctx* c, int n, cudaStream_t s) {
         double2* cr = ring_at(c, F.off.chain_ring, ch * BM);
         TDSE_CK(c, cudaMemcpyAsync(cu + ch * BM, c->P<double2>(F.off.uhat), BM * 16, cudaMemcpyDeviceToDevice, s));
         TDSE_CK(c, launch_copy_slot(cr, c->P<void>(F.off.ring), c->RS, slot_of(c, n - 1), c->B, F.NM, c->rsz, s));
-        const int len = SUB >> ch;
-        for (int i = 0; i < (1 << ch); ++i) {
+        const int len = SUB >> ch, last = (1 << ch) - 1;
+        auto sub = [&](int i) {     // trapezoid sub-step i of the chain
             FsArgs a = fs_base(c);
             a.uhat = cu + ch * BM;
             a.ring = cr;
@@ -439,9 +446,10 @@ tdse_status fs_startup_step(tdse_ctx* c, int n, cudaStream_t s) {
             a.out_slot = 0;
             a.interval[0] = startup_interval(c, n, ch, i);
             set_time(c, a, SUB * (n - 1) + (i + 1) * len);
-            tdse_status st = one_step(c, a, s);
-            if (st != TDSE_OK) return st;
-        }
+            return a;
+        };
+        tdse_status st = fs_chain(c, sub, 0, last, s);
+        if (st != TDSE_OK) return st;
     }
     TDSE_CK(c, launch_combine(c->P<void>(F.off.uhat), cu, BM, c->L, c->rich, BM, false, s));
     TDSE_CK(c, launch_combine(c->P<void>(F.off.u), cx, BX, c->L, c->rich, BX, false, s));
@@ -461,27 +469,8 @@ FsArgs adams_args(const tdse_ctx* c, int n) {
     return a;
 }
 
-// Adams steps n0+1 .. n0+k.  2D / 3D: row begin, (grid part, row end+begin)
-// x (k-1), grid part, row end.
 tdse_status fs_adams(tdse_ctx* c, int n0, int k, cudaStream_t s) {
-    const int f32 = c->F.f32 ? 1 : 0;
-    if (c->d == 1) {
-        for (int n = n0 + 1; n <= n0 + k; ++n) TDSE_CK(c, launch_fs_1d(adams_args(c, n), FS_1D_STEP, f32, s));
-        return TDSE_OK;
-    }
-    TDSE_CK(c, launch_fs_row(adams_args(c, n0 + 1), FS_ROW_BEGIN, f32, s));
-    for (int n = n0 + 1; n < n0 + k; ++n) {
-        tdse_status st = grid_part(c, adams_args(c, n), f32, s);
-        if (st != TDSE_OK) return st;
-        FsArgs f = adams_args(c, n + 1);
-        f.out_slot = slot_of(c, n);
-        TDSE_CK(c, launch_fs_row(f, FS_ROW_END | FS_ROW_BEGIN, f32, s));
-    }
-    const FsArgs last = adams_args(c, n0 + k);
-    tdse_status st = grid_part(c, last, f32, s);
-    if (st != TDSE_OK) return st;
-    TDSE_CK(c, launch_fs_row(last, FS_ROW_END, f32, s));
-    return TDSE_OK;
+    return fs_chain(c, [&](int n) { return adams_args(c, n); }, n0 + 1, n0 + k, s);
 }
 
 // FP64 residual of the implicit step just completed (step c->step, FP32

@@ -102,6 +102,25 @@ FX_HD long long fx_times_rsqrt2(long long v) {
     return v - ((long long)hi * CH + (cr >> 32));
 }
 
+// v w 2^K / 2^64 for a real factor w = h 2^32 + l (units of 2^-61, as fx_mul).
+template <int K>
+FX_HD long long fx_mul_real(long long v, int2 w) {
+    const int vl = (int)v, vh = (int)(v >> 32) + (int)((unsigned)vl >> 31);
+    const long long hi = (long long)vh * w.x;
+    const long long cr = (long long)vl * w.x + ((long long)vh * w.y + (1ll << (31 - K)));
+    return (long long)((unsigned long long)hi << K) + (cr >> (32 - K));
+}
+
+// Table factors as 2^61 values, and such a value (a product of factors) as a
+// factor again; its low bit is set so that the low limb can be negated.
+FX_HD longlong2 fx_value(int4 w) {
+    return make_longlong2(((long long)w.x << 32) + w.y, ((long long)w.z << 32) + w.w);
+}
+FX_HD int4 fx_as_factor(longlong2 v) {
+    const int xl = (int)v.x | 1, yl = (int)v.y | 1;
+    return make_int4((int)(v.x >> 32) + (int)((unsigned)xl >> 31), xl, (int)(v.y >> 32) + (int)((unsigned)yl >> 31), yl);
+}
+
 // The two limbs of a table factor's component v (units of 2^-61).
 FX_HD void fx_limbs(long long v, int& h, int& l) {
     l = (int)v;

@@ -45,6 +45,9 @@ struct KArgs {
     int nhist;                // history terms j = 1..nhist
     double h;                 // step size
     double mu[MAX_HIST + 1];  // mu_0 .. mu_nhist
+    int2 mu_w[MAX_HIST + 1];  // mu_j / 2 and h 2^-h_e as fixed-point factors (fx.cuh; FP64 steps)
+    int2 h_w;
+    int h_e;
     float h_hi, h_lo;         // h split into two floats (double-float arithmetic)
     float hmu0_hi, hmu0_lo;   // h mu_0 split
     float mu_hi[MAX_HIST + 1], mu_lo[MAX_HIST + 1];
@@ -78,13 +81,13 @@ struct KArgs {
     double dt;
     const double* phi;        // [B][d][ntf], phi at t = m dt / 8
     // 1D relative phases p(k) = kin[c][m] * adv[hi] * adv[lo]
-    const double2* kin64;     // [L][N]
+    const int4* kin64;        // [L][N], fixed-point factors (fx.cuh), as adv64 and q64
     const float4* kinff;
-    const double2* adv64;     // [B][n_int][nh + nl]
+    const int4* adv64;        // [B][n_int][nh + nl]
     const float4* advff;
     int nh, nl, lb;
     // 2D relative phases p(k0,k1) = q[int][m0] * q[int][n0 + m1]
-    const double2* q64;       // [B][n_int][n0 + n1]
+    const int4* q64;          // [B][n_int][n0 + n1]
     const float4* qff;
     // interaction-picture phases E_n(k) = exp(-i |k|^2 t_n + i k.phi(t_n)) in FP32
     const float2* e2d;        // [B][nsteps + 1][n0 + n1]   (2D: separable)
@@ -200,11 +203,11 @@ cudaError_t launch_four_step_read(const KArgs& a, const int4* tw128, cudaStream_
 // in FP32 with its rounding residual; launch_roots: in FP64 (and FP32).
 cudaError_t launch_twiddles(int4* tw64, float2* tw32, float2* tw32lo, int n, cudaStream_t s);
 cudaError_t launch_roots(double2* w64, float2* w32, int n, cudaStream_t s);
-cudaError_t launch_kin1d(double2* kin64, float4* kinff, int n, int L, double dt, cudaStream_t s);
-cudaError_t launch_adv1d(double2* adv64, float4* advff, const int2* intervals, int n_int, const double* phi,
+cudaError_t launch_kin1d(int4* kin64, float4* kinff, int n, int L, double dt, cudaStream_t s);
+cudaError_t launch_adv1d(int4* adv64, float4* advff, const int2* intervals, int n_int, const double* phi,
                          int ntf, int n, int nh, int nl, cudaStream_t s);
 // 2D / 3D separable phase tables over the axes n0, n1 (and n2 > 0 for 3D): n0 + n1 + n2 entries per row
-cudaError_t launch_q2d(double2* q64, float4* qff, const int2* intervals, int n_int, const double* phi, int ntf,
+cudaError_t launch_q2d(int4* q64, float4* qff, const int2* intervals, int n_int, const double* phi, int ntf,
                        int n0, int n1, int n2, double dt, cudaStream_t s);
 cudaError_t launch_e2d(float2* e, const double* phi, int ntf, int nsteps, int n0, int n1, int n2, double dt,
                        cudaStream_t s);

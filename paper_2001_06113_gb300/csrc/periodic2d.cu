@@ -44,16 +44,23 @@ constexpr int T2D = 256;
 #ifndef TDSE_MINB2D_ROW
 #define TDSE_MINB2D_ROW TDSE_MINB2D
 #endif
-// FP64 kernels: two CTAs per SM (up to 128 registers) instead of four (64
-// registers and 0.6-1.9 KB of spills per thread): 0.494 -> 0.488 ms per
-// 4 x 512^2 FP64 step (the FP64 pipe bounds it either way).
-#ifndef TDSE_MINB2D64
-#define TDSE_MINB2D64 2
-#endif
-template <class C>
-constexpr int min_blocks_2d() { return std::is_same<C, float2>::value ? TDSE_MINB2D : TDSE_MINB2D64; }
-template <class C>
-constexpr int row_min_blocks() { return std::is_same<C, float2>::value ? TDSE_MINB2D_ROW : TDSE_MINB2D64; }
+// FP64 kernels: 4 lines per CTA (64-byte segments of double2 columns) and one
+// radix-8 butterfly per thread, three CTAs of 256 threads per SM.  8 lines and
+// two butterflies per thread left a 4-instance batch with 3.4 warps per
+// scheduler waiting on their own integer chains: 512^2 x 4, 100 steps, 42.5 ->
+// 32 ms (with the fused start-up passes).
+template <class C> constexpr int lanes_2d() { return std::is_same<C, float2>::value ? LANES2D : 4; }
+template <class C, int N> constexpr int threads_2d() {
+    if (std::is_same<C, float2>::value) return T2D;
+    return N / 2 < 64 ? 64 : N / 2;
+}
+template <class C, int N> constexpr int min_blocks_2d() {
+    if (std::is_same<C, float2>::value) return TDSE_MINB2D;
+    return 768 / threads_2d<C, N>() < 1 ? 1 : 768 / threads_2d<C, N>();
+}
+template <class C, int N> constexpr int row_min_blocks() {
+    return std::is_same<C, float2>::value ? TDSE_MINB2D_ROW : min_blocks_2d<C, N>();
+}
 
 // 16-byte asynchronous global -> shared copies (no registers held while in flight)
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
@@ -68,9 +75,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // 16 bytes) in flight before their stores: the loads are L2 hits of the other
 // pass's output, and issuing them one element at a time left the passes
 // waiting on L2 latency (0.181 -> 0.153 ms per 512^2 x16 mixed step).
-template <class C, int TOTAL, class Load, class Store>
+template <class C, int TOTAL, int T, class Load, class Store>
 __device__ __forceinline__ void batched_copy(Load load, Store store) {
-    constexpr int PER = (TOTAL + T2D - 1) / T2D;
+    constexpr int PER = (TOTAL + T - 1) / T;
     constexpr int LIM = sizeof(C) <= 8 ? 16 : 8;
     constexpr int G = PER < LIM ? PER : LIM;
 #pragma unroll 1
@@ -78,13 +85,13 @@ __device__ __forceinline__ void batched_copy(Load load, Store store) {
         C v[G];
 #pragma unroll
         for (int k = 0; k < G; ++k) {
-            const int item = threadIdx.x + (k0 + k) * T2D;
-            if (TOTAL % T2D == 0 || item < TOTAL) v[k] = load(item);
+            const int item = threadIdx.x + (k0 + k) * T;
+            if (TOTAL % T == 0 || item < TOTAL) v[k] = load(item);
         }
 #pragma unroll
         for (int k = 0; k < G; ++k) {
-            const int item = threadIdx.x + (k0 + k) * T2D;
-            if (TOTAL % T2D == 0 || item < TOTAL) store(item, v[k]);
+            const int item = threadIdx.x + (k0 + k) * T;
+            if (TOTAL % T == 0 || item < TOTAL) store(item, v[k]);
         }
     }
 }
@@ -166,9 +173,9 @@ __device__ __forceinline__ void end_elem(const KArgs& a, bool step, int b, state
 
 // ---------------------------------------------------------------- col_begin
 template <class C, class RT, int N0>
-__global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_begin(const KArgs a) {
-    constexpr int L = LANES2D;
-    using FI = CtaFft<C, N0, L, L, T2D, true>;
+__global__ void __launch_bounds__(threads_2d<C, N0>(), min_blocks_2d<C, N0>()) k_col_begin(const KArgs a) {
+    constexpr int L = lanes_2d<C>(), T = threads_2d<C, N0>();
+    using FI = CtaFft<C, N0, L, L, T, true>;
     using ST = state_t<RT>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
@@ -184,7 +191,7 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_begin(const KAr
     const bool step = (a.mode == MODE_STEP);
 
 #pragma unroll 1
-    for (int item = threadIdx.x; item < N0 * L; item += T2D) {
+    for (int item = threadIdx.x; item < N0 * L; item += T) {
         const int lane = item % L, m0 = item / L;
         const int m1 = c0 + lane;
         buf[m0 * L + lane] = begin_elem<C, RT>(a, step, b, st, ringb, NP, (size_t)m0 * n1 + m1, m0, m1, a.e_step);
@@ -192,7 +199,7 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_begin(const KAr
     __syncthreads();
     FI::run(buf, tw, twl);
     C* T1 = reinterpret_cast<C*>(a.aux) + (size_t)b * NP;
-    for (int item = threadIdx.x; item < N0 * L; item += T2D) {
+    for (int item = threadIdx.x; item < N0 * L; item += T) {
         const int lane = item % L, i0 = item / L;
         T1[(size_t)i0 * n1 + c0 + lane] = buf[i0 * L + lane];
     }
@@ -220,11 +227,11 @@ __device__ __forceinline__ float2 tw1d(const KArgs& a, int r, int c, float2 v) {
 #define TDSE_ROW_VG 8
 #endif
 template <class C, int N1>
-__global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArgs a) {
-    constexpr int L = LANES2D;
+__global__ void __launch_bounds__(threads_2d<C, N1>(), row_min_blocks<C, N1>()) k_row_mid(const KArgs a) {
+    constexpr int L = lanes_2d<C>(), T = threads_2d<C, N1>();
     constexpr int LS = L + 1;
-    using FI = CtaFft<C, N1, L, LS, T2D, true>;
-    using FW = CtaFft<C, N1, L, LS, T2D, false>;
+    using FI = CtaFft<C, N1, L, LS, T, true>;
+    using FW = CtaFft<C, N1, L, LS, T, false>;
     using R = typename cx_traits<C>::real;
     constexpr bool F64 = is_f64<C>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -249,7 +256,7 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
         C* T2 = reinterpret_cast<C*>(a.aux2) + (size_t)b * NP;
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
-            for (int item = threadIdx.x; item < N1 * L; item += T2D) {
+            for (int item = threadIdx.x; item < N1 * L; item += T) {
                 const int lane = item / N1, j1 = item % N1;
                 const size_t idx = (size_t)(r0 + lane) * N1 + j1;
                 const C u = cvt<C>(u0[idx]);
@@ -258,7 +265,7 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
             __syncthreads();
             run_fwd<FW>(buf, tw, twl, ilog2(N1));
             C* dst = pass == 0 ? T2 : T1;
-            for (int item = threadIdx.x; item < N1 * L; item += T2D) {
+            for (int item = threadIdx.x; item < N1 * L; item += T) {
                 const int lane = item / N1, k1 = item % N1;
                 C v = buf[k1 * LS + lane];
                 if (a.flat1d) v = tw1d<false>(a, r0 + lane, k1, v);
@@ -272,19 +279,19 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
     if (!F64 && a.mode == MODE_STEP) prefetch_l2(V0f + (size_t)r0 * N1, (size_t)L * N1 * sizeof(float2));
     const C* T1 = reinterpret_cast<const C*>(a.aux) + (size_t)b * NP;
     if (a.flat1d)
-        batched_copy<C, N1 * L>([&](int item) { return T1[(size_t)(r0 + item / N1) * N1 + item % N1]; },
+        batched_copy<C, N1 * L, T>([&](int item) { return T1[(size_t)(r0 + item / N1) * N1 + item % N1]; },
                                 [&](int item, C v) {
                                     buf[(item % N1) * LS + item / N1] = tw1d<true>(a, r0 + item / N1, item % N1, v);
                                 });
     else
-        batched_copy<C, N1 * L>([&](int item) { return T1[(size_t)(r0 + item / N1) * N1 + item % N1]; },
+        batched_copy<C, N1 * L, T>([&](int item) { return T1[(size_t)(r0 + item / N1) * N1 + item % N1]; },
                                 [&](int item, C v) { buf[(item % N1) * LS + item / N1] = v; });
     __syncthreads();
     FI::run(buf, tw, twl);
 
     if (a.mode == MODE_READ) {
         double2* out = a.aux2 + (size_t)b * NP;
-        for (int item = threadIdx.x; item < N1 * L; item += T2D) {
+        for (int item = threadIdx.x; item < N1 * L; item += T) {
             const int lane = item / N1, j1 = item % N1;
             out[(size_t)(r0 + lane) * N1 + j1] = cvt<double2>(buf[j1 * LS + lane]);
         }
@@ -293,28 +300,41 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
 
     const R hmu0 = (a.mode == MODE_STEP) ? (R)(a.h * a.mu[0]) : (R)0;
     if constexpr (F64) {
-        for (int item = threadIdx.x; item < N1 * L; item += T2D) {
-            const int lane = item / N1, j1 = item % N1;
-            const size_t idx = (size_t)(r0 + lane) * N1 + j1;
-            buf[j1 * LS + lane] = implicit_solve_times_V(buf[j1 * LS + lane], (R)(vfac * V0[idx]), (R)0, hmu0);
+        constexpr int PER = (N1 * L + T - 1) / T, G = PER < TDSE_ROW_VG ? PER : TDSE_ROW_VG;
+#pragma unroll 1
+        for (int k0 = 0; k0 < PER; k0 += G) {
+            double v[G];
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                const int item = threadIdx.x + (k0 + k) * T;
+                if ((N1 * L) % T == 0 || item < N1 * L) v[k] = V0[(size_t)(r0 + item / N1) * N1 + item % N1];
+            }
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                const int item = threadIdx.x + (k0 + k) * T;
+                if ((N1 * L) % T == 0 || item < N1 * L) {
+                    C& y = buf[(item % N1) * LS + item / N1];
+                    y = implicit_solve_times_V(y, vfac * v[k], hmu0);
+                }
+            }
         }
     } else {
         // V hi/lo of TDSE_ROW_VG points per thread in flight at a time (L2 hits after the prefetch)
-        constexpr int PER = (N1 * L + T2D - 1) / T2D;
+        constexpr int PER = (N1 * L + T - 1) / T;
         constexpr int G = PER < TDSE_ROW_VG ? PER : TDSE_ROW_VG;
 #pragma unroll 1
         for (int k0 = 0; k0 < PER; k0 += G) {
             float2 v2[G];
 #pragma unroll
             for (int k = 0; k < G; ++k) {
-                const int item = threadIdx.x + (k0 + k) * T2D;
-                if ((N1 * L) % T2D == 0 || item < N1 * L)
+                const int item = threadIdx.x + (k0 + k) * T;
+                if ((N1 * L) % T == 0 || item < N1 * L)
                     v2[k] = __ldg(&V0f[(size_t)(r0 + item / N1) * N1 + item % N1]);
             }
 #pragma unroll
             for (int k = 0; k < G; ++k) {
-                const int item = threadIdx.x + (k0 + k) * T2D;
-                if ((N1 * L) % T2D == 0 || item < N1 * L) {
+                const int item = threadIdx.x + (k0 + k) * T;
+                if ((N1 * L) % T == 0 || item < N1 * L) {
                     const int lane = item / N1, j1 = item % N1;
                     const float vh = fh * v2[k].x;
                     const float vl = fmaf(fh, v2[k].x, -vh) + fmaf(fh, v2[k].y, fl * v2[k].x);
@@ -326,7 +346,7 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
     __syncthreads();
     run_fwd<FW>(buf, tw, twl, ilog2(N1));
     C* T2 = reinterpret_cast<C*>(a.aux2) + (size_t)b * NP;
-    for (int item = threadIdx.x; item < N1 * L; item += T2D) {
+    for (int item = threadIdx.x; item < N1 * L; item += T) {
         const int lane = item / N1, k1 = item % N1;
         C v = buf[k1 * LS + lane];
         if (a.flat1d) v = tw1d<false>(a, r0 + lane, k1, v);
@@ -336,10 +356,10 @@ __global__ void __launch_bounds__(T2D, row_min_blocks<C>()) k_row_mid(const KArg
 
 // ------------------------------------------------------ col_end / col_fused
 template <class C, class RT, int N0, bool FUSED>
-__global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs a) {
-    constexpr int L = LANES2D;
-    using FW = CtaFft<C, N0, L, L, T2D, false>;
-    using FI = CtaFft<C, N0, L, L, T2D, true>;
+__global__ void __launch_bounds__(threads_2d<C, N0>(), min_blocks_2d<C, N0>()) k_col_end(const KArgs a) {
+    constexpr int L = lanes_2d<C>(), T = threads_2d<C, N0>();
+    using FW = CtaFft<C, N0, L, L, T, false>;
+    using FI = CtaFft<C, N0, L, L, T, true>;
     using R = typename cx_traits<C>::real;
     using ST = state_t<RT>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -356,7 +376,7 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs
     const R scale = (R)1 / (R)N0;
 
     auto load_tile = [&](const C* src) {
-        batched_copy<C, N0 * L>([&](int item) { return src[(size_t)(item / L) * n1 + c0 + item % L]; },
+        batched_copy<C, N0 * L, T>([&](int item) { return src[(size_t)(item / L) * n1 + c0 + item % L]; },
                                 [&](int item, C v) { buf[item] = v; });
         __syncthreads();
         run_fwd<FW>(buf, tw, twl, ilog2(N0));
@@ -364,13 +384,13 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs
     load_tile(reinterpret_cast<const C*>(a.aux2) + (size_t)b * NP);
 
     if (a.mode == MODE_INIT) {
-        for (int item = threadIdx.x; item < N0 * L; item += T2D) {
+        for (int item = threadIdx.x; item < N0 * L; item += T) {
             const int lane = item % L, m0 = item / L;
             ringb[(size_t)a.out_slot * NP + (size_t)m0 * n1 + c0 + lane] = cvt<RT>(norm_of(buf[m0 * L + lane], scale));
         }
         __syncthreads();
         load_tile(reinterpret_cast<const C*>(a.aux) + (size_t)b * NP);
-        for (int item = threadIdx.x; item < N0 * L; item += T2D) {
+        for (int item = threadIdx.x; item < N0 * L; item += T) {
             const int lane = item % L, m0 = item / L;
             st[(size_t)m0 * n1 + c0 + lane] = d_to_st<ST>(cvt<double2>(norm_of(buf[m0 * L + lane], scale)));
         }
@@ -379,7 +399,7 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs
 
     const bool step = (a.mode == MODE_STEP);
 #pragma unroll 1
-    for (int item = threadIdx.x; item < N0 * L; item += T2D) {
+    for (int item = threadIdx.x; item < N0 * L; item += T) {
         const int lane = item % L, m0 = item / L;
         const int m1 = c0 + lane;
         const size_t idx = (size_t)m0 * n1 + m1;
@@ -390,7 +410,7 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_col_end(const KArgs
         __syncthreads();
         FI::run(buf, tw, twl);
         C* T1 = reinterpret_cast<C*>(a.aux) + (size_t)b * NP;
-        for (int item = threadIdx.x; item < N0 * L; item += T2D) {
+        for (int item = threadIdx.x; item < N0 * L; item += T) {
             const int lane = item % L, i0 = item / L;
             T1[(size_t)i0 * n1 + c0 + lane] = buf[i0 * L + lane];
         }
@@ -467,7 +487,7 @@ __global__ void __launch_bounds__(T2D, TDSE_MINB2D) k_col_fused_ip(const KArgs a
     if (NCH > 1) stage(1);
 
     const float2* T2 = reinterpret_cast<const float2*>(a.aux2) + (size_t)b * NP;
-    batched_copy<float2, N0 * L>([&](int item) { return T2[(size_t)(item / L) * n1 + c0 + item % L]; },
+    batched_copy<float2, N0 * L, T2D>([&](int item) { return T2[(size_t)(item / L) * n1 + c0 + item % L]; },
                                  [&](int item, float2 v) { buf[item] = v; });
     __syncthreads();
     FW::run(buf, a.tw32_0, a.tw32lo_0);
@@ -574,21 +594,21 @@ static cudaError_t set_smem(K kern, size_t smem, bool& done) {
 
 template <class C, class RT, int N0>
 static cudaError_t col_begin_n(const KArgs& a, cudaStream_t s) {
-    const size_t smem = (size_t)N0 * LANES2D * sizeof(C);
+    const size_t smem = (size_t)N0 * lanes_2d<C>() * sizeof(C);
     static bool done = false;
     cudaError_t e = set_smem(k_col_begin<C, RT, N0>, smem, done);
     if (e != cudaSuccess) return e;
-    k_col_begin<C, RT, N0><<<dim3(a.n1 / LANES2D, a.B), T2D, smem, s>>>(a);
+    k_col_begin<C, RT, N0><<<dim3(a.n1 / lanes_2d<C>(), a.B), threads_2d<C, N0>(), smem, s>>>(a);
     return cudaGetLastError();
 }
 
 template <class C, class RT, int N0, bool FUSED>
 static cudaError_t col_end_n(const KArgs& a, cudaStream_t s) {
-    const size_t smem = (size_t)N0 * LANES2D * sizeof(C);
+    const size_t smem = (size_t)N0 * lanes_2d<C>() * sizeof(C);
     static bool done = false;
     cudaError_t e = set_smem(k_col_end<C, RT, N0, FUSED>, smem, done);
     if (e != cudaSuccess) return e;
-    k_col_end<C, RT, N0, FUSED><<<dim3(a.n1 / LANES2D, a.B), T2D, smem, s>>>(a);
+    k_col_end<C, RT, N0, FUSED><<<dim3(a.n1 / lanes_2d<C>(), a.B), threads_2d<C, N0>(), smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -606,11 +626,11 @@ static cudaError_t col_fused_ip_n(const KArgs& a, cudaStream_t s) {
 
 template <class C, int N1>
 static cudaError_t row_mid_n(const KArgs& a, cudaStream_t s) {
-    const size_t smem = (size_t)N1 * (LANES2D + 1) * sizeof(C);
+    const size_t smem = (size_t)N1 * (lanes_2d<C>() + 1) * sizeof(C);
     static bool done = false;
     cudaError_t e = set_smem(k_row_mid<C, N1>, smem, done);
     if (e != cudaSuccess) return e;
-    k_row_mid<C, N1><<<dim3(a.n0 / LANES2D, a.B), T2D, smem, s>>>(a);
+    k_row_mid<C, N1><<<dim3(a.n0 / lanes_2d<C>(), a.B), threads_2d<C, N1>(), smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -684,16 +704,16 @@ static cudaError_t part2d(const KArgs& a, int part, cudaStream_t s) {
 // Transform along axis 1 of [B n0][N1][n2] (one CTA per 8 consecutive i2 of
 // one (instance, i0) plane), in place in X: forward with 1/N1, or inverse.
 template <class C, int N1, bool INV>
-__global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_axis1(const KArgs a, C* X) {
-    constexpr int L = LANES2D;
-    using F = CtaFft<C, N1, L, L, T2D, INV>;
+__global__ void __launch_bounds__(threads_2d<C, N1>(), min_blocks_2d<C, N1>()) k_axis1(const KArgs a, C* X) {
+    constexpr int L = lanes_2d<C>(), T = threads_2d<C, N1>();
+    using F = CtaFft<C, N1, L, L, T, INV>;
     using R = typename cx_traits<C>::real;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     const int n2 = a.tn2;
     const size_t plane = (size_t)blockIdx.z * a.tn0 + blockIdx.y;
     C* base = X + plane * (size_t)N1 * n2 + (size_t)blockIdx.x * L;
-    batched_copy<C, N1 * L>([&](int item) { return base[(size_t)(item / L) * n2 + item % L]; },
+    batched_copy<C, N1 * L, T>([&](int item) { return base[(size_t)(item / L) * n2 + item % L]; },
                             [&](int item, C v) { buf[item] = v; });
     __syncthreads();
     const tw_t<C>* tw;
@@ -701,19 +721,19 @@ __global__ void __launch_bounds__(T2D, min_blocks_2d<C>()) k_axis1(const KArgs a
     if constexpr (is_f64<C>::value) { tw = a.tw64_1; twl = tw; } else { tw = a.tw32_1; twl = a.tw32lo_1; }
     run_fwd<F>(buf, tw, twl, INV ? 0 : ilog2(N1));
     const R scale = (R)1 / (R)N1;
-    for (int item = threadIdx.x; item < N1 * L; item += T2D)
+    for (int item = threadIdx.x; item < N1 * L; item += T)
         base[(size_t)(item / L) * n2 + item % L] = INV ? buf[item] : norm_of(buf[item], scale);
 }
 
 template <class C, int N1>
 static cudaError_t axis1_n(const KArgs& a, bool inv, void* X, cudaStream_t s) {
-    const size_t smem = (size_t)N1 * LANES2D * sizeof(C);
+    const size_t smem = (size_t)N1 * lanes_2d<C>() * sizeof(C);
     static bool done_f = false, done_i = false;
     cudaError_t e = inv ? set_smem(k_axis1<C, N1, true>, smem, done_i) : set_smem(k_axis1<C, N1, false>, smem, done_f);
     if (e != cudaSuccess) return e;
-    const dim3 grid(a.tn2 / LANES2D, a.tn0, a.B);
-    if (inv) k_axis1<C, N1, true><<<grid, T2D, smem, s>>>(a, static_cast<C*>(X));
-    else k_axis1<C, N1, false><<<grid, T2D, smem, s>>>(a, static_cast<C*>(X));
+    const dim3 grid(a.tn2 / lanes_2d<C>(), a.tn0, a.B);
+    if (inv) k_axis1<C, N1, true><<<grid, threads_2d<C, N1>(), smem, s>>>(a, static_cast<C*>(X));
+    else k_axis1<C, N1, false><<<grid, threads_2d<C, N1>(), smem, s>>>(a, static_cast<C*>(X));
     return cudaGetLastError();
 }
 

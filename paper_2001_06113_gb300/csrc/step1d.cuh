@@ -184,7 +184,8 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
                 for (int r = 0; r < FI::RL; ++r) {
                     R vh, vl;
                     Vat(j + r * FI::NBL, vh, vl);
-                    m[p][r] = implicit_solve_times_V(m[p][r], vh, vl, hmu0);
+                    if constexpr (F64) m[p][r] = implicit_solve_times_V(m[p][r], vh, hmu0);
+                    else m[p][r] = implicit_solve_times_V(m[p][r], vh, vl, hmu0);
                 }
             }
         }

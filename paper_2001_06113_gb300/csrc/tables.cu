@@ -6,7 +6,7 @@
 //          [t_a, t_b] e^{i k (phi(t_b) - phi(t_a))} = adv[m >> lb] adv[nh + (m & (nl-1))],
 //          k = m - n [m >= n/2] split as (m_hi nl - n [m_hi nl >= n/2]) + m_lo;
 //      2D: q_d[m] = e^{-i k_d^2 h + i k_d (phi_d(t_b) - phi_d(t_a))} per interval/axis;
-//    stored as FP64 (FP64 mode) or double-float (mixed start-up);
+//    stored as fixed-point factors (fx.cuh; FP64 mode) or double-float (mixed start-up);
 //  * absolute phases for the interaction picture, E_n = e^{-i |k|^2 t_n + i k.phi(t_n)}:
 //      2D: separable per axis, e_d[n][m];  1D: kinetic part split over n as
 //      e^{-i k^2 n dt} = khi[n / 32][m] klo[n % 32][m], advective part as above;
@@ -50,7 +50,7 @@ __global__ void k_roots(double2* w64, float2* w32, int n) {
     w32[m] = make_float2((float)c, (float)s);
 }
 
-__global__ void k_kin1d(double2* kin64, float4* kinff, int n, int L, double dt) {
+__global__ void k_kin1d(int4* kin64, float4* kinff, int n, int L, double dt) {
     int m = blockIdx.x * blockDim.x + threadIdx.x;
     int c = blockIdx.y;
     if (m >= n || c >= L) return;
@@ -58,7 +58,7 @@ __global__ void k_kin1d(double2* kin64, float4* kinff, int n, int L, double dt) 
     const double h = dt / (double)(1 << c);
     double s, co;
     sincos(-(k * k) * h, &s, &co);
-    if (kin64) kin64[(size_t)c * n + m] = make_double2(co, s);
+    if (kin64) kin64[(size_t)c * n + m] = fx_factor(co, s);
     if (kinff) kinff[(size_t)c * n + m] = ff_from_cs(co, s);
 }
 
@@ -70,7 +70,7 @@ __device__ __forceinline__ double split_k(int t, int n, int nh, int nl) {
     return (double)(t - nh);
 }
 
-__global__ void k_adv1d(double2* adv64, float4* advff, const int2* iv, int n_int, const double* phi, int ntf, int n,
+__global__ void k_adv1d(int4* adv64, float4* advff, const int2* iv, int n_int, const double* phi, int ntf, int n,
                         int nh, int nl) {
     const int i = blockIdx.x;
     const int2 ab = iv[i];
@@ -79,14 +79,14 @@ __global__ void k_adv1d(double2* adv64, float4* advff, const int2* iv, int n_int
     for (int t = threadIdx.x; t < nh + nl; t += blockDim.x) {
         double s, c;
         sincos(split_k(t, n, nh, nl) * dphi, &s, &c);
-        if (adv64) adv64[base + t] = make_double2(c, s);
+        if (adv64) adv64[base + t] = fx_factor(c, s);
         if (advff) advff[base + t] = ff_from_cs(c, s);
     }
 }
 
 // Separable one-step phases of the 2D / 3D steps, one row of n0 + n1 (+ n2)
 // factors per interval: exp(-i k^2 h + i k dphi_axis) for each axis's k.
-__global__ void k_q2d(double2* q64, float4* qff, const int2* iv, int n_int, const double* phi, int ntf, int n0,
+__global__ void k_q2d(int4* q64, float4* qff, const int2* iv, int n_int, const double* phi, int ntf, int n0,
                       int n1, int n2, double dt) {
     const int i = blockIdx.x;
     const int2 ab = iv[i];
@@ -103,7 +103,7 @@ __global__ void k_q2d(double2* q64, float4* qff, const int2* iv, int n_int, cons
         const double k = kmode(m, ax == 0 ? n0 : (ax == 1 ? n1 : n2));
         double s, c;
         sincos(-(k * k) * h + k * (ax == 0 ? d0 : (ax == 1 ? d1 : d2)), &s, &c);
-        if (q64) q64[base + t] = make_double2(c, s);
+        if (q64) q64[base + t] = fx_factor(c, s);
         if (qff) qff[base + t] = ff_from_cs(c, s);
     }
 }
@@ -277,19 +277,19 @@ cudaError_t launch_twiddles(int4* tw64, float2* tw32, float2* tw32lo, int n, cud
     return cudaGetLastError();
 }
 
-cudaError_t launch_kin1d(double2* kin64, float4* kinff, int n, int L, double dt, cudaStream_t s) {
+cudaError_t launch_kin1d(int4* kin64, float4* kinff, int n, int L, double dt, cudaStream_t s) {
     k_kin1d<<<dim3((n + 255) / 256, L), 256, 0, s>>>(kin64, kinff, n, L, dt);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adv1d(double2* adv64, float4* advff, const int2* intervals, int n_int, const double* phi, int ntf,
+cudaError_t launch_adv1d(int4* adv64, float4* advff, const int2* intervals, int n_int, const double* phi, int ntf,
                          int n, int nh, int nl, cudaStream_t s) {
     if (n_int <= 0) return cudaSuccess;
     k_adv1d<<<n_int, 128, 0, s>>>(adv64, advff, intervals, n_int, phi, ntf, n, nh, nl);
     return cudaGetLastError();
 }
 
-cudaError_t launch_q2d(double2* q64, float4* qff, const int2* intervals, int n_int, const double* phi, int ntf,
+cudaError_t launch_q2d(int4* q64, float4* qff, const int2* intervals, int n_int, const double* phi, int ntf,
                        int n0, int n1, int n2, double dt, cudaStream_t s) {
     if (n_int <= 0) return cudaSuccess;
     k_q2d<<<n_int, 256, 0, s>>>(q64, qff, intervals, n_int, phi, ntf, n0, n1, n2, dt);
