@@ -1013,6 +1013,24 @@ tdse_status tdse_step(tdse_ctx* c, int nsteps, void* stream) {
         tdse_status st = do_init(c, s);
         if (st != TDSE_OK) return st;
     }
+    if (c->d == 1 && !c->four1d && !c->mixed && run1d64_supported(c->n0)) {
+        KArgs a = base_args(c);
+        set_weights(a, c->cfg.dt, c->mu, c->m);
+        Run1DArgs g{};
+        g.n_first = c->step + 1;
+        g.k = nsteps;
+        g.order = c->m;
+        g.L = c->L;
+        g.S = c->S;
+        g.S_eff = c->S_eff;
+        g.n_int_startup = c->n_int_startup;
+        g.vtable = c->vtable ? 1 : 0;
+        std::copy(c->rich, c->rich + 4, g.rich);
+        for (int2& w : g.half_w) w = make_int2(1 << 27, 0);     // (1/2) / 2 in units of 2^-61
+        TDSE_CK(c, launch_run1d64(a, g, s));
+        c->step += nsteps;
+        return TDSE_OK;
+    }
     int k = 0;
     while (k < nsteps) {
         const int n = c->step + 1;

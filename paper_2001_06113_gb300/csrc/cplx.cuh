@@ -126,6 +126,17 @@ template <int N, bool INV> struct FftPlan {
     static constexpr int ns(int s) { return s == 0 ? 1 : ns(s - 1) * radix(s - 1); }
 };
 
+// Radix-4 passes (and one radix-2 pass, placed as above) for transforms whose
+// latency counts: half the work and registers per thread of a radix-8 pass.
+template <int N, bool INV> struct FftPlan4 {
+    static constexpr int P = ilog2(N);
+    static constexpr int NPASS = (P + 1) / 2;
+    static constexpr int radix(int s) {
+        return P % 2 == 0 ? 4 : (NPASS >= 3 ? (s == 1 ? 2 : 4) : ((INV ? (s == NPASS - 1) : (s == 0)) ? 2 : 4));
+    }
+    static constexpr int ns(int s) { return s == 0 ? 1 : ns(s - 1) * radix(s - 1); }
+};
+
 // v * w (w from tw, conjugated for the inverse).
 // TDSE_TWIDDLE_LO = 1 applies the FP32 twiddle as hi + lo.  Off by default:
 // on the 512^2 mixed workload it lowers the 2000-step error from 5.1e-7 to
@@ -375,9 +386,9 @@ struct CtaFft {
 //
 // Pass S of radix R with its butterflies' values in v: twiddle and 1/R for
 // S > 0, then the R-point DFT.
-template <int N, bool INV>
+template <int N, bool INV, class PlanT = FftPlan<N, INV>>
 struct FxPass {
-    using Plan = FftPlan<N, INV>;
+    using Plan = PlanT;
     static constexpr int S0 = 62 - ilog2(Plan::radix(0));       // input scale
     static constexpr int GAIN = ilog2(N / Plan::radix(0));      // the passes' 1/R
     template <int S>

@@ -129,6 +129,20 @@ cudaError_t periodic1d_prepare(int n, int combo);
 // launch shape `shape` (0 default, 1 alternative); 0 if that shape is not built.
 int periodic1d_f32_threads(int n, int shape);
 
+// ---- 1D FP64 runs: steps n_first .. n_first + k - 1 of every instance in one
+// launch (run1d64.cu); a: the arguments of an Adams step (dt, weights) with
+// V0 at row 0.
+struct Run1DArgs {
+    int n_first, k;
+    int order, L, S, S_eff;   // Adams order, Richardson chains, start-up steps
+    int n_int_startup;        // first phase interval of the steps after the start-up
+    int vtable;               // V0 holds one row per evaluation time
+    double rich[4];           // Richardson coefficients of the chains
+    int2 half_w[2];           // the trapezoidal weights, as KArgs::mu_w
+};
+bool run1d64_supported(int n);
+cudaError_t launch_run1d64(const KArgs& a, const Run1DArgs& g, cudaStream_t s);
+
 // ---- uneven 1D batches: one persistent launch for many contexts (mixed steps)
 // A CTA of MULTI_CTA threads takes the next item from a global counter; an
 // item runs `count` instances of one context with the launch variant `var`

@@ -230,14 +230,10 @@ __device__ __forceinline__ float4 mixed_X(const KArgs& a, float4 st, const float
 // sum of |mu_j| is below 4.4, so |S| stays under 2^61.7), u^ and h S_1 share
 // Ex >= E(u^).  100 steps of 4 x 512^2: 51.4 -> 42.5 ms.
 // (Ring loads issued together, lags beyond nhist contribute zero.)
-template <class Ph>
-__device__ __forceinline__ double2 horner_W64(const KArgs& a, double2 uh, const double2* __restrict__ ringb,
-                                              size_t NP, size_t idx, const Ph& ph) {
+template <class W>
+__device__ __forceinline__ double2 fx_horner(double2 uh, const double2 (&r)[MAX_HIST], int nhist,
+                                             const int2* mu_w, int2 h_w, int h_e, W w) {
     constexpr int S0 = 59;
-    double2 r[MAX_HIST];
-#pragma unroll
-    for (int j = 1; j <= MAX_HIST; ++j)
-        r[j - 1] = (j <= a.nhist) ? ringb[(size_t)a.hist_slot[j - 1] * NP + idx] : make_double2(0.0, 0.0);
     unsigned mr = 0;
 #pragma unroll
     for (int j = 1; j <= MAX_HIST; ++j) mr = max(mr, fx_hi(r[j - 1]));
@@ -246,22 +242,31 @@ __device__ __forceinline__ double2 horner_W64(const KArgs& a, double2 uh, const 
     longlong2 S = make_longlong2(0, 0);
 #pragma unroll
     for (int j = MAX_HIST; j >= 1; --j) {
-        if (j <= a.nhist) {
-            if (j < a.nhist) S = fx_mul<false, 3>(S, ph.w64(j));
+        if (j <= nhist) {
+            if (j < nhist) S = fx_mul<false, 3>(S, w(j));
             const longlong2 R = fx_from(r[j - 1], S0, E);
-            S.x += fx_mul_real<4>(R.x, a.mu_w[j]);
-            S.y += fx_mul_real<4>(R.y, a.mu_w[j]);
+            S.x += fx_mul_real<4>(R.x, mu_w[j]);
+            S.y += fx_mul_real<4>(R.y, mu_w[j]);
         }
     }
     // X = u^ - i h S, h = h_w 2^h_e: the shift of h_w S to the scale of u^ is at least 3
-    const int Ex = max(fx_exponent(mu), E + a.h_e + 3);
-    const int sh = min(Ex - E - a.h_e, 63);
-    const long long tx = fx_mul_real<3>(S.x, a.h_w) >> sh, ty = fx_mul_real<3>(S.y, a.h_w) >> sh;
+    const int Ex = max(fx_exponent(mu), E + h_e + 3);
+    const int sh = min(Ex - E - h_e, 63);
+    const long long tx = fx_mul_real<3>(S.x, h_w) >> sh, ty = fx_mul_real<3>(S.y, h_w) >> sh;
     longlong2 X = fx_from(uh, S0, Ex);
     X.x += ty;
     X.y -= tx;
     const int xe = max(mr, mu) >= 0x7ff00000u ? FX_NAN : Ex - 1022 - S0;
-    return fx_to(fx_mul<false, 3>(X, ph.w64(0)), xe);
+    return fx_to(fx_mul<false, 3>(X, w(0)), xe);
+}
+template <class Ph>
+__device__ __forceinline__ double2 horner_W64(const KArgs& a, double2 uh, const double2* __restrict__ ringb,
+                                              size_t NP, size_t idx, const Ph& ph) {
+    double2 r[MAX_HIST];
+#pragma unroll
+    for (int j = 1; j <= MAX_HIST; ++j)
+        r[j - 1] = (j <= a.nhist) ? ringb[(size_t)a.hist_slot[j - 1] * NP + idx] : make_double2(0.0, 0.0);
+    return fx_horner(uh, r, a.nhist, a.mu_w, a.h_w, a.h_e, [&](int j) { return ph.w64(j); });
 }
 
 // 1/d for 1 <= d: the hardware's estimate and one step of Halley's third-order
