@@ -168,6 +168,7 @@ static void plan_workspace(tdse_ctx* c) {
     c->off.err = take(256);
     c->off.scratch = take(256);
     c->off.end = o;
+    c->ws_ckpt = o;
     c->ws_need = o;
 }
 
@@ -629,12 +630,12 @@ static tdse_status set_field(tdse_ctx* c, int instance, tdse_field_fn A, void* u
         std::vector<double> gx, gw;
         gauss_legendre(8, gx, gw);
         const double hs = c->cfg.dt / SUB;
-        double acc[2] = {0.0, 0.0}, comp[2] = {0.0, 0.0};
-        double Av[2] = {0.0, 0.0};
+        double acc[3] = {0.0, 0.0, 0.0}, comp[3] = {0.0, 0.0, 0.0};
+        double Av[3] = {0.0, 0.0, 0.0};
         for (int mm = 0; mm + 1 < c->ntf; ++mm) {
             const double t0 = (double)mm * hs, t1 = (double)(mm + 1) * hs;
             const double half = 0.5 * (t1 - t0), mid = 0.5 * (t0 + t1);
-            double part[2] = {0.0, 0.0};
+            double part[3] = {0.0, 0.0, 0.0};
             for (int q = 0; q < 8; ++q) {
                 A(mid + half * gx[q], Av, user);
                 for (int dd = 0; dd < c->d; ++dd) part[dd] += gw[q] * Av[dd];
@@ -647,6 +648,12 @@ static tdse_status set_field(tdse_ctx* c, int instance, tdse_field_fn A, void* u
                 phi[(size_t)dd * c->ntf + mm + 1] = acc[dd] + comp[dd];
             }
         }
+    }
+    if (c->fs) {
+        double dphi[3] = {0.0, 0.0, 0.0};
+        fs_largest_dphi(c, phi.data(), dphi);
+        const tdse_status st = fs_field_range(c, lo, hi, dphi, s);
+        if (st != TDSE_OK) return st;
     }
     for (int b = lo; b < hi; ++b) {
         TDSE_CK(c, cudaMemcpyAsync(c->P<double>(c->off.phi) + (size_t)b * c->d * c->ntf, phi.data(),
@@ -671,6 +678,11 @@ tdse_status tdse_set_pulse(tdse_ctx* c, int instance, double A0, double omega, d
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // phi in closed form on the device (no host pass over the fine time grid)
     const double d2[3] = {dir[0], c->d >= 2 ? dir[1] : 0.0, c->d == 3 ? dir[2] : 0.0};
+    if (c->fs) {
+        const double dphi[3] = {A0 * c->cfg.dt * d2[0], A0 * c->cfg.dt * d2[1], A0 * c->cfg.dt * d2[2]};
+        const tdse_status st = fs_field_range(c, lo, hi, dphi, s);
+        if (st != TDSE_OK) return st;
+    }
     for (int b = lo; b < hi; ++b) {
         TDSE_CK(c, launch_pulse_phi(c->P<double>(c->off.phi) + (size_t)b * c->d * c->ntf, c->ntf, c->d,
                                     c->cfg.dt / SUB, A0, omega, Tp, d2, s));
@@ -1183,7 +1195,7 @@ tdse_status tdse_residual_report(tdse_ctx* c, double* rho, int* corrections, int
     return TDSE_OK;
 }
 
-// ---- checkpoint: header, then the whole workspace
+// ---- checkpoint: header, then the workspace up to ws_ckpt
 namespace {
 constexpr char kCkptMagic[8] = {'T', 'D', 'S', 'E', 'C', 'K', 'P', '2'};
 struct CkptHeader {
@@ -1206,7 +1218,7 @@ void fill_header(const tdse_ctx* c, CkptHeader& h) {
         h.n_r = g.n_r; h.H = g.H;
     }
     h.dt = g.dt;
-    h.ws_bytes = c->ws_need;
+    h.ws_bytes = c->ws_ckpt;
     h.step = c->step; h.inited = c->inited; h.ip = c->ip;
     h.res_every = c->res_every; h.res_checks = c->res_checks; h.res_tol = c->res_tol;
 }
@@ -1214,7 +1226,7 @@ void fill_header(const tdse_ctx* c, CkptHeader& h) {
 
 tdse_status tdse_save(tdse_ctx* c, void* blob, size_t* size, void* stream) {
     if (!c || !size) return TDSE_EINVAL;
-    const size_t need = sizeof(CkptHeader) + 2 * (size_t)c->B + c->ws_need;
+    const size_t need = sizeof(CkptHeader) + 2 * (size_t)c->B + c->ws_ckpt;
     if (!blob) {
         *size = need;
         return TDSE_OK;
@@ -1227,10 +1239,11 @@ tdse_status tdse_save(tdse_ctx* c, void* blob, size_t* size, void* stream) {
     char* out = static_cast<char*>(blob);
     std::memcpy(out, &h, sizeof(h));
     for (int b = 0; b < c->B; ++b) {
-        out[sizeof(h) + 2 * b] = c->have_V[b];
+        // free space: the scale of the phase tables rides in the flag (g + 1 above bit 0)
+        out[sizeof(h) + 2 * b] = (char)(c->have_V[b] | (c->fs ? (c->F.g[b] + 1) << 1 : 0));
         out[sizeof(h) + 2 * b + 1] = c->have_u0[b];
     }
-    TDSE_CK(c, cudaMemcpyAsync(out + sizeof(h) + 2 * (size_t)c->B, c->ws, c->ws_need, cudaMemcpyDeviceToHost, s));
+    TDSE_CK(c, cudaMemcpyAsync(out + sizeof(h) + 2 * (size_t)c->B, c->ws, c->ws_ckpt, cudaMemcpyDeviceToHost, s));
     TDSE_CK(c, cudaStreamSynchronize(s));
     *size = need;
     return TDSE_OK;
@@ -1239,7 +1252,7 @@ tdse_status tdse_save(tdse_ctx* c, void* blob, size_t* size, void* stream) {
 tdse_status tdse_load(tdse_ctx* c, const void* blob, size_t size, void* stream) {
     if (!c || !blob) return TDSE_EINVAL;
     if (!c->ws) return c->fail(TDSE_ESTATE, "workspace not bound");
-    const size_t need = sizeof(CkptHeader) + 2 * (size_t)c->B + c->ws_need;
+    const size_t need = sizeof(CkptHeader) + 2 * (size_t)c->B + c->ws_ckpt;
     if (size < need) return c->fail(TDSE_EINVAL, "checkpoint too short");
     CkptHeader h, mine;
     std::memcpy(&h, blob, sizeof(h));
@@ -1253,15 +1266,16 @@ tdse_status tdse_load(tdse_ctx* c, const void* blob, size_t size, void* stream) 
     if (!same) return c->fail(TDSE_EINVAL, "checkpoint of a different configuration");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const char* in = static_cast<const char*>(blob);
-    TDSE_CK(c, cudaMemcpyAsync(c->ws, in + sizeof(h) + 2 * (size_t)c->B, c->ws_need, cudaMemcpyHostToDevice, s));
+    TDSE_CK(c, cudaMemcpyAsync(c->ws, in + sizeof(h) + 2 * (size_t)c->B, c->ws_ckpt, cudaMemcpyHostToDevice, s));
     // the transform and phase tables (functions of the configuration and of
     // phi) are built again: the checkpoint's may be in another version's form
-    tdse_status ts = c->fs ? fs_upload_twiddles(c, s) : build_twiddles(c, s);
+    tdse_status ts = c->fs ? fs_upload_tables(c, s) : build_twiddles(c, s);
+    if (c->fs && ts == TDSE_OK) ts = fs_loaded_field_range(c, in + sizeof(h), s);
     for (int b = 0; b < c->B && ts == TDSE_OK; ++b) ts = build_phase_tables(c, b, s);
     if (ts != TDSE_OK) return ts;
     TDSE_CK(c, cudaStreamSynchronize(s));
     for (int b = 0; b < c->B; ++b) {
-        c->have_V[b] = in[sizeof(h) + 2 * b];
+        c->have_V[b] = in[sizeof(h) + 2 * b] & 1;
         c->have_u0[b] = in[sizeof(h) + 2 * b + 1];
     }
     c->step = h.step;

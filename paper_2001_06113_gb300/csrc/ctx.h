@@ -23,6 +23,7 @@ struct FsAxisHost {
     int M = 0, nu = 0, R = 0, NE = 0, ND = 0, NC = 0, N = 0, p = 0, kappa = 0, q = 0, n_r = 0;
     int NT = 0;                 // terms of the Chebyshev form of the C-type transforms (0: direct sums)
     double H = 0, K = 0, h = 0;
+    int xI = 0;                 // scale of the fixed-point table preI (FsAxis)
     std::vector<double> zeta;   // [N][2] nodes (complex)
     std::vector<double> w;      // [N][2] weights (complex)
 };
@@ -31,10 +32,11 @@ struct FsState {
     FsAxisHost ax[3];
     size_t NM = 0;   // modes per instance (N0 N1 N2)
     size_t NX = 0;   // grid points per instance (M0 M1 M2)
+    std::vector<int> g;     // per instance: extra powers of two in the phase tables' scale (fs_field_range)
     bool f32 = false;   // TDSE_MIXED: FP32 transforms, ring, intermediate and history sum
     struct {
         size_t uhat, ring, chain_uhat, chain_ring, chain_u, u, Z, Y, V0, tfac, phi, iv, scratch, end;
-        size_t zeta[3], preI[3], postI[3], preF[3], postF[3], Gd[3], Fd[3], tw[3], P[3];
+        size_t g, xj[3], zeta[3], preI[3], postI[3], preF[3], postF[3], Gd[3], Fd[3], tw[3], P[3];
         // FP32 copies (f32 only; 0 otherwise)
         size_t preI_f[3], postI_f[3], preF_f[3], postF_f[3], Gd_f[3], Fd_f[3], tw_f[3], P_f[3];
         // FP64 residual check of the FP32 step (f32 only): W / corrected state, R64, u64, intermediates
@@ -71,6 +73,7 @@ struct tdse_ctx {
     // workspace
     char* ws = nullptr;
     size_t ws_need = 0;
+    size_t ws_ckpt = 0;         // leading part that a checkpoint holds (the rest: tables of the configuration, scratch)
     struct {
         size_t uhat, ring, chain_uhat, chain_ring, aux, aux2, V0, V0f, tfac, phi, kin64, kinff, adv64, advff,
             q64, qff, e2d, k1lo, k1hi, a1d, tw64_0, tw32_0, tw64_1, tw32_1, tw32lo_0, tw32lo_1, tw64_2, tw32_2,
@@ -153,7 +156,10 @@ inline size_t vrow(const tdse_ctx* c, int tf) {
 // once the common fields of the context are set.
 tdse_status fs_create(tdse_ctx* c);
 tdse_status fs_bind(tdse_ctx* c, cudaStream_t s);
-tdse_status fs_upload_twiddles(tdse_ctx* c, cudaStream_t s);
+tdse_status fs_upload_tables(tdse_ctx* c, cudaStream_t s);
+tdse_status fs_field_range(tdse_ctx* c, int lo, int hi, const double* dphi, cudaStream_t s);
+tdse_status fs_loaded_field_range(tdse_ctx* c, const char* flags, cudaStream_t s);
+void fs_largest_dphi(const tdse_ctx* c, const double* phi, double* dphi);
 tdse_status fs_build_phase_tables(tdse_ctx* c, int b, cudaStream_t s);
 tdse_status fs_set_initial(tdse_ctx* c, int b, const double* u0, cudaMemcpyKind kind, cudaStream_t s);
 tdse_status fs_steps(tdse_ctx* c, int nsteps, cudaStream_t s);

@@ -7,7 +7,7 @@ namespace {
 
 // P[iv][m] = exp(-i zeta_m^2 s + i zeta_m (phi(t1) - phi(t0))), s = t1 - t0
 // (eq. uhatxirecur with zeta for k), one instance.
-__global__ void k_fs_phase(double2* P, const double2* zeta, int N, const int2* iv, int n_int, const double* phi,
+__global__ void k_fs_phase(int4* P, float2* Pf, double scale, const double2* zeta, int N, const int2* iv, int n_int, const double* phi,
                            double dt8) {
     for (int it = blockIdx.y; it < n_int; it += gridDim.y) {
         const int2 q = iv[it];
@@ -20,14 +20,10 @@ __global__ void k_fs_phase(double2* P, const double2* zeta, int N, const int2* i
             double sn, cs;
             sincos(im, &sn, &cs);
             const double e = exp(re);
-            P[(size_t)it * N + m] = make_double2(e * cs, e * sn);
+            P[(size_t)it * N + m] = fx_factor(scale * (e * cs), scale * (e * sn));
+            if (Pf) Pf[(size_t)it * N + m] = make_float2((float)(e * cs), (float)(e * sn));
         }
     }
-}
-
-__global__ void k_fs_to_f32(float2* dst, const double2* src, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dst[i] = make_float2((float)src[i].x, (float)src[i].y);
 }
 
 // ---- FP64 residual check of the FP32-transform step
@@ -103,7 +99,7 @@ __global__ void k_fs_res_apply(const int* flags, size_t NM, size_t NX, size_t to
 
 cudaError_t run(const FsArgs& a, int which, int flag, int f32, cudaStream_t s) {
     if (f32) return launch_fs_f32(a, which, flag, s);
-    return fs::dispatch<double2>(a, fs::axis_of(a, which), which, flag, s);
+    return fs::dispatch<fs::NumF64>(a, fs::axis_of(a, which), which, flag, s);
 }
 
 }  // namespace
@@ -121,11 +117,12 @@ cudaError_t launch_fs_phys(const FsArgs& a, int from_usrc, int f32, cudaStream_t
 }
 cudaError_t launch_fs_mid(const FsArgs& a, int dir, int f32, cudaStream_t s) { return run(a, 3, dir, f32, s); }
 
-cudaError_t launch_fs_phase(double2* P, const double2* zeta, int N, const int2* intervals, int n_int,
+cudaError_t launch_fs_phase(int4* P, float2* Pf, int g, const double2* zeta, int N, const int2* intervals, int n_int,
                             const double* phi, double dt, cudaStream_t s) {
     if (n_int <= 0) return cudaSuccess;
     const unsigned gy = n_int < 65535 ? (unsigned)n_int : 65535u;
-    k_fs_phase<<<dim3((N + 255) / 256, gy), 256, 0, s>>>(P, zeta, N, intervals, n_int, phi, dt / 8.0);
+    k_fs_phase<<<dim3((N + 255) / 256, gy), 256, 0, s>>>(P, Pf, ldexp(1.0, -(1 + g)), zeta, N, intervals, n_int, phi,
+                                                            dt / 8.0);
     return cudaGetLastError();
 }
 
@@ -163,14 +160,6 @@ cudaError_t launch_fs_res_apply(const int* flags, int B, size_t NM, size_t NX, d
     const size_t tm = NM * (size_t)B, tx = NX * (size_t)B;
     k_fs_res_apply<<<grid_of(tm > tx ? tm : tx), 256, 0, s>>>(flags, NM, NX, tm, tx, uhat, Wc, ring, rstride, R64, u,
                                                                 u64);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fs_to_f32(float2* dst, const double2* src, size_t n, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    size_t g = (n + 255) / 256;
-    if (g > 4096) g = 4096;
-    k_fs_to_f32<<<(unsigned)g, 256, 0, s>>>(dst, src, n);
     return cudaGetLastError();
 }
 

@@ -4,7 +4,7 @@
 namespace tdse {
 
 cudaError_t launch_fs_f32(const FsArgs& a, int which, int flag, cudaStream_t s) {
-    return fs::dispatch<float2>(a, fs::axis_of(a, which), which, flag, s);
+    return fs::dispatch<fs::NumF32>(a, fs::axis_of(a, which), which, flag, s);
 }
 
 }  // namespace tdse

@@ -226,7 +226,7 @@ void make_cheb_tables(const FsAxisHost& A, AxisTables& T) {
 // Host tables of one axis (fsargs.h FsAxis), in FP64 from long double phases.
 AxisTables make_tables(const FsAxisHost& A) {
     AxisTables T;
-    const int M = A.M, R = A.R, nu = A.nu, NE = A.NE, ND = A.ND;
+    const int M = A.M, R = A.M > 256 ? 2 * A.R : A.R, nu = A.nu, NE = A.NE, ND = A.ND;   // R lines per block (freespace.cuh)
     const long double h = A.h;
     T.zeta = A.zeta;
     auto put = [](std::vector<double>& v, double mag, long double theta) {
@@ -272,7 +272,8 @@ AxisTables make_tables(const FsAxisHost& A) {
             T.Fd.push_back(-f * s);
         }
     }
-    for (int m = 0; m < M; ++m) put(T.tw, 1.0, -2.0L * kPiL * m / M);
+    const int MF = A.M > 256 ? M / 2 : M;        // transform length
+    for (int m = 0; m < MF; ++m) put(T.tw, 1.0, -2.0L * kPiL * m / MF);
     if (A.NT > 0) make_cheb_tables(A, T);
     return T;
 }
@@ -296,20 +297,22 @@ FsArgs fs_base(const tdse_ctx* c) {
         X.NE = A.NE;
         X.ND = A.ND;
         X.N = A.N;
-        X.preI = c->P<double2>(F.off.preI[x]);
-        X.postI = c->P<double2>(F.off.postI[x]);
-        X.preF = c->P<double2>(F.off.preF[x]);
-        X.postF = c->P<double2>(F.off.postF[x]);
-        X.Gd = c->P<double2>(F.off.Gd[x]);
-        X.Fd = c->P<double2>(F.off.Fd[x]);
+        X.preI = c->P<int4>(F.off.preI[x]);
+        X.postI = c->P<int4>(F.off.postI[x]);
+        X.preF = c->P<int4>(F.off.preF[x]);
+        X.postF = c->P<int4>(F.off.postF[x]);
+        X.Gd = c->P<int4>(F.off.Gd[x]);
+        X.Fd = c->P<int4>(F.off.Fd[x]);
         X.tw = c->P<int4>(F.off.tw[x]);
-        X.P = c->P<double2>(F.off.P[x]);
+        X.P = c->P<int4>(F.off.P[x]);
+        X.xI = A.xI;
+        X.xj = c->P<int>(F.off.xj[x]);
         X.p = A.p;
         X.NC = A.NC;
         X.NT = A.NT;
         if (A.NT > 0) {
-            X.Lf = c->P<double2>(F.off.Lf[x]);
-            X.Li = c->P<double2>(F.off.Li[x]);
+            X.Lf = c->P<int4>(F.off.Lf[x]);
+            X.Li = c->P<int4>(F.off.Li[x]);
             X.Tc = c->P<double>(F.off.Tc[x]);
             X.TcW = c->P<double2>(F.off.TcW[x]);
             if (F.f32) {
@@ -330,6 +333,7 @@ FsArgs fs_base(const tdse_ctx* c) {
             X.P_f = c->P<float2>(F.off.P_f[x]);
         }
     }
+    a.g = c->P<int>(F.off.g);
     a.n_int = c->n_int;
     a.uhat = c->P<double2>(F.off.uhat);
     a.ring = c->P<double2>(F.off.ring);
@@ -348,6 +352,17 @@ FsArgs fs_base(const tdse_ctx* c) {
 void set_time(const tdse_ctx* c, FsArgs& a, int tf) {
     a.tf = tf;
     a.V0 = c->P<double>(c->F.off.V0) + vrow(c, tf) * c->F.NX;
+}
+
+// Step size and weights of a step with n history terms.
+void set_weights(FsArgs& a, double h, const double* mu, int n) {
+    auto factor = [](double x, int2& w) { fx_limbs(std::llround(std::ldexp(x, 61)), w.x, w.y); };
+    a.nhist = n;
+    a.h = h;
+    for (int j = 0; j <= n; ++j) {
+        a.mu[j] = mu[j];
+        factor(0.5 * mu[j], a.mu_w[j]);
+    }
 }
 
 // Ring slot `slot` of a ring with rsz-byte elements (as the kernels' double2* field).
@@ -438,10 +453,8 @@ tdse_status fs_startup_step(tdse_ctx* c, int n, cudaStream_t s) {
             a.ring = cr;
             a.ring_slots = 1;
             a.u = cx + ch * BX;
-            a.nhist = 1;
-            a.h = c->cfg.dt / (double)(1 << ch);
-            a.mu[0] = 0.5;
-            a.mu[1] = 0.5;
+            const double half[2] = {0.5, 0.5};
+            set_weights(a, c->cfg.dt / (double)(1 << ch), half, 1);
             a.hist_slot[0] = 0;
             a.out_slot = 0;
             a.interval[0] = startup_interval(c, n, ch, i);
@@ -459,9 +472,7 @@ tdse_status fs_startup_step(tdse_ctx* c, int n, cudaStream_t s) {
 
 FsArgs adams_args(const tdse_ctx* c, int n) {
     FsArgs a = fs_base(c);
-    a.nhist = c->m - 1;
-    a.h = c->cfg.dt;
-    for (int j = 0; j < c->m; ++j) a.mu[j] = c->mu[j];
+    set_weights(a, c->cfg.dt, c->mu, c->m - 1);
     for (int j = 1; j <= a.nhist; ++j) a.hist_slot[j - 1] = slot_of(c, n - j);
     a.out_slot = slot_of(c, n);
     for (int i = 0; i < a.nhist; ++i) a.interval[i] = main_interval(c, n - i);
@@ -497,9 +508,7 @@ tdse_status fs_residual_check(tdse_ctx* c, cudaStream_t s) {
     a.u = u64;
     a.Z = F.off.Z64 ? c->P<double2>(F.off.Z64) : nullptr;
     a.Y = F.off.Y64 ? c->P<double2>(F.off.Y64) : nullptr;
-    a.nhist = 0;
-    a.h = c->cfg.dt;
-    a.mu[0] = c->mu[0];
+    set_weights(a, c->cfg.dt, c->mu, 0);
     a.out_slot = 0;
     a.interval[0] = F.zero_iv;
     set_time(c, a, SUB * n);
@@ -625,6 +634,21 @@ tdse_status fs_create(tdse_ctx* c) {
     }
     F.off.scratch = take(256);
     F.off.end = o;
+    c->ws_ckpt = o;
+    F.off.g = take(B * sizeof(int));
+    // not part of a checkpoint: exponents of the fixed-point tables; factor tables
+    // of twice the lines for grids of more than 256 points
+    for (int x = 0; x < c->d; ++x) {
+        const FsAxisHost& A = F.ax[x];
+        F.off.xj[x] = take((size_t)6 * A.M * sizeof(int));
+        if (A.M <= 256) continue;
+        F.off.postI[x] = take((size_t)4 * A.nu * 16);
+        F.off.preF[x] = take((size_t)4 * A.nu * 16);
+        if (F.f32) {
+            F.off.postI_f[x] = take((size_t)4 * A.nu * 8);
+            F.off.preF_f[x] = take((size_t)4 * A.nu * 8);
+        }
+    }
     c->ws_need = o;
     // fields the shared entry points use
     c->off = {};
@@ -642,32 +666,80 @@ tdse_status fs_create(tdse_ctx* c) {
     return TDSE_OK;
 }
 
-tdse_status fs_bind(tdse_ctx* c, cudaStream_t s) {
+namespace {
+// Power of two that brings the modulus `big` into 1/2..1.
+int exponent_of(double big) {
+    int x = 0;
+    if (big > 0.0) std::frexp(big, &x);
+    return x;
+}
+// Fixed-point factors of complex values v, value i scaled by 2^-x(i).
+template <class X>
+std::vector<int4> factors(const std::vector<double>& v, X x) {
+    std::vector<int4> w(v.size() / 2);
+    for (size_t i = 0; i < w.size(); ++i) {
+        fx_limbs(std::llround(std::ldexp(v[2 * i], 61 - x(i))), w[i].x, w[i].y);
+        fx_limbs(std::llround(std::ldexp(v[2 * i + 1], 61 - x(i))), w[i].z, w[i].w);
+    }
+    return w;
+}
+}  // namespace
+
+// The tables of every axis (functions of the configuration alone).
+tdse_status fs_upload_tables(tdse_ctx* c, cudaStream_t s) {
     FsState& F = c->F;
     for (int x = 0; x < c->d; ++x) {
-        const AxisTables T = make_tables(F.ax[x]);
-        auto up = [&](size_t off, const std::vector<double>& v) {
-            return cudaMemcpyAsync(c->P<double>(off), v.data(), v.size() * 8, cudaMemcpyHostToDevice, s);
+        FsAxisHost& A = F.ax[x];
+        const AxisTables T = make_tables(A);
+        const size_t M = A.M, R = A.M > 256 ? 2 * A.R : A.R;
+        // largest modulus of entries first, first + step, .. of a table
+        auto largest = [](const std::vector<double>& v, size_t first, size_t step, size_t n) {
+            double big = 0.0;
+            for (size_t i = 0; i < n; ++i)
+                big = std::fmax(big, std::hypot(v[2 * (first + i * step)], v[2 * (first + i * step) + 1]));
+            return big;
         };
-        TDSE_CK(c, up(F.off.zeta[x], T.zeta));
-        TDSE_CK(c, up(F.off.preI[x], T.preI));
-        TDSE_CK(c, up(F.off.postI[x], T.postI));
-        TDSE_CK(c, up(F.off.preF[x], T.preF));
-        TDSE_CK(c, up(F.off.postF[x], T.postF));
-        TDSE_CK(c, up(F.off.Gd[x], T.Gd));
-        TDSE_CK(c, up(F.off.Fd[x], T.Fd));
-        if (F.ax[x].NT > 0) {
-            TDSE_CK(c, up(F.off.Lf[x], T.Lf));
-            TDSE_CK(c, up(F.off.Li[x], T.Li));
-            TDSE_CK(c, up(F.off.Tc[x], T.Tc));
-            TDSE_CK(c, up(F.off.TcW[x], T.TcW));
+        A.xI = exponent_of(largest(T.preI, 0, 1, T.preI.size() / 2));
+        std::vector<int> xj(6 * M);
+        for (size_t j = 0; j < M; ++j) {
+            for (size_t b = 0; b < 2; ++b) {
+                xj[b * M + j] = exponent_of(largest(T.preF, (b * M + j) * R, 1, R));
+                xj[(3 + b) * M + j] = exponent_of(largest(T.postI, (b * M + j) * R, 1, R));
+            }
+            xj[2 * M + j] = exponent_of(std::fmax(largest(T.Fd, j, M, A.ND), A.NT ? largest(T.Lf, j, M, A.NT) : 0.0));
+            xj[5 * M + j] = exponent_of(std::fmax(largest(T.Gd, j, M, A.ND), A.NT ? largest(T.Li, j, M, A.NT) : 0.0));
+        }
+        auto point = [&](int c) { return [&xj, M, c](size_t i) { return xj[c * M + i % M]; }; };     // [rows][M]
+        auto lines = [&](int c) { return [&xj, R, M, c](size_t i) { return xj[c * M + i / R]; }; };  // [2][M][R], block 1 at c + 1
+        auto whole = [](int x) { return [x](size_t) { return x; }; };
+        auto up = [&](size_t off, const void* p, size_t bytes) -> cudaError_t {
+            const cudaError_t e = cudaMemcpyAsync(c->P<char>(off), p, bytes, cudaMemcpyHostToDevice, s);
+            return e != cudaSuccess ? e : cudaStreamSynchronize(s);   // the source is a temporary
+        };
+        auto up64 = [&](size_t off, const std::vector<double>& v) { return up(off, v.data(), v.size() * 8); };
+        auto upfx = [&](size_t off, const std::vector<double>& v, auto e) {
+            const std::vector<int4> w = factors(v, e);
+            return up(off, w.data(), w.size() * sizeof(int4));
+        };
+        TDSE_CK(c, up64(F.off.zeta[x], T.zeta));
+        TDSE_CK(c, up(F.off.xj[x], xj.data(), xj.size() * sizeof(int)));
+        TDSE_CK(c, upfx(F.off.preI[x], T.preI, whole(A.xI)));
+        TDSE_CK(c, upfx(F.off.postI[x], T.postI, lines(3)));
+        TDSE_CK(c, upfx(F.off.preF[x], T.preF, lines(0)));
+        TDSE_CK(c, upfx(F.off.postF[x], T.postF, whole(0)));
+        TDSE_CK(c, upfx(F.off.Gd[x], T.Gd, point(5)));
+        TDSE_CK(c, upfx(F.off.Fd[x], T.Fd, point(2)));
+        TDSE_CK(c, upfx(F.off.tw[x], T.tw, whole(0)));
+        if (A.NT > 0) {
+            TDSE_CK(c, upfx(F.off.Lf[x], T.Lf, point(2)));
+            TDSE_CK(c, upfx(F.off.Li[x], T.Li, point(5)));
+            TDSE_CK(c, up64(F.off.Tc[x], T.Tc));
+            TDSE_CK(c, up64(F.off.TcW[x], T.TcW));
         }
         // FP32 copies: each complex value rounded from the FP64 table
-        std::vector<float> t32;
-        auto up32 = [&](size_t off, const std::vector<double>& v) -> cudaError_t {
-            t32.assign(v.begin(), v.end());
-            const cudaError_t e = cudaMemcpyAsync(c->P<float>(off), t32.data(), t32.size() * 4, cudaMemcpyHostToDevice, s);
-            return e != cudaSuccess ? e : cudaStreamSynchronize(s);   // t32 is reused
+        auto up32 = [&](size_t off, const std::vector<double>& v) {
+            const std::vector<float> t32(v.begin(), v.end());
+            return up(off, t32.data(), t32.size() * 4);
         };
         if (F.f32) {
             TDSE_CK(c, up32(F.off.preI_f[x], T.preI));
@@ -677,32 +749,71 @@ tdse_status fs_bind(tdse_ctx* c, cudaStream_t s) {
             TDSE_CK(c, up32(F.off.Gd_f[x], T.Gd));
             TDSE_CK(c, up32(F.off.Fd_f[x], T.Fd));
             TDSE_CK(c, up32(F.off.tw_f[x], T.tw));
-            if (F.ax[x].NT > 0) {
+            if (A.NT > 0) {
                 TDSE_CK(c, up32(F.off.Lf_f[x], T.Lf));
                 TDSE_CK(c, up32(F.off.Li_f[x], T.Li));
                 TDSE_CK(c, up32(F.off.Tc_f[x], T.Tc));
                 TDSE_CK(c, up32(F.off.TcW_f[x], T.TcW));
             }
         }
-        TDSE_CK(c, cudaStreamSynchronize(s));    // T goes out of scope
     }
-    return fs_upload_twiddles(c, s);
+    return TDSE_OK;
 }
 
-// The fixed-point twiddles of every axis (functions of the grid alone).
-tdse_status fs_upload_twiddles(tdse_ctx* c, cudaStream_t s) {
-    const FsState& F = c->F;
+tdse_status fs_bind(tdse_ctx* c, cudaStream_t s) {
+    c->F.g.assign(c->B, 0);
+    TDSE_CK(c, cudaMemsetAsync(c->P<int>(c->F.off.g), 0, (size_t)c->B * sizeof(int), s));
+    return fs_upload_tables(c, s);
+}
+
+// The one-step phase of an axis has modulus at most e^{H |dphi|}; over the
+// history and all axes at most e^{7 H sum |dphi|}.  Its fixed-point factors
+// hold moduli below 2^(1 + g): g of instances [lo, hi) for a field that changes
+// by at most dphi per step (their phase tables are built after this).
+tdse_status fs_field_range(tdse_ctx* c, int lo, int hi, const double* dphi, cudaStream_t s) {
+    FsState& F = c->F;
+    double growth = 0.0;
+    for (int x = 0; x < c->d; ++x) growth += 7.0 * F.ax[x].H * std::fabs(dphi[x]);
+    const int g = std::max(0, (int)std::ceil(std::min(growth / M_LN2, 25.0) - 1.0));
+    for (int b = lo; b < hi; ++b) F.g[b] = g;
+    TDSE_CK(c, cudaMemcpyAsync(c->P<int>(F.off.g) + lo, F.g.data() + lo, (size_t)(hi - lo) * sizeof(int),
+                               cudaMemcpyHostToDevice, s));    // pageable: taken before the call returns
+    return TDSE_OK;
+}
+
+// Largest change of phi per step and axis (the sum of the |changes| of its
+// eighths), phi [d][ntf].
+void fs_largest_dphi(const tdse_ctx* c, const double* phi, double* dphi) {
     for (int x = 0; x < c->d; ++x) {
-        const int M = F.ax[x].M;
-        std::vector<int4> w(M);
-        for (int m = 0; m < M; ++m) {
-            const long double th = -2.0L * kPiL * m / M;
-            fx_limbs(llroundl(cosl(th) * 0x1p61L), w[m].x, w[m].y);
-            fx_limbs(llroundl(sinl(th) * 0x1p61L), w[m].z, w[m].w);
+        const double* p = phi + (size_t)x * c->ntf;
+        for (int m = 0; m + SUB < c->ntf; m += SUB) {
+            double t = 0.0;
+            for (int i = 0; i < SUB; ++i) t += std::fabs(p[m + i + 1] - p[m + i]);
+            dphi[x] = std::fmax(dphi[x], t);
         }
-        TDSE_CK(c, cudaMemcpyAsync(c->P<int4>(F.off.tw[x]), w.data(), w.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-        TDSE_CK(c, cudaStreamSynchronize(s));    // w goes out of scope
     }
+}
+
+// After a checkpoint is loaded: the range of its fields, from its flags (two
+// bytes per instance, g + 1 above bit 0 of the first) or, where they have none,
+// from its phi tables.
+tdse_status fs_loaded_field_range(tdse_ctx* c, const char* flags, cudaStream_t s) {
+    FsState& F = c->F;
+    std::vector<double> phi((size_t)c->d * c->ntf);
+    for (int b = 0; b < c->B; ++b) {
+        const int g = (unsigned char)flags[2 * b] >> 1;
+        double dphi[3] = {0.0, 0.0, 0.0};
+        if (!g) {
+            TDSE_CK(c, cudaMemcpyAsync(phi.data(), c->P<double>(F.off.phi) + (size_t)b * phi.size(), phi.size() * 8,
+                                       cudaMemcpyDeviceToHost, s));
+            TDSE_CK(c, cudaStreamSynchronize(s));
+            fs_largest_dphi(c, phi.data(), dphi);
+        }
+        const tdse_status st = fs_field_range(c, b, b + 1, dphi, s);
+        if (st != TDSE_OK) return st;
+        if (g) F.g[b] = g - 1;
+    }
+    TDSE_CK(c, cudaMemcpyAsync(c->P<int>(F.off.g), F.g.data(), (size_t)c->B * sizeof(int), cudaMemcpyHostToDevice, s));
     return TDSE_OK;
 }
 
@@ -711,12 +822,10 @@ tdse_status fs_build_phase_tables(tdse_ctx* c, int b, cudaStream_t s) {
     const int2* iv = c->P<int2>(F.off.iv);
     for (int x = 0; x < c->d; ++x) {
         const FsAxisHost& A = F.ax[x];
-        double2* P = c->P<double2>(F.off.P[x]) + (size_t)b * c->n_int * A.N;
+        const size_t at = (size_t)b * c->n_int * A.N;
         const double* phi = c->P<double>(F.off.phi) + ((size_t)b * c->d + x) * c->ntf;
-        TDSE_CK(c, launch_fs_phase(P, c->P<double2>(F.off.zeta[x]), A.N, iv, c->n_int, phi, c->cfg.dt, s));
-        if (F.f32)
-            TDSE_CK(c, launch_fs_to_f32(c->P<float2>(F.off.P_f[x]) + (size_t)b * c->n_int * A.N, P,
-                                        (size_t)c->n_int * A.N, s));
+        TDSE_CK(c, launch_fs_phase(c->P<int4>(F.off.P[x]) + at, F.f32 ? c->P<float2>(F.off.P_f[x]) + at : nullptr, F.g[b],
+                                   c->P<double2>(F.off.zeta[x]), A.N, iv, c->n_int, phi, c->cfg.dt, s));
     }
     return TDSE_OK;
 }

@@ -24,7 +24,6 @@
 
 namespace tdse {
 
-constexpr int FS_T = 256;         // threads per CTA of every free-space kernel
 constexpr int FS_MAX_ND = 128;    // dense (Alpert + Gauss) modes per axis
 constexpr int FS_MAX_HIST = 7;
 constexpr int FS_MAX_NT = 64;     // terms of the Chebyshev interpolant of the C-type transforms
@@ -36,14 +35,22 @@ struct FsAxis {
     int NE;       // modes per equispaced block
     int ND;       // dense modes (A1, C, A3)
     int N;        // all modes: 2 NE + ND
-    const double2* preI;   // [2][NE]    inverse, block b: (h / 2pi) e^{-i i h}
-    const double2* postI;  // [2][M][R]  inverse: e^{i zeta0_b x_j} e^{+2 pi i j s / nu}
-    const double2* preF;   // [2][M][R]  forward: (2/M) e^{-i zeta0_b x_j} e^{-2 pi i j s / nu}
-    const double2* postF;  // [2][NE]    forward: e^{+i i h}
-    const double2* Gd;     // [ND][M]    inverse dense: (w_d / 2pi) e^{i zeta_d x_j}
-    const double2* Fd;     // [ND][M]    forward dense: (2/M) e^{-i zeta_d x_j}
+    // FP64 tables: fixed-point factors (fx.cuh), scaled by powers of two to a
+    // modulus in 1/2..1 at their largest: preI by 2^-xI, P by 2^-(1 + g)
+    // (FsArgs::g), the others per grid point by 2^-xj:
+    // xj[0], [1]: preF of block 0, 1; [2]: Fd and Lf; [3], [4]: postI; [5]: Gd and
+    // Li; M entries each.  Grids of M > 256 points: R stands for 2 nu / M in the
+    // tables and the line count.
+    int xI;
+    const int* xj;
+    const int4* preI;   // [2][NE]    inverse, block b: (h / 2pi) e^{-i i h}
+    const int4* postI;  // [2][M][R]  inverse: e^{i zeta0_b x_j} e^{+2 pi i j s / nu}
+    const int4* preF;   // [2][M][R]  forward: (2/M) e^{-i zeta0_b x_j} e^{-2 pi i j s / nu}
+    const int4* postF;  // [2][NE]    forward: e^{+i i h}
+    const int4* Gd;     // [ND][M]    inverse dense: (w_d / 2pi) e^{i zeta_d x_j}
+    const int4* Fd;     // [ND][M]    forward dense: (2/M) e^{-i zeta_d x_j}
     const int4* tw;        // [M]        e^{-2 pi i m / M}, fixed-point factors (fx.cuh)
-    const double2* P;      // [B][n_int][N] one-step phases e^{-i zeta^2 s + i zeta (phi(t1) - phi(t0))}
+    const int4* P;      // [B][n_int][N] one-step phases e^{-i zeta^2 s + i zeta (phi(t1) - phi(t0))}
     // FP32 copies for the FP32-transform variant (TDSE_MIXED), same layouts
     const float2* preI_f;
     const float2* postI_f;
@@ -64,8 +71,8 @@ struct FsAxis {
     int p;                 // Alpert modes per side: the C rows are dd = p .. p + NC - 1
     int NC;                // Gauss (C) modes
     int NT;                // interpolant terms, 0 = C rows by direct sums
-    const double2* Lf;     // [NT][M]  (2/M) lambda_l(x_j)
-    const double2* Li;     // [NT][M]  rho_l(x_j)
+    const int4* Lf;     // [NT][M]  (2/M) lambda_l(x_j)
+    const int4* Li;     // [NT][M]  rho_l(x_j)
     const double* Tc;      // [NC][NT] T_l(tau_k / H)
     const double2* TcW;    // [NT][NC] T_l(tau_k / H) w_k / 2pi
     const float2* Lf_f;
@@ -83,6 +90,8 @@ struct FsArgs {
     int nhist;             // history terms j = 1..nhist
     double h;              // step size
     double mu[FS_MAX_HIST + 1];
+    int2 mu_w[FS_MAX_HIST + 1];   // mu_j / 2 as fixed-point factors
+    const int* g;          // [B] extra powers of two in the scale of P (0 unless the phases' moduli are large)
     int hist_slot[FS_MAX_HIST];   // ring slot of lag j (index j-1)
     int out_slot;          // ring slot receiving the new (Vu)^
     int interval[FS_MAX_HIST];    // interval id of the one-step phase p_i, i = 0..nhist-1
@@ -121,8 +130,6 @@ cudaError_t launch_fs_phys(const FsArgs& a, int from_usrc, int f32, cudaStream_t
 cudaError_t launch_fs_mid(const FsArgs& a, int dir, int f32, cudaStream_t s);
 cudaError_t launch_fs_1d(const FsArgs& a, int mode, int f32, cudaStream_t s);
 cudaError_t launch_fs_f32(const FsArgs& a, int which, int flag, cudaStream_t s);   // freespace_f32.cu
-// FP32 copy of n complex values
-cudaError_t launch_fs_to_f32(float2* dst, const double2* src, size_t n, cudaStream_t s);
 
 // FP64 residual check of the FP32-transform step (free space).  Per instance b
 // (NM modes, ring slot R_n in FP32 at ring + b rstride):
@@ -139,9 +146,9 @@ cudaError_t launch_fs_res_decide(const double* sums, int B, double hm0, double t
 cudaError_t launch_fs_res_apply(const int* flags, int B, size_t NM, size_t NX, double2* uhat, const double2* Wc,
                                 float2* ring, size_t rstride, const double2* R64, double2* u, const double2* u64,
                                 cudaStream_t s);
-// P[iv][m] of one instance and axis: zeta [N] complex, phi_axis [ntf] = that
-// component of phi at t = m dt / 8.
-cudaError_t launch_fs_phase(double2* P, const double2* zeta, int N, const int2* intervals, int n_int,
+// P[iv][m] of one instance and axis (times 2^-(1 + g); and in FP32, unscaled, if
+// Pf): zeta [N] complex, phi_axis [ntf] = that component of phi at t = m dt / 8.
+cudaError_t launch_fs_phase(int4* P, float2* Pf, int g, const double2* zeta, int N, const int2* intervals, int n_int,
                             const double* phi_axis, double dt, cudaStream_t s);
 
 }  // namespace tdse

@@ -76,19 +76,25 @@ FX_HD unsigned long long fx_to_bits(long long v, int X) {
     return sign | (((unsigned long long)(unsigned)e << 52) + (t >> 11) + ((t >> 10) & 1));
 }
 
-// a w 2^K / 2^64 (w in units of 2^-61: K = 3 multiplies by w, K = 3 - log2 R by w / R).
+// a w 2^K / 2^64 (w in units of 2^-61: K = 3 multiplies by w, K = 3 - log2 R by w / R;
+// K may be negative), |a| <= 2^62.5 and the result likewise.
 template <bool CONJ, int K>
 FX_HD longlong2 fx_mul(longlong2 a, int4 w) {
     const int xl = (int)a.x, yl = (int)a.y;
     const int xh = (int)(a.x >> 32) + (int)((unsigned)xl >> 31), yh = (int)(a.y >> 32) + (int)((unsigned)yl >> 31);
     const int sh = CONJ ? -w.z : w.z, sl = CONJ ? -w.w : w.w, nsh = CONJ ? w.z : -w.z, nsl = CONJ ? w.w : -w.w;
-    const long long half = 1ll << (31 - K);
+    const long long half = K < 0 ? 1ll << 31 : 1ll << (31 - K);
     long long re = (long long)xh * w.x + (long long)yh * nsh;
     long long im = (long long)xh * sh + (long long)yh * w.x;
     const long long cr = (long long)xl * w.x + ((long long)yl * nsh + ((long long)xh * w.y + ((long long)yh * nsl + half)));
     const long long ci = (long long)xl * sh + ((long long)yl * w.x + ((long long)xh * sl + ((long long)yh * w.y + half)));
-    re = (long long)((unsigned long long)re << K) + (cr >> (32 - K));
-    im = (long long)((unsigned long long)im << K) + (ci >> (32 - K));
+    if constexpr (K >= 0) {
+        re = (long long)((unsigned long long)re << K) + (cr >> (32 - K));
+        im = (long long)((unsigned long long)im << K) + (ci >> (32 - K));
+    } else {
+        re = (re + (cr >> 32) + (1ll << (-K - 1))) >> -K;
+        im = (im + (ci >> 32) + (1ll << (-K - 1))) >> -K;
+    }
     return make_longlong2(re, im);
 }
 

@@ -236,7 +236,8 @@ __device__ __forceinline__ double2 fx_horner(double2 uh, const double2 (&r)[MAX_
     constexpr int S0 = 59;
     unsigned mr = 0;
 #pragma unroll
-    for (int j = 1; j <= MAX_HIST; ++j) mr = max(mr, fx_hi(r[j - 1]));
+    for (int j = 1; j <= MAX_HIST; ++j)
+        if (j <= nhist) mr = max(mr, fx_hi(r[j - 1]));
     const unsigned mu = fx_hi(uh);
     const int E = fx_exponent(mr);
     longlong2 S = make_longlong2(0, 0);
