@@ -215,6 +215,7 @@ static std::vector<float> cluster_weight_table(const tdse_ctx* c) {
 static KArgs base_args(const tdse_ctx* c) {
     KArgs a{};
     a.B = c->B;
+    a.overlap = 1;
     a.n0 = c->n0;
     a.n1 = c->n1;
     a.tn0 = c->n0;
@@ -877,6 +878,7 @@ static KArgs adams_args(const tdse_ctx* c, int n) {
 static KArgs group_args(const tdse_ctx* c, KArgs a, int lo, int hi) {
     const size_t l = (size_t)lo, NP = c->NP;
     a.B = hi - lo;
+    if (a.B < c->B) a.overlap = 0;         // one of several chains
     a.uhat = static_cast<char*>(a.uhat) + l * NP * 16;
     a.ring = static_cast<char*>(a.ring) + l * a.ring_slots * NP * c->rsz;
     a.aux += l * NP;
@@ -1442,7 +1444,11 @@ static tdse_status member_status(tdse_batch* b, tdse_ctx* c, tdse_status st) {
 // four-step layout: the step's part of the 2D pass chain (adams_chain_2d).
 static cudaError_t four1d_chain_step(const tdse_ctx* c, int n0, int k, int n, cudaStream_t s) {
     const int combo = step_combo(c);
-    auto A = [&](int m) { return group_args(c, adams_args(c, m), 0, c->B); };
+    auto A = [&](int m) {
+        KArgs a = adams_args(c, m);
+        a.overlap = 0;                      // beside the other members' kernels
+        return a;
+    };
     cudaError_t e = cudaSuccess;
     if (n == n0 + 1) e = step_part(c, A(n), combo, PART_COL_BEGIN, s);
     if (e == cudaSuccess) e = step_part(c, A(n), combo, PART_ROW_MID, s);

@@ -27,6 +27,8 @@ constexpr int E1D_NLO = 32;    // 1D absolute kinetic phase: e^{-i k^2 n dt} = K
 
 struct KArgs {
     int mode;
+    int overlap;              // pass kernels: may start while the launch before drains (one chain on the GPU;
+                              // beside other chains its waiting CTAs would take their slots)
     int B;                    // instances in this launch
     int n0, n1;               // launch geometry: lines x line length (n1 = 1 for 1D); for 3D the
                               // column pass sees [n0][n1 n2] and the row pass [n0 n1][n2]
