@@ -169,6 +169,9 @@ static void plan_workspace(tdse_ctx* c) {
     c->off.scratch = take(256);
     c->off.end = o;
     c->ws_ckpt = o;
+    // not part of a checkpoint: the weight table of 1D mixed runs
+    if (c->d == 1 && c->mixed && !c->four1d && run1d32_supported(c->n0))
+        c->off.run_tab = take(((size_t)c->cfg.nsteps + 1) * CL_TAB * sizeof(float));
     c->ws_need = o;
 }
 
@@ -189,10 +192,10 @@ static void zinv(const tdse_ctx* c, int m, double w, float* hi, float* lo) {
     split(-w * zy / n2, hi[1], lo[1]);
 }
 
-// The same weights for every step m, as rows of the cluster kernel's table
-// (layout in kargs.h); lags before step 0 are zero (never used: Adams steps
+// The same weights for every step m, as rows of a table (cluster kernel, 1D
+// runs; layout in kargs.h); lags before step 0 are zero (never used: Adams steps
 // start after the start-up).
-static std::vector<float> cluster_weight_table(const tdse_ctx* c) {
+static std::vector<float> weight_table(const tdse_ctx* c) {
     std::vector<float> t(((size_t)c->cfg.nsteps + 1) * CL_TAB, 0.0f);
     for (int m = 0; m <= c->cfg.nsteps; ++m) {
         float* r = t.data() + (size_t)m * CL_TAB;
@@ -504,8 +507,14 @@ tdse_status tdse_bind_workspace(tdse_ctx* c, void* dev, size_t bytes, void* stre
         TDSE_CK(c, launch_k1d(c->P<float2>(c->off.k1lo), c->P<float2>(c->off.k1hi), c->nhi, c->n0, c->cfg.dt, s));
     TDSE_CK(c, cudaMemsetAsync(c->P<int>(c->off.err), 0, sizeof(int), s));
     c->cl_ok = false;
+    if (c->off.run_tab) {
+        const std::vector<float> tab = weight_table(c);
+        TDSE_CK(c, cudaMemcpyAsync(c->P<float>(c->off.run_tab), tab.data(), tab.size() * sizeof(float),
+                                   cudaMemcpyHostToDevice, s));
+        TDSE_CK(c, cudaStreamSynchronize(s));      // the host table is freed on return
+    }
     if (c->off.cl_tab) {
-        const std::vector<float> tab = cluster_weight_table(c);
+        const std::vector<float> tab = weight_table(c);
         TDSE_CK(c, cudaMemcpyAsync(c->P<float>(c->off.cl_tab), tab.data(), tab.size() * sizeof(float),
                                    cudaMemcpyHostToDevice, s));
         TDSE_CK(c, cudaStreamSynchronize(s));      // the host table is freed on return
@@ -778,7 +787,28 @@ static tdse_status startup_step(tdse_ctx* c, int n, cudaStream_t s) {
     char* chain_u = c->P<char>(c->off.chain_uhat);
     char* chain_r = c->P<char>(c->off.chain_ring);
     const double half[2] = {0.5, 0.5};
-    for (int ch = 0; ch < c->L; ++ch) {
+    const bool one_launch = c->off.run_tab != 0;        // 1D mixed: every chain in one launch
+    if (one_launch) {
+        KArgs a = base_args(c);
+        Start1DArgs g{};
+        g.L = c->L;
+        g.slot = slot_of(c, n - 1);
+        g.interval0 = startup_interval(c, n, 0, 0);
+        g.tf0 = SUB * (n - 1);
+        g.vtable = c->vtable ? 1 : 0;
+        g.chains = reinterpret_cast<float4*>(chain_u);
+        for (int ch = 0; ch < c->L; ++ch) {
+            KArgs w{};
+            set_weights(w, c->cfg.dt / (double)(1 << ch), half, 2);
+            g.hmu0[ch] = w.h * w.mu[0];
+            g.h_hi[ch] = w.h_hi;
+            g.h_lo[ch] = w.h_lo;
+            g.hmu0_hi[ch] = w.hmu0_hi;
+            g.hmu0_lo[ch] = w.hmu0_lo;
+        }
+        TDSE_CK(c, launch_start1d32(a, g, s));
+    }
+    for (int ch = 0; ch < c->L && !one_launch; ++ch) {
         void* cu = chain_u + (size_t)ch * NPB * 16;
         void* cr = chain_r + (size_t)ch * NPB * c->rsz;
         TDSE_CK(c, cudaMemcpyAsync(cu, c->P<void>(c->off.uhat), NPB * 16, cudaMemcpyDeviceToDevice, s));
@@ -899,6 +929,22 @@ static KArgs group_args(const tdse_ctx* c, KArgs a, int lo, int hi) {
 
 static tdse_status adams_chain_2d(tdse_ctx* c, int n0, int k, int lo, int hi, cudaStream_t s);
 
+// 1D mixed Adams steps of a context run in one launch: one CTA per instance in
+// the default launch shape (the alternative one keeps a launch per step).
+static bool use_run1d32(const tdse_ctx* c) { return c->off.run_tab && c->shape1d == 0; }
+static cudaError_t run1d32(const tdse_ctx* c, int n_first, int k, cudaStream_t s) {
+    KArgs a = base_args(c);
+    set_weights(a, c->cfg.dt, c->mu, c->m);
+    Run1DArgs g{};
+    g.n_first = n_first;
+    g.k = k;
+    g.order = c->m;
+    g.S = c->S;
+    g.S_eff = c->S_eff;
+    g.vtable = c->vtable ? 1 : 0;
+    return launch_run1d32(a, g, c->P<float>(c->off.run_tab), s);
+}
+
 // k consecutive Adams steps n0+1 .. n0+k.  2D runs them as col_begin,
 // (row_mid, col_fused) x (k-1), row_mid, col_end; with step groups, one such
 // chain per group of instances on parallel streams.
@@ -916,6 +962,10 @@ static tdse_status adams_steps(tdse_ctx* c, int n0, int k, cudaStream_t s) {
         ca.tab = c->P<float>(c->off.cl_tab);
         ca.err = c->P<int>(c->off.err);
         TDSE_CK(c, launch_step2d_cluster(a, ca, c->cl, s));
+        return TDSE_OK;
+    }
+    if (use_run1d32(c)) {
+        TDSE_CK(c, run1d32(c, n0 + 1, k, s));
         return TDSE_OK;
     }
     if ((c->d == 1 && !c->four1d) || k == 1) {
@@ -1429,6 +1479,7 @@ static tdse_status batch_prepare(tdse_batch* b) {
     for (tdse_ctx* c : b->m) {
         if (c->four1d) continue;            // the 2D pass kernels set their attributes at first launch
         if (e == cudaSuccess) e = periodic1d_prepare(c->n0, COMBO_F32);
+        if (e == cudaSuccess && c->off.run_tab) e = run1d32_prepare(c->n0);
         if (e == cudaSuccess && !c->off.tw128) e = periodic1d_prepare(c->n0, COMBO_F64_R32);
     }
     if (e != cudaSuccess) return b->fail(TDSE_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
@@ -1495,9 +1546,11 @@ static tdse_status batch_adams(tdse_batch* b, int n0, int k, int grid, cudaStrea
 static tdse_status batch_adams_streams(tdse_batch* b, int n0, int k, cudaStream_t s) {
     cudaError_t e = cudaEventRecord(b->fork, s);
     for (size_t g = 0; g < b->m.size() && e == cudaSuccess; ++g) e = cudaStreamWaitEvent(b->streams[g], b->fork, 0);
+    for (size_t g = 0; g < b->m.size() && e == cudaSuccess; ++g)
+        if (use_run1d32(b->m[g])) e = run1d32(b->m[g], n0 + 1, k, b->streams[g]);
     for (int n = n0 + 1; n <= n0 + k && e == cudaSuccess; ++n)
         for (size_t g = 0; g < b->m.size() && e == cudaSuccess; ++g)
-            e = b->m[g]->four1d ? four1d_chain_step(b->m[g], n0, k, n, b->streams[g])
+            if (!use_run1d32(b->m[g])) e = b->m[g]->four1d ? four1d_chain_step(b->m[g], n0, k, n, b->streams[g])
                                 : run(b->m[g], adams_args(b->m[g], n), step_combo(b->m[g]), b->streams[g]);
     for (size_t g = 0; g < b->m.size(); ++g) {   // always join, so that a capture can end
         cudaError_t j = cudaEventRecord(b->join[g], b->streams[g]);
@@ -1509,41 +1562,50 @@ static tdse_status batch_adams_streams(tdse_batch* b, int n0, int k, cudaStream_
     return TDSE_OK;
 }
 
+// Start of the members (initial transforms, start-up steps, change of frame) up
+// to `steps` steps from where they are, each on its own stream: forked from and
+// joined to s.  One after another on one stream the members' small launches
+// left the GPU mostly idle: 512 members of 256..16384 points, 200 steps, 44.7 ->
+// 33.2 ms with the chains of run1d32.cu.
+static tdse_status batch_start(tdse_batch* b, int steps, cudaStream_t s) {
+    const int from = b->m[0]->step, S = b->m[0]->S;
+    const int to = std::min(from + steps, S);
+    bool work = false;
+    for (tdse_ctx* c : b->m) work = work || !c->inited || from < to || (from + steps > S && !c->ip);
+    if (!work) return TDSE_OK;
+    cudaError_t e = cudaEventRecord(b->fork, s);
+    for (size_t g = 0; g < b->m.size() && e == cudaSuccess; ++g) e = cudaStreamWaitEvent(b->streams[g], b->fork, 0);
+    tdse_status st = TDSE_OK;
+    auto each = [&](auto f) {
+        for (size_t g = 0; g < b->m.size() && e == cudaSuccess && st == TDSE_OK; ++g)
+            st = member_status(b, b->m[g], f(b->m[g], b->streams[g]));
+    };
+    each([&](tdse_ctx* c, cudaStream_t q) { return c->inited ? TDSE_OK : do_init(c, q); });
+    for (int n = from + 1; n <= to; ++n)
+        each([&](tdse_ctx* c, cudaStream_t q) {
+            const tdse_status r = startup_step(c, n, q);
+            if (r == TDSE_OK) c->step = n;
+            return r;
+        });
+    if (from + steps > S)
+        each([&](tdse_ctx* c, cudaStream_t q) { return c->ip ? TDSE_OK : enter_interaction(c, c->step, q); });
+    for (size_t g = 0; g < b->m.size(); ++g) {   // always join, so that a capture can end
+        cudaError_t j = cudaEventRecord(b->join[g], b->streams[g]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, b->join[g], 0);
+        if (e == cudaSuccess) e = j;
+    }
+    if (st != TDSE_OK) return st;
+    return e == cudaSuccess ? TDSE_OK : b->fail(TDSE_ECUDA, std::string("member start: ") + cudaGetErrorString(e));
+}
+
 // The launch sequence of nsteps steps (no capture logic).
 static tdse_status batch_run(tdse_batch* b, int nsteps, cudaStream_t s) {
-    for (tdse_ctx* c : b->m)
-        if (!c->inited) {
-            tdse_status st = member_status(b, c, do_init(c, s));
-            if (st != TDSE_OK) return st;
-        }
-    int k = 0;
-    while (k < nsteps) {
-        const int n = b->m[0]->step + 1;
-        if (n <= b->m[0]->S) {
-            for (tdse_ctx* c : b->m) {
-                tdse_status st = member_status(b, c, startup_step(c, n, s));
-                if (st != TDSE_OK) return st;
-                c->step = n;
-            }
-            ++k;
-            continue;
-        }
-        for (tdse_ctx* c : b->m)
-            if (!c->ip) {
-                tdse_status st = member_status(b, c, enter_interaction(c, c->step, s));
-                if (st != TDSE_OK) return st;
-            }
-        if (b->mode == 1) {
-            tdse_status st = batch_adams_streams(b, n - 1, nsteps - k, s);
-            if (st != TDSE_OK) return st;
-            k = nsteps;
-            continue;
-        }
-        tdse_status st = batch_adams(b, n - 1, nsteps - k, b->grid, s);
-        if (st != TDSE_OK) return st;
-        k = nsteps;
-    }
-    return TDSE_OK;
+    const int from = b->m[0]->step;
+    const tdse_status st = batch_start(b, nsteps, s);
+    if (st != TDSE_OK) return st;
+    const int n = b->m[0]->step, k = from + nsteps - n;
+    if (k <= 0) return TDSE_OK;
+    return b->mode == 1 ? batch_adams_streams(b, n, k, s) : batch_adams(b, n, k, b->grid, s);
 }
 
 static tdse_status batch_check(tdse_batch* b, int nsteps) {
@@ -1803,19 +1865,23 @@ tdse_status tdse_batch_tune(tdse_batch* b, int trial_steps, void* stream) {
     // the members' own kernels on parallel streams against the best fused launch
     b->mode = 0;
     if (st == TDSE_OK && b->m.size() >= 1) {
+        // (runs of several steps where there are as many: a member's run loads its
+        // state and history once)
+        const int run_len = std::min(16, b->m[0]->cfg.nsteps - (n - 1));
         auto timed_streams = [&](float& ms) -> tdse_status {
-            tdse_status r = batch_adams_streams(b, n - 1, 1, s);
+            tdse_status r = batch_adams_streams(b, n - 1, run_len, s);
             for (tdse_ctx* c : b->m) c->step = n - 1;
             if (r != TDSE_OK) return r;
             cudaEventRecord(e0, s);
             for (int i = 0; i < trial_steps && r == TDSE_OK; ++i) {
-                r = batch_adams_streams(b, n - 1, 1, s);
+                r = batch_adams_streams(b, n - 1, run_len, s);
                 for (tdse_ctx* c : b->m) c->step = n - 1;
             }
             if (r != TDSE_OK) return r;
             cudaEventRecord(e1, s);
             if (cudaEventSynchronize(e1) != cudaSuccess) return b->fail(TDSE_ECUDA, "event sync");
             cudaEventElapsedTime(&ms, e0, e1);
+            ms /= (float)run_len;
             return TDSE_OK;
         };
         float ms = 0;

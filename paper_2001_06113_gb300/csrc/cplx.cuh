@@ -195,6 +195,9 @@ struct FftShape {
     }
 };
 
+// Buffer elements of a single padded line of N points (FP64: not padded).
+template <class C> constexpr int fft_len(int n) { return sizeof(C) == 8 ? n + n / 16 : n; }
+
 template <class C, int N, int L, int PS, int T, bool INV>
 struct Fft : FftShape<N, L, T, INV> {
     using Shape = FftShape<N, L, T, INV>;
@@ -207,6 +210,14 @@ struct Fft : FftShape<N, L, T, INV> {
     using Shape::PL;
     using Shape::RF;
     using Shape::RL;
+
+    // Element (pos, line) of the buffer.  A single line is padded by one element
+    // in 16: without it the stride-8 stores of the first pass meet in two of
+    // 16 banks (192 -> 72 shared-memory cycles per butterfly of a 512-point
+    // line); fft_len(N) elements in all.
+    __device__ static __forceinline__ int at(int pos, int line) {
+        return L == 1 && PS == 1 ? pos + (pos >> 4) : pos * PS + line;
+    }
 
     template <int S, class Sync>
     __device__ static __forceinline__ void mid_pass(C* buf, const C* __restrict__ tw, const C* __restrict__ twl,
@@ -221,7 +232,7 @@ struct Fft : FftShape<N, L, T, INV> {
             int j, line;
             if (item(p, NB, j, line, tid)) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[p][r] = buf[(j + r * NB) * PS + line];
+                for (int r = 0; r < R; ++r) v[p][r] = buf[at(j + r * NB, line)];
             }
         }
         sync();
@@ -236,7 +247,7 @@ struct Fft : FftShape<N, L, T, INV> {
                 dft_r<R, INV>(v[p]);
                 const int base = (j - k) * R + k;
 #pragma unroll
-                for (int r = 0; r < R; ++r) buf[(base + r * Ns) * PS + line] = v[p][r];
+                for (int r = 0; r < R; ++r) buf[at(base + r * Ns, line)] = v[p][r];
             }
         }
         sync();
@@ -272,7 +283,7 @@ struct Fft : FftShape<N, L, T, INV> {
                 if (item(p, NBF, j, line, tid)) {
                     dft_r<RF, INV>(in[p]);
 #pragma unroll
-                    for (int r = 0; r < RF; ++r) buf[(j * RF + r) * PS + line] = in[p][r];
+                    for (int r = 0; r < RF; ++r) buf[at(j * RF + r, line)] = in[p][r];
                 }
             }
             sync();
@@ -282,7 +293,7 @@ struct Fft : FftShape<N, L, T, INV> {
                 int j, line;
                 if (item(p, NBL, j, line, tid)) {
 #pragma unroll
-                    for (int r = 0; r < RL; ++r) out[p][r] = buf[(j + r * NBL) * PS + line];
+                    for (int r = 0; r < RL; ++r) out[p][r] = buf[at(j + r * NBL, line)];
 #pragma unroll
                     for (int r = 1; r < RL; ++r) out[p][r] = twiddle<INV>(out[p][r], tw, twl, j * r);
                     dft_r<RL, INV>(out[p]);
@@ -301,7 +312,7 @@ struct Fft : FftShape<N, L, T, INV> {
         if (item(p, NBF, j, line, tid)) {
             dft_r<RF, INV>(v);
 #pragma unroll
-            for (int r = 0; r < RF; ++r) buf[(j * RF + r) * PS + line] = v[r];
+            for (int r = 0; r < RF; ++r) buf[at(j * RF + r, line)] = v[r];
         }
     }
     template <class Sync>
@@ -315,7 +326,7 @@ struct Fft : FftShape<N, L, T, INV> {
         int line;
         if (!item(p, NBL, j, line, tid)) return false;
 #pragma unroll
-        for (int r = 0; r < RL; ++r) v[r] = buf[(j + r * NBL) * PS + line];
+        for (int r = 0; r < RL; ++r) v[r] = buf[at(j + r * NBL, line)];
 #pragma unroll
         for (int r = 1; r < RL; ++r) v[r] = twiddle<INV>(v[r], tw, twl, j * r);
         dft_r<RL, INV>(v);

@@ -142,6 +142,23 @@ struct Run1DArgs {
     double rich[4];           // Richardson coefficients of the chains
     int2 half_w[2];           // the trapezoidal weights, as KArgs::mu_w
 };
+// Mixed-precision Adams steps n_first .. n_first + k - 1 > S in the interaction
+// picture, likewise (run1d32.cu), weights from rows of a weight table
+// (CL_TAB floats per step, layout below).
+// Richardson chains 0 .. L - 1 of one mixed start-up step (lab frame) from the
+// state and ring slot `slot` to chains [L][B][N].
+struct Start1DArgs {
+    int L, slot;
+    int interval0, tf0;       // first phase interval and fine time index of the step
+    int vtable;
+    float4* chains;
+    double hmu0[4];           // h mu_0 of the chains (h = dt / 2^c, mu_0 = 1/2), and h, h mu_0 as hi + lo
+    float h_hi[4], h_lo[4], hmu0_hi[4], hmu0_lo[4];
+};
+cudaError_t launch_start1d32(const KArgs& a, const Start1DArgs& g, cudaStream_t s);
+bool run1d32_supported(int n);
+cudaError_t run1d32_prepare(int n);
+cudaError_t launch_run1d32(const KArgs& a, const Run1DArgs& g, const float* wtab, cudaStream_t s);
 bool run1d64_supported(int n);
 cudaError_t launch_run1d64(const KArgs& a, const Run1DArgs& g, cudaStream_t s);
 

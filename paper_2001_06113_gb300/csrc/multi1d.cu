@@ -23,7 +23,7 @@ template <int N, int T>
 __device__ __noinline__ void run_group(const KArgs& a, int b0, int count, float2* smem) {
     const int g = threadIdx.x / T, tid = threadIdx.x % T;
     if (g >= count) return;
-    float2* buf = smem + (size_t)g * N;
+    float2* buf = smem + (size_t)g * fft_len<float2>(N);
     if constexpr (T == MULTI_CTA)
         step1d<float2, float2, N, T>(a, b0, tid, CtaSync{}, buf);
     else if constexpr (T == 32)
@@ -74,7 +74,9 @@ int multi_variant(int n, int t) {
         if (kVariants[v].n == n && kVariants[v].t == t) return v;
     return -1;
 }
-size_t multi_item_smem(int var, int count) { return (size_t)count * multi_variant_n(var) * sizeof(float2); }
+size_t multi_item_smem(int var, int count) {
+    return (size_t)count * fft_len<float2>(multi_variant_n(var)) * sizeof(float2);
+}
 
 int multi_occupancy(size_t smem) {
     int nb = 0;

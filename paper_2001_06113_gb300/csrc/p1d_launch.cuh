@@ -51,7 +51,7 @@ template <class C, class RT, int N, int T = threads_1d(N)>
 static cudaError_t prepare_n() {
     static bool configured = false;
     if (configured) return cudaSuccess;
-    const size_t smem = (size_t)N * sizeof(C);
+    const size_t smem = (size_t)fft_len<C>(N) * sizeof(C);
     cudaError_t e = cudaFuncSetAttribute(k_periodic1d<C, RT, N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e == cudaSuccess)
@@ -63,7 +63,7 @@ static cudaError_t prepare_n() {
 
 template <class C, class RT, int N, int T = threads_1d(N)>
 static cudaError_t launch_n(const KArgs& a, cudaStream_t s) {
-    const size_t smem = (size_t)N * sizeof(C);
+    const size_t smem = (size_t)fft_len<C>(N) * sizeof(C);
     cudaError_t e = prepare_n<C, RT, N, T>();
     if (e != cudaSuccess) return e;
     k_periodic1d<C, RT, N, T><<<a.B, T, smem, s>>>(a);

@@ -217,6 +217,23 @@ __device__ __forceinline__ float4 ip_update(const KArgs& a, float4 X, float2 q) 
     return ffc_add_f(X, py, -px);
 }
 
+// The same with the weights of step m as a row of a weight table (layout in
+// kargs.h): c_j of one lag added to S, and the update.
+__device__ __forceinline__ float2 ip_add_lag(const float4 c, float2 q, float2 S) {
+    S.x = fmaf(c.z, q.x, fmaf(-c.w, q.y, S.x));
+    S.y = fmaf(c.z, q.y, fmaf(c.w, q.x, S.y));
+    S.x = fmaf(c.x, q.x, fmaf(-c.y, q.y, S.x));
+    S.y = fmaf(c.x, q.y, fmaf(c.y, q.x, S.y));
+    return S;
+}
+__device__ __forceinline__ float4 ip_update(const float4 d, float4 X, float2 q) {
+    float px = fmaf(d.z, q.x, -d.w * q.y);
+    float py = fmaf(d.z, q.y, d.w * q.x);
+    px = fmaf(d.x, q.x, fmaf(-d.y, q.y, px));
+    py = fmaf(d.x, q.y, fmaf(d.y, q.x, py));
+    return ffc_add_f(X, py, -px);
+}
+
 // X = st - i h S (mixed, double-float, real weights: lab-frame start-up)
 __device__ __forceinline__ float4 mixed_X(const KArgs& a, float4 st, const float2* __restrict__ ringb, size_t NP,
                                           size_t idx) {
