@@ -865,7 +865,7 @@ static tdse_status enter_interaction(tdse_ctx* c, int n, cudaStream_t s) {
         zs[2 * q + 1] = j >= 0 ? c->zdither[2 * j + 1] : 0.f;
     }
     KArgs a = base_args(c);
-    TDSE_CK(c, launch_to_interaction(a, n, steps, zs, c->RS < 8 ? c->RS : 8, s));
+    TDSE_CK(c, launch_to_interaction(a, n, steps, zs, c->RS < 8 ? c->RS : 8, c->P<void>(c->off.chain_uhat), s));
     c->ip = true;
     return TDSE_OK;
 }

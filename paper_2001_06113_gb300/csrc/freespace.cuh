@@ -545,25 +545,10 @@ __device__ __forceinline__ longlong2 pmul(longlong2 v, int4 p, int g) {
 }
 __device__ __forceinline__ int4 pmul(int4 a, int4 b, int g) { return fx_as_factor(pmul(fx_value(a), b, g)); }
 
-// FP64 bits -> FP32, rounded to nearest (ties away), in integer arithmetic.
-__device__ __forceinline__ float fx_to_float(double v) {
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const int e = (int)((hi >> 20) & 0x7ff) - 896;
-    unsigned f = ((unsigned)e << 23 | (hi & 0xfffffu) << 3 | lo >> 29) + ((lo >> 28) & 1);
-    if (e <= 0) f = 0;
-    if (e >= 255) f = 0x7f800000u + (e == 1151 && ((hi & 0xfffffu) | lo) ? 0x400000u : 0);
-    return __uint_as_float(f | (hi & 0x80000000u));
-}
 __device__ __forceinline__ float2 to_c(double2 v, float2) { return make_float2(fx_to_float(v.x), fx_to_float(v.y)); }
 __device__ __forceinline__ double2 to_c(double2 v, double2) { return v; }
 
-// FP32 value as FP64 bits (subnormals become 0), in integer arithmetic.
-__device__ __forceinline__ double widen(float x) {
-    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xff;
-    const unsigned hi = e == 0 ? 0u : ((b & 0x7fffffffu) >> 3) + (e == 255 ? 0x70000000u : 0x38000000u);
-    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(e == 0 ? 0u : b << 29));
-}
-__device__ __forceinline__ double2 widen(float2 x) { return make_double2(widen(x.x), widen(x.y)); }
+__device__ __forceinline__ double2 widen(float2 x) { return make_double2(fx_widen(x.x), fx_widen(x.y)); }
 __device__ __forceinline__ double2 widen(double2 x) { return x; }
 // v * (-i c) added to u
 __device__ __forceinline__ double2 add_minus_i(double2 u, double c, double2 v) {

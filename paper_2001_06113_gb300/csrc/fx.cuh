@@ -167,6 +167,21 @@ __device__ __forceinline__ double2 fx_factor_to_d(int4 w) {
     const double u = 1.0 / 536870912.0, l = 1.0 / 2305843009213693952.0;
     return make_double2(fma((double)w.y, l, (double)w.x * u), fma((double)w.w, l, (double)w.z * u));
 }
+// FP64 bits -> FP32, rounded to nearest (ties away), in integer arithmetic.
+__device__ __forceinline__ float fx_to_float(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const int e = (int)((hi >> 20) & 0x7ff) - 896;
+    unsigned f = ((unsigned)e << 23 | (hi & 0xfffffu) << 3 | lo >> 29) + ((lo >> 28) & 1);
+    if (e <= 0) f = 0;
+    if (e >= 255) f = 0x7f800000u + (e == 1151 && ((hi & 0xfffffu) | lo) ? 0x400000u : 0);
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+// FP32 value as FP64 bits (subnormals become 0), in integer arithmetic.
+__device__ __forceinline__ double fx_widen(float x) {
+    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xff;
+    const unsigned hi = e == 0 ? 0u : ((b & 0x7fffffffu) >> 3) + (e == 255 ? 0x70000000u : 0x38000000u);
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(e == 0 ? 0u : b << 29));
+}
 // Largest value of v over the T threads of a CTA (all of them call it).
 template <int T>
 __device__ __forceinline__ unsigned fx_cta_max(unsigned v) {

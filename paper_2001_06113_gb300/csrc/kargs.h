@@ -265,7 +265,8 @@ cudaError_t launch_copy_slot(void* dst, const void* ring, int ring_slots, int sl
 cudaError_t launch_count_nonfinite(const void* x, size_t nwords, bool ff, int* count, cudaStream_t s);
 // Convert the double-float state at step n and the ring slots of steps
 // slot_steps[0..nslots) to the interaction picture (divide by E in FP64).
+// scratch: at least 9 rows of tn0 + tn1 + tn2 16-byte factors per instance (2D, 3D).
 cudaError_t launch_to_interaction(const KArgs& a, int n, const int* slot_steps, const float* slot_z, int nslots,
-                                  cudaStream_t s);
+                                  void* scratch, cudaStream_t s);
 
 }  // namespace tdse

@@ -161,6 +161,30 @@ __global__ void k_split_float(float2* hilo, const double* src, size_t n) {
 
 struct Coef4 { double c[4]; };
 
+// Double-float states: FP64 sums of products with the FP32 parts (4 fused
+// multiply-adds per chain instead of conversions and sums of each pair: the
+// FP64 pipe bounds it; 5 x 128^3: 0.76 -> 0.37 ms).
+__global__ void k_combine_ff(float4* state, const float4* chains, size_t stride, int L, Coef4 co, size_t n) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        float4 v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c < L) v[c] = chains[c * stride + i];
+        double re = 0.0, im = 0.0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (c < L) {
+                re = fma(co.c[c], fx_widen(v[c].x), re);
+                im = fma(co.c[c], fx_widen(v[c].y), im);
+                re = fma(co.c[c], fx_widen(v[c].z), re);
+                im = fma(co.c[c], fx_widen(v[c].w), im);
+            }
+        }
+        const float rh = fx_to_float(re), ih = fx_to_float(im);
+        state[i] = make_float4(rh, ih, fx_to_float(re - fx_widen(rh)), fx_to_float(im - fx_widen(ih)));
+    }
+}
+
 template <class ST>
 __global__ void k_combine(ST* state, const ST* chains, size_t stride, int L, Coef4 co, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -199,34 +223,86 @@ __global__ void k_count_nonfinite(const double* x, size_t nwords, bool ff, int* 
 struct Steps8 { int s[8]; float z[8][2]; };
 
 // state (double-float, lab frame at step n) -> v^ = conj(E_n) u^, and ring slot
-// q (FP32, lab frame at step steps.s[q]) -> r~ = z_q conj(E) R; E in FP64.
-__global__ void k_to_interaction(float4* state, float2* ring, int ring_slots, const double* phi, int ntf, int d,
-                                 int n0, int n1, int n2, double dt, int n, Steps8 steps, int nslots) {
+// q (FP32, lab frame at step steps.s[q]) -> r~ = z_q conj(E) R; E in FP64.  1D.
+__global__ void k_to_interaction(float4* state, float2* ring, int ring_slots, const double* phi, int ntf, int n0, double dt,
+                                 int n, Steps8 steps, int nslots) {
     const int b = blockIdx.y;
-    const size_t NP = (size_t)n0 * n1 * n2;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < NP; idx += (size_t)gridDim.x * blockDim.x) {
-        const int m0 = (int)(idx / ((size_t)n1 * n2));
-        const int rem = (int)(idx - (size_t)m0 * n1 * n2);
-        const int m1 = rem / n2, m2 = rem - (rem / n2) * n2;
-        const double k0 = kmode(m0, n0), k1 = d >= 2 ? kmode(m1, n1) : 0.0, k2 = d == 3 ? kmode(m2, n2) : 0.0;
-        const double* ph = phi + (size_t)b * d * ntf;
+    const double* ph = phi + (size_t)b * ntf;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n0; idx += gridDim.x * blockDim.x) {
+        const double k = kmode(idx, n0);
         auto E = [&](int step) {
-            double arg = d == 3 ? -(k0 * k0 + k1 * k1 + k2 * k2) * ((double)step * dt) + k0 * ph[8 * (size_t)step]
-                                : -(k0 * k0 + k1 * k1) * ((double)step * dt) + k0 * ph[8 * (size_t)step];
-            if (d >= 2) arg += k1 * ph[ntf + 8 * (size_t)step];
-            if (d == 3) arg += k2 * ph[2 * (size_t)ntf + 8 * (size_t)step];
             double s, c;
-            sincos(arg, &s, &c);
+            sincos(-(k * k) * ((double)step * dt) + k * ph[8 * (size_t)step], &s, &c);
             return make_double2(c, -s);     // conj(E)
         };
-        float4* sv = state + (size_t)b * NP + idx;
+        float4* sv = state + (size_t)b * n0 + idx;
         *sv = d_to_ffc(cmul(E(n), ffc_to_d(*sv)));
         for (int q = 0; q < nslots; ++q) {
             if (steps.s[q] < 0) continue;
-            float2* r = ring + ((size_t)b * ring_slots + q) * NP + idx;
+            float2* r = ring + ((size_t)b * ring_slots + q) * n0 + idx;
             const double2 zq = make_double2(steps.z[q][0], steps.z[q][1]);
             const double2 v = cmul(zq, cmul(E(steps.s[q]), make_double2(r->x, r->y)));
             *r = make_float2((float)v.x, (float)v.y);
+        }
+    }
+}
+
+// The same in 2D and 3D, where conj(E) is a product of one factor per axis.
+// Factors of the steps to convert: tab[b][q][n0 + n1 (+ n2)], q = 0 the state's
+// step in FP64, q = 1 + slot the ring's in double-float with the ring dither on
+// axis 0 (exact phases per mode instead took 10.9 ms of FP64 sines for 64 x
+// 512^2, 7.0 ms for 5 x 128^3).
+__global__ void k_interaction_tables(double2* tab, const double* phi, int ntf, int n0, int n1, int n2, double dt, int n,
+                                     Steps8 steps, int nslots) {
+    const int q = blockIdx.x, b = blockIdx.y, d = n2 > 0 ? 3 : 2, len = n0 + n1 + n2;
+    const int step = q == 0 ? n : steps.s[q - 1];
+    if (step < 0) return;
+    const double* ph = phi + (size_t)b * d * ntf;
+    double2* row = tab + ((size_t)b * (nslots + 1) + q) * len;
+    for (int j = threadIdx.x; j < len; j += blockDim.x) {
+        const int ax = j < n0 ? 0 : (j < n0 + n1 ? 1 : 2);
+        const double k = kmode(ax == 0 ? j : (ax == 1 ? j - n0 : j - n0 - n1), ax == 0 ? n0 : (ax == 1 ? n1 : n2));
+        double s, c;
+        sincos(-(k * k) * ((double)step * dt) + k * ph[(size_t)ax * ntf + 8 * (size_t)step], &s, &c);
+        double2 e = make_double2(c, -s);        // conj(E)
+        if (q > 0) {
+            if (ax == 0) e = cmul(make_double2(steps.z[q - 1][0], steps.z[q - 1][1]), e);
+            *reinterpret_cast<float4*>(&row[j]) = d_to_ffc(e);
+        } else {
+            row[j] = e;
+        }
+    }
+}
+
+__global__ void k_to_interaction_sep(float4* state, float2* ring, int ring_slots, const double2* tab, int n0, int n1, int n2,
+                                     Steps8 steps, int nslots) {
+    const int b = blockIdx.y, len = n0 + n1 + n2;
+    const int inner = n2 > 0 ? n1 * n2 : n1;
+    const size_t NP = (size_t)n0 * inner;
+    const double2* t0 = tab + (size_t)b * (nslots + 1) * len;
+    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < NP; idx += (size_t)gridDim.x * blockDim.x) {
+        const int m0 = (int)(idx / inner), rem = (int)(idx - (size_t)m0 * inner);
+        const int m1 = n2 > 0 ? rem / n2 : rem, m2 = n2 > 0 ? rem - m1 * n2 : 0;
+        float2 r[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q < nslots && steps.s[q] >= 0) r[q] = ring[((size_t)b * ring_slots + q) * NP + idx];
+        float4* sv = state + (size_t)b * NP + idx;
+        const float4 x = *sv;
+        double2 e = cmul(__ldg(&t0[m0]), __ldg(&t0[n0 + m1]));
+        if (n2 > 0) e = cmul(e, __ldg(&t0[n0 + n1 + m2]));
+        const double2 v = cmul(e, make_double2(fx_widen(x.x) + fx_widen(x.z), fx_widen(x.y) + fx_widen(x.w)));
+        const float vh = fx_to_float(v.x), wh = fx_to_float(v.y);
+        *sv = make_float4(vh, wh, fx_to_float(v.x - fx_widen(vh)), fx_to_float(v.y - fx_widen(wh)));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            if (q < nslots && steps.s[q] >= 0) {
+                const float4* t = reinterpret_cast<const float4*>(t0 + (size_t)(q + 1) * len);
+                float4 w = ffc_mul(__ldg(&t[m0]), __ldg(&t[n0 + m1]));
+                if (n2 > 0) w = ffc_mul(w, __ldg(&t[n0 + n1 + m2]));
+                const float4 p = ffc_mul(w, make_float4(r[q].x, r[q].y, 0.f, 0.f));
+                ring[((size_t)b * ring_slots + q) * NP + idx] = make_float2(p.x, p.y);
+            }
         }
     }
 }
@@ -353,8 +429,7 @@ cudaError_t launch_combine(void* state, const void* chains, size_t chain_stride,
     Coef4 co{};
     for (int c = 0; c < L && c < 4; ++c) co.c[c] = coef[c];
     if (ff)
-        k_combine<float4><<<grid_for(n, 256), 256, 0, s>>>((float4*)state, (const float4*)chains, chain_stride, L,
-                                                              co, n);
+        k_combine_ff<<<grid_for(n, 256), 256, 0, s>>>((float4*)state, (const float4*)chains, chain_stride, L, co, n);
     else
         k_combine<double2><<<grid_for(n, 256), 256, 0, s>>>((double2*)state, (const double2*)chains, chain_stride,
                                                                L, co, n);
@@ -376,7 +451,7 @@ cudaError_t launch_count_nonfinite(const void* x, size_t nwords, bool ff, int* c
 }
 
 cudaError_t launch_to_interaction(const KArgs& a, int n, const int* slot_steps, const float* slot_z, int nslots,
-                                  cudaStream_t s) {
+                                  void* scratch, cudaStream_t s) {
     Steps8 st{};
     for (int q = 0; q < 8; ++q) {
         st.s[q] = q < nslots ? slot_steps[q] : -1;
@@ -389,8 +464,17 @@ cudaError_t launch_to_interaction(const KArgs& a, int n, const int* slot_steps, 
     const size_t NP = (size_t)n0 * n1 * n2;
     size_t gx = (NP + 255) / 256;
     if (gx > 1024) gx = 1024;
-    k_to_interaction<<<dim3((unsigned)gx, a.B), 256, 0, s>>>((float4*)a.uhat, (float2*)a.ring, a.ring_slots, a.phi,
-                                                              a.ntf, d, n0, n1, n2, a.dt, n, st, nslots);
+    if (d >= 2) {
+        const int m2 = d == 3 ? n2 : 0;
+        double2* tab = static_cast<double2*>(scratch);
+        k_interaction_tables<<<dim3((unsigned)(nslots + 1), a.B), 256, 0, s>>>(tab, a.phi, a.ntf, n0, n1, m2, a.dt, n, st,
+                                                                               nslots);
+        k_to_interaction_sep<<<dim3((unsigned)gx, a.B), 256, 0, s>>>((float4*)a.uhat, (float2*)a.ring, a.ring_slots, tab, n0,
+                                                                     n1, m2, st, nslots);
+        return cudaGetLastError();
+    }
+    k_to_interaction<<<dim3((unsigned)gx, a.B), 256, 0, s>>>((float4*)a.uhat, (float2*)a.ring, a.ring_slots, a.phi, a.ntf, n0,
+                                                             a.dt, n, st, nslots);
     return cudaGetLastError();
 }
 
