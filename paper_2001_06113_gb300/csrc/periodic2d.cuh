@@ -498,6 +498,72 @@ __global__ void __launch_bounds__((threads_2d<C, N0, L>()), (min_blocks_2d<C, N0
     }
 }
 
+// ------------------------------------- col_fused of the mixed start-up (lab frame)
+// End of a trapezoid sub-step and begin of the next (one history term, the
+// value just transformed): nothing but the state crosses HBM, since the new
+// (Vu)^ goes from the transform into the history sum in registers and the
+// chain's ring slot is written by the chain's last pass only.  State loads four
+// at a time.  The general pass (k_col_end with FUSED) read the state back twice
+// and moved the ring slot: 225 -> 138 us for 5 x 128^3.
+template <int N0, int L>
+__global__ void __launch_bounds__((threads_2d<float2, N0, L>()), (min_blocks_2d<float2, N0, L>())) k_col_chain(const __grid_constant__ KArgs a) {
+    constexpr int T = threads_2d<float2, N0, L>(), PER = (N0 * L + T - 1) / T, G = PER < 4 ? PER : 4;
+    using FW = CtaFft<float2, N0, L, L, T, false>;
+    using FI = CtaFft<float2, N0, L, L, T, true>;
+    static_assert(T % L == 0, "a thread keeps its column");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2* buf = reinterpret_cast<float2*>(smem_raw);
+    const int b = blockIdx.y, c0 = blockIdx.x * L, n1 = a.n1, m1 = c0 + (int)threadIdx.x % L;
+    const size_t NP = (size_t)N0 * n1;
+    float4* st = reinterpret_cast<float4*>(a.uhat) + (size_t)b * NP;
+    wait_previous();
+    allow_next();
+    const float2* T2 = reinterpret_cast<const float2*>(a.aux2) + (size_t)b * NP;
+    batched_copy<float2, N0 * L, T>([&](int item) { return T2[(size_t)(item / L) * n1 + c0 + item % L]; },
+                                    [&](int item, float2 v) { buf[item] = v; });
+    // factors of p_0 of the thread's column (2D, 3D)
+    const Phase2D ph{a, b, 0, m1};
+    const float4* q = a.flat1d ? nullptr : a.qff + ph.base(0);
+    float4 qc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!a.flat1d) {
+        int i1, i2;
+        split12(a, m1, i1, i2);
+        qc = __ldg(&q[a.tn0 + i1]);
+        if (a.tn2 != 0) qc = ffc_mul(qc, __ldg(&q[a.tn0 + a.tn1 + i2]));
+    }
+    __syncthreads();
+    FW::run(buf, a.tw32_0, a.tw32lo_0);
+    const float scale = 1.0f / (float)N0;
+#pragma unroll 1
+    for (int k0 = 0; k0 < PER; k0 += G) {
+        float4 v[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            const int item = threadIdx.x + (k0 + k) * T;
+            if ((N0 * L) % T == 0 || item < N0 * L) v[k] = st[(size_t)(item / L) * n1 + m1];
+        }
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            const int item = threadIdx.x + (k0 + k) * T;
+            if ((N0 * L) % T == 0 || item < N0 * L) {
+                const int m0 = item / L;
+                const float2 R = cscale(buf[item], scale);
+                const float4 u = update_ff(a, v[k], R);
+                const float2 S = make_float2(fmaf(a.mu_lo[1], R.x, a.mu_hi[1] * R.x), fmaf(a.mu_lo[1], R.y, a.mu_hi[1] * R.y));
+                const float4 X = ff_minus_i_times(u, a.h_hi, a.h_lo, S);
+                const float4 p0 = a.flat1d ? Phase2D{a, b, m0, m1}.pff(0) : ffc_mul(__ldg(&q[m0]), qc);
+                const float4 W = ffc_mul(p0, X);
+                st[(size_t)m0 * n1 + m1] = W;
+                buf[item] = make_float2(W.x, W.y);
+            }
+        }
+    }
+    __syncthreads();
+    FI::run(buf, a.tw32_0, a.tw32lo_0);
+    float2* T1 = reinterpret_cast<float2*>(a.aux) + (size_t)b * NP;
+    for (int item = threadIdx.x; item < N0 * L; item += T) T1[(size_t)(item / L) * n1 + c0 + item % L] = buf[item];
+}
+
 // ------------------------------------- col_fused, mixed interaction-picture step
 // Same work as k_col_end<float2, float2, N0, true> for MODE_STEP with the state
 // in the interaction picture, with the mode-space reads staged: the state and
@@ -505,17 +571,11 @@ __global__ void __launch_bounds__((threads_2d<C, N0, L>()), (min_blocks_2d<C, N0
 // into shared memory with cp.async (16-byte copies, no registers held), two
 // chunks ahead, so that the DRAM reads of the step overlap the column FFT
 // and the element work of the previous chunk.  The intermediate v^_n is not
-// stored (the state slot receives X_{n+1} directly).
+// stored (the state slot receives X_{n+1} directly).  (Measured slower: the
+// column's values in registers between the transforms, as in the row pass, one
+// butterfly per thread, 505 against 465 us per 64 x 512^2 step.)
 #ifndef TDSE_PF_ROWS
 #define TDSE_PF_ROWS 32
-#endif
-// 3D mixed chains use this kernel for their fused column pass as well
-#ifndef TDSE_COL_IP_3D
-#define TDSE_COL_IP_3D 1
-#endif
-// ... and 1D grids in the four-step layout
-#ifndef TDSE_COL_IP_1D
-#define TDSE_COL_IP_1D 1
 #endif
 // Rows per chunk: 32, two chunks in flight; with 4 columns (small launches, bound
 // by latency) up to 128, so that most lines have everything in flight at once.
@@ -728,6 +788,16 @@ static cudaError_t col_end_n(const KArgs& a, cudaStream_t s) {
     });
 }
 
+template <int N0>
+static cudaError_t col_chain_n(const KArgs& a, cudaStream_t s) {
+    return with_lanes<float2>((long long)a.n1 * a.B, [&](auto l) {
+        constexpr int L = decltype(l)::value;
+        static bool done = false;
+        return launch_pass(k_col_chain<N0, L>, dim3(a.n1 / L, a.B), threads_2d<float2, N0, L>(), (size_t)N0 * L * sizeof(float2),
+                           done, s, a);
+    });
+}
+
 template <int N0, int VAR = 0>
 static cudaError_t col_fused_ip_n(const KArgs& a, cudaStream_t s) {
     return with_lanes<float2>((long long)a.n1 * a.B, [&](auto l) {
@@ -778,11 +848,20 @@ static cudaError_t row_mid_n(const KArgs& a, cudaStream_t s) {
 #define TDSE_CB(n) col_begin_n<C, RT, n>
 #define TDSE_CE(n) col_end_n<C, RT, n, false>
 #define TDSE_CF(n) col_end_n<C, RT, n, true>
+#define TDSE_CH(n) col_chain_n<n>
 #define TDSE_RM(n) row_mid_n<C, n>
 
 template <class C, class RT> static cudaError_t col_begin(const KArgs& a, cudaStream_t s) { TDSE_SWITCH_N(a.n0, TDSE_CB) }
 template <class C, class RT> static cudaError_t col_end(const KArgs& a, cudaStream_t s) { TDSE_SWITCH_N(a.n0, TDSE_CE) }
-template <class C, class RT> static cudaError_t col_fused(const KArgs& a, cudaStream_t s) { TDSE_SWITCH_N(a.n0, TDSE_CF) }
+// FP64; mixed: a sub-step of the start-up (lab frame, one history term).
+template <class C, class RT> static cudaError_t col_fused(const KArgs& a, cudaStream_t s) {
+    if constexpr (is_f32<C>()) {
+        if (a.ip || a.nhist != 1 || a.hist_slot[0] != a.out_slot) return cudaErrorInvalidValue;
+        TDSE_SWITCH_N(a.n0, TDSE_CH)
+    } else {
+        TDSE_SWITCH_N(a.n0, TDSE_CF)
+    }
+}
 template <class C> static cudaError_t row_mid(const KArgs& a, cudaStream_t s) { TDSE_SWITCH_N(a.n1, TDSE_RM) }
 
 template <class C, class RT>
@@ -818,7 +897,7 @@ static cudaError_t part2d(const KArgs& a, int part, cudaStream_t s) {
                     TDSE_SWITCH_N(a.n0, TDSE_CFI)
 #undef TDSE_CFI
                 }
-                if (TDSE_COL_IP_1D && a.mode == MODE_STEP && a.ip && a.flat1d) {
+                if (a.mode == MODE_STEP && a.ip && a.flat1d) {
 #define TDSE_CFI1(n) col_fused_ip_n<n, 2>
                     TDSE_SWITCH_N(a.n0, TDSE_CFI1)
 #undef TDSE_CFI1
@@ -906,7 +985,7 @@ static KArgs row3(const KArgs& a) {
 template <class C, class RT>
 static cudaError_t col_fused_3d(const KArgs& a, cudaStream_t s) {
     if constexpr (std::is_same<C, float2>::value && std::is_same<RT, float2>::value) {
-        if (TDSE_COL_IP_3D && a.mode == MODE_STEP && a.ip) {
+        if (a.mode == MODE_STEP && a.ip) {
 #define TDSE_CFI3(n) col_fused_ip_n<n, 1>
             TDSE_SWITCH_N(a.n0, TDSE_CFI3)
 #undef TDSE_CFI3
