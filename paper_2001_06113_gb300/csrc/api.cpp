@@ -811,8 +811,11 @@ static tdse_status startup_step(tdse_ctx* c, int n, cudaStream_t s) {
     for (int ch = 0; ch < c->L && !one_launch; ++ch) {
         void* cu = chain_u + (size_t)ch * NPB * 16;
         void* cr = chain_r + (size_t)ch * NPB * c->rsz;
-        TDSE_CK(c, cudaMemcpyAsync(cu, c->P<void>(c->off.uhat), NPB * 16, cudaMemcpyDeviceToDevice, s));
-        TDSE_CK(c, launch_copy_slot(cr, c->P<void>(c->off.ring), c->RS, slot_of(c, n - 1), c->B, c->NP, c->rsz, s));
+        const bool passes = c->d > 1 || c->four1d;
+        if (!passes) {
+            TDSE_CK(c, cudaMemcpyAsync(cu, c->P<void>(c->off.uhat), NPB * 16, cudaMemcpyDeviceToDevice, s));
+            TDSE_CK(c, launch_copy_slot(cr, c->P<void>(c->off.ring), c->RS, slot_of(c, n - 1), c->B, c->NP, c->rsz, s));
+        }
         const int len = SUB >> ch, last = (1 << ch) - 1;
         auto sub = [&](int i) {     // trapezoid sub-step i of the chain
             KArgs a = base_args(c);
@@ -829,7 +832,7 @@ static tdse_status startup_step(tdse_ctx* c, int n, cudaStream_t s) {
             set_time(c, a, SUB * (n - 1) + (i + 1) * len);
             return a;
         };
-        if (c->d == 1 && !c->four1d) {
+        if (!passes) {
             for (int i = 0; i <= last; ++i) TDSE_CK(c, run(c, sub(i), step_combo(c), s));
             continue;
         }
@@ -837,7 +840,13 @@ static tdse_status startup_step(tdse_ctx* c, int n, cudaStream_t s) {
         // pass as in the Adams steps (the arguments are those of i + 1; ring slot,
         // h and weights are the chain's), 15 + 4 column passes per start-up step
         // instead of 30: 64 x 512^2 mixed, 300 steps, 221.6 -> 211.8 ms.
-        TDSE_CK(c, step_part(c, sub(0), step_combo(c), PART_COL_BEGIN, s));
+        // The first begin reads the state and the last (Vu)^ where they are.
+        KArgs first = sub(0);
+        first.uhat_src = c->P<void>(c->off.uhat);
+        first.ring = c->P<void>(c->off.ring);
+        first.ring_slots = c->RS;
+        first.hist_slot[0] = slot_of(c, n - 1);
+        TDSE_CK(c, step_part(c, first, step_combo(c), PART_COL_BEGIN, s));
         for (int i = 0; i <= last; ++i) {
             TDSE_CK(c, step_part(c, sub(i), step_combo(c), PART_ROW_MID, s));
             TDSE_CK(c, i < last ? step_part(c, sub(i + 1), step_combo(c), PART_COL_FUSED, s)

@@ -566,6 +566,7 @@ __device__ __forceinline__ float2 cmul_add2(float2 c, float2 R, float2 b, float2
 template <class N> struct PhaseTab;
 template <class N> struct RowPtr {
     using C = typename N::C;
+    const double2* src;
     double2* uh;
     C* out;
     const C* lag[FS_MAX_HIST];
@@ -651,11 +652,12 @@ __device__ __forceinline__ void row_factors(const FsArgs& a, int g, Sm& sm, int 
 }
 
 template <class N>
-__device__ __forceinline__ RowPtr<N> row_ptr(const FsArgs& a, bool end, double2* uh, typename N::C* ring, size_t slot_stride,
+__device__ __forceinline__ RowPtr<N> row_ptr(const FsArgs& a, bool end, const double2* src, double2* uh, typename N::C* ring, size_t slot_stride,
                                              const int4* P, const typename PhaseTab<N>::type* Pc, int Nm) {
     RowPtr<N> p;
+    p.src = src;
     p.uh = uh;
-    p.out = ring + (size_t)a.out_slot * slot_stride;
+    p.out = ring + (size_t)(a.out_slot < 0 ? 0 : a.out_slot) * slot_stride;      // (not written by a begin alone)
 #pragma unroll
     for (int j = 0; j < FS_MAX_HIST; ++j) {
         const int i = j < a.nhist ? j : 0;
@@ -676,7 +678,7 @@ template <class N>
 __device__ __forceinline__ double2 update_mode(const FsArgs& a, int g, const int4* c, bool end, bool begin, int m,
                                                typename N::C F, const RowPtr<N>& p) {
     using C = typename N::C;
-    double2 u = p.uh[m];
+    double2 u = p.src[m];
     C r[FS_MAX_HIST];
     int4 b0 = make_int4(0, 0, 0, 0);
     if (begin) {
@@ -783,7 +785,7 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
     row_factors<N>(a, g, sm, G::T, [&](int) { return make_int4(1 << (28 - g), 0, 0, 0); });    // 1
     __syncthreads();
     unsigned mx = 0;
-    const RowPtr<N> rp = row_ptr<N>(a, false, uh, ring, (size_t)Nm, P, Pc, Nm);
+    const RowPtr<N> rp = row_ptr<N>(a, false, uh, uh, ring, (size_t)Nm, P, Pc, Nm);
     each_mode<N, Ln>(ax, sm, false, 0, [&](int m, C F, C* at) {
         *at = to_c(update_mode<N>(a, g, sm.c, false, true, m, F, rp), C());
         if constexpr (N::FX) mx = max(mx, fx_hi(*at));
@@ -824,6 +826,7 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
     const int nrows = d3 ? N0 * a.ax[1].N : N0;
     const size_t NPm = (size_t)nrows * N1;
     double2* urow = a.uhat + (size_t)b * NPm + (size_t)k0 * N1;
+    const double2* usrc = a.uhat_src ? a.uhat_src + (size_t)b * NPm + (size_t)k0 * N1 : urow;
     C* zrow = reinterpret_cast<C*>(a.Z) + ((size_t)b * nrows + k0) * M;
     const bool end = flags & FS_ROW_END, begin = flags & FS_ROW_BEGIN;
     if (begin) {   // phase of the row over interval iv: P0 (2D), P0 P1 of axes 0 and 1 (3D)
@@ -840,7 +843,7 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
     if (begin) {
         const C* ring0 = reinterpret_cast<const C*>(a.ring) + (size_t)b * a.ring_slots * NPm + (size_t)k0 * N1;
         for (int off = (int)threadIdx.x * 128; off < N1 * 16; off += G::T * 128) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(urow) + off));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(usrc) + off));
             if (off < N1 * (int)sizeof(C))
                 for (int j = 0; j < a.nhist; ++j)
                     if (!(end && a.hist_slot[j] == a.out_slot))
@@ -870,7 +873,7 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
     const auto* P1c = PhaseTab<N>::get(ax) + (size_t)b * a.n_int * N1;
     C* ring = reinterpret_cast<C*>(a.ring) + (size_t)b * a.ring_slots * NPm + (size_t)k0 * N1;
     unsigned mx = 0;
-    const RowPtr<N> rp = row_ptr<N>(a, end, urow, ring, NPm, P1, P1c, N1);
+    const RowPtr<N> rp = row_ptr<N>(a, end, usrc, urow, ring, NPm, P1, P1c, N1);
     each_mode<N, Ln>(ax, sm, end, xe, [&](int m, C F, C* at) {
         const double2 W = update_mode<N>(a, g, sm.c, end, begin, m, F, rp);
         if (begin) {

@@ -413,17 +413,18 @@ tdse_status fs_init(tdse_ctx* c, cudaStream_t s) {
     return TDSE_OK;
 }
 
-// Steps first..last of a chain, step i described by args(i).  2D / 3D: row
+// Steps first..last of a chain, step i described by args(i), the begin of the
+// first by begin().  2D / 3D: row
 // begin, (grid part, row end + begin) x (last - first), grid part, row end;
 // the end of step i runs with the arguments of i + 1 and the ring slot of i.
-template <class Args>
-tdse_status fs_chain(tdse_ctx* c, Args args, int first, int last, cudaStream_t s) {
+template <class Begin, class Args>
+tdse_status fs_chain(tdse_ctx* c, Begin begin, Args args, int first, int last, cudaStream_t s) {
     const int f32 = c->F.f32 ? 1 : 0;
     if (c->d == 1) {
         for (int i = first; i <= last; ++i) TDSE_CK(c, launch_fs_1d(args(i), FS_1D_STEP, f32, s));
         return TDSE_OK;
     }
-    TDSE_CK(c, launch_fs_row(args(first), FS_ROW_BEGIN, f32, s));
+    TDSE_CK(c, launch_fs_row(begin(), FS_ROW_BEGIN, f32, s));
     for (int i = first; i <= last; ++i) {
         const FsArgs a = args(i);
         tdse_status st = grid_part(c, a, f32, s);
@@ -444,8 +445,10 @@ tdse_status fs_startup_step(tdse_ctx* c, int n, cudaStream_t s) {
     double2* cx = c->P<double2>(F.off.chain_u);
     for (int ch = 0; ch < c->L; ++ch) {
         double2* cr = ring_at(c, F.off.chain_ring, ch * BM);
-        TDSE_CK(c, cudaMemcpyAsync(cu + ch * BM, c->P<double2>(F.off.uhat), BM * 16, cudaMemcpyDeviceToDevice, s));
-        TDSE_CK(c, launch_copy_slot(cr, c->P<void>(F.off.ring), c->RS, slot_of(c, n - 1), c->B, F.NM, c->rsz, s));
+        if (c->d == 1) {
+            TDSE_CK(c, cudaMemcpyAsync(cu + ch * BM, c->P<double2>(F.off.uhat), BM * 16, cudaMemcpyDeviceToDevice, s));
+            TDSE_CK(c, launch_copy_slot(cr, c->P<void>(F.off.ring), c->RS, slot_of(c, n - 1), c->B, F.NM, c->rsz, s));
+        }
         const int len = SUB >> ch, last = (1 << ch) - 1;
         auto sub = [&](int i) {     // trapezoid sub-step i of the chain
             FsArgs a = fs_base(c);
@@ -461,7 +464,17 @@ tdse_status fs_startup_step(tdse_ctx* c, int n, cudaStream_t s) {
             set_time(c, a, SUB * (n - 1) + (i + 1) * len);
             return a;
         };
-        tdse_status st = fs_chain(c, sub, 0, last, s);
+        // 2D / 3D: the first begin reads the state and the last (Vu)^ where they are
+        auto first = [&]() {
+            FsArgs a = sub(0);
+            a.uhat_src = c->P<double2>(F.off.uhat);
+            a.ring = c->P<double2>(F.off.ring);
+            a.ring_slots = c->RS;
+            a.hist_slot[0] = slot_of(c, n - 1);
+            a.out_slot = -1;
+            return a;
+        };
+        tdse_status st = fs_chain(c, first, sub, 0, last, s);
         if (st != TDSE_OK) return st;
     }
     TDSE_CK(c, launch_combine(c->P<void>(F.off.uhat), cu, BM, c->L, c->rich, BM, false, s));
@@ -481,7 +494,8 @@ FsArgs adams_args(const tdse_ctx* c, int n) {
 }
 
 tdse_status fs_adams(tdse_ctx* c, int n0, int k, cudaStream_t s) {
-    return fs_chain(c, [&](int n) { return adams_args(c, n); }, n0 + 1, n0 + k, s);
+    auto args = [&](int n) { return adams_args(c, n); };
+    return fs_chain(c, [&]() { return args(n0 + 1); }, args, n0 + 1, n0 + k, s);
 }
 
 // FP64 residual of the implicit step just completed (step c->step, FP32

@@ -97,6 +97,7 @@ struct FsArgs {
     int interval[FS_MAX_HIST];    // interval id of the one-step phase p_i, i = 0..nhist-1
     int tf;                // fine time index of the new time (t = tf dt / 8)
     // ---- buffers
+    const double2* uhat_src;   // row begin: the state to start from, if not uhat (a start-up chain's first sub-step)
     double2* uhat;         // [B][N0 N1] mode state: u^ between steps, W inside a step (FP64 in both variants)
     double2* ring;         // [B][ring_slots][N0 N1] history of (Vu)^ (elements of the transform type)
     int ring_slots;

@@ -69,6 +69,7 @@ struct KArgs {
     int e_next;               // fused column pass: n of the next step's E
     // ---- state
     void* uhat;               // [B][NP] state (ST)
+    const void* uhat_src;     // col_begin: the state to start from, if not uhat (a start-up chain's first sub-step)
     void* ring;               // [B][ring_slots][NP] ring (RT)
     int ring_slots;
     double2* aux;             // 2D intermediate T1 (16 B per element)

@@ -126,11 +126,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
 // Start of a step at mode (m0, m1): returns the inverse-DFT input and updates
 // the state slot (W or X) in MODE_STEP.
 template <class C, class RT>
-__device__ __forceinline__ C begin_elem(const KArgs& a, bool step, int b, state_t<RT>* st, const RT* ringb,
+__device__ __forceinline__ C begin_elem(const KArgs& a, bool step, int b, const state_t<RT>* src, state_t<RT>* st, const RT* ringb,
                                         size_t NP, size_t idx, int m0, int m1, int n_e) {
     using ST = state_t<RT>;
     constexpr bool FF = !is_f64<RT>::value;
-    ST W = st[idx];
+    ST W = src[idx];
     if (step) {
         if constexpr (!FF) {
             Phase2D ph{a, b, m0, m1};
@@ -193,6 +193,7 @@ __global__ void __launch_bounds__((threads_2d<C, N0, L>()), (min_blocks_2d<C, N0
     const int n1 = a.n1;
     const size_t NP = (size_t)N0 * n1;
     ST* st = reinterpret_cast<ST*>(a.uhat) + (size_t)b * NP;
+    const ST* src = a.uhat_src ? reinterpret_cast<const ST*>(a.uhat_src) + (size_t)b * NP : st;
     const RT* ringb = reinterpret_cast<const RT*>(a.ring) + (size_t)b * a.ring_slots * NP;
     const tw_t<C>* tw;
     const tw_t<C>* twl;
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__((threads_2d<C, N0, L>()), (min_blocks_2d<C, N0
     for (int item = threadIdx.x; item < N0 * L; item += T) {
         const int lane = item % L, m0 = item / L;
         const int m1 = c0 + lane;
-        buf[m0 * L + lane] = begin_elem<C, RT>(a, step, b, st, ringb, NP, (size_t)m0 * n1 + m1, m0, m1, a.e_step);
+        buf[m0 * L + lane] = begin_elem<C, RT>(a, step, b, src, st, ringb, NP, (size_t)m0 * n1 + m1, m0, m1, a.e_step);
     }
     __syncthreads();
     FI::run(buf, tw, twl);
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__((threads_2d<C, N0, L>()), (min_blocks_2d<C, N0
         const int m1 = c0 + lane;
         const size_t idx = (size_t)m0 * n1 + m1;
         end_elem<C, RT>(a, step, b, st, ringb, NP, idx, m0, m1, norm_of(buf[m0 * L + lane], scale), a.e_step);
-        if constexpr (FUSED) buf[m0 * L + lane] = begin_elem<C, RT>(a, true, b, st, ringb, NP, idx, m0, m1, a.e_next);
+        if constexpr (FUSED) buf[m0 * L + lane] = begin_elem<C, RT>(a, true, b, st, st, ringb, NP, idx, m0, m1, a.e_next);
     }
     if constexpr (FUSED) {
         __syncthreads();
