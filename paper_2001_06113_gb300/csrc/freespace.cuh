@@ -205,9 +205,10 @@ template <int M_, int R_> struct Geo {
     static constexpr int LA = ilog2(A), LB = ilog2(B), LR = ilog2(R), LF = ilog2(FOLD), LM = ilog2(M);
 };
 // Resident CTAs: 2 of 256 threads for the fixed-point kernels (up to 128
-// registers), FS_MINB32 for the FP32 ones.
+// registers), FS_MINB32 for the FP32 ones (256^2, per step: 3, 4, 5, 6 CTAs 317,
+// 294, 289, 329 us).
 #ifndef FS_MINB32
-#define FS_MINB32 4
+#define FS_MINB32 5
 #endif
 template <class N, class G> constexpr int min_blocks() {
     const int t = N::FX ? 512 : 256 * FS_MINB32;
@@ -729,6 +730,7 @@ __device__ __forceinline__ typename N::C mode_value(typename N::V v, int xe) {
 // f(m, F, W) for every mode m of this thread, equispaced and dense: F its
 // forward result (where have_F), W where its input of the inverse transform
 // goes.  One rolled loop: the mode update is the kernel's largest piece of code.
+// (Loads issued one mode ahead were slower: 307 to 356 us, for 3 to 5 CTAs.)
 template <class N, class Ln, class Fn>
 __device__ __forceinline__ void each_mode(const FsAxis& ax, typename Ln::Sm& sm, bool have_F, int xe, Fn f) {
     using C = typename N::C;
