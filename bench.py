@@ -61,9 +61,6 @@ METRIC = "point-steps/s (2D periodic 512^2, 8th-order, T=2)"
 # Algorithmic HBM bytes per point-step of the step operator: read u^ (16) and
 # 7 history slots, write u^ (16) and one slot; V read once (real).
 ALGO_BYTES = {"fp64": 16 + 7 * 16 + 8 + 16 + 16, "mixed": 16 + 7 * 8 + 4 + 16 + 8}
-# FP64 FMA throughput of this GB300 pool (register-resident FMA chains, all
-# SMs), TFLOP/s: the peak of the FP64-bound free-space step.
-FP64_PEAK_TFLOPS = 1.25          # nominal FP64 rate, context only (the lines divide by fp64_peak())
 
 
 def parse():
@@ -180,19 +177,15 @@ class ClockSampler:
 
 
 # ------------------------------------------------------------------- GPU arm
-def launches_per_solve(dim: int, mixed: bool, path: str = "passes") -> int:
-    """Kernel launches of one tdse_step(NSTEPS) call (init, start-up, Adams);
+def launches_per_solve(mixed: bool, path: str = "passes", groups: int = 1) -> int:
+    """Kernel launches of one 2D tdse_step(NSTEPS) call (init, start-up, Adams);
     the cluster path runs all Adams steps of the call in one launch."""
     L = ORDER // 2
     sub = sum(2 ** c for c in range(L))      # trapezoid sub-steps per start-up step
-    per_op = 1 if dim == 1 else 3            # kernels per unfused application of the step operator
-    startup = STARTUP * (L + sub * per_op + 1 + per_op)   # copy_slot per chain, sub-steps, combine, refresh
-    init = 1 if dim == 1 else 2
+    startup = STARTUP * (L + sub * 2 + 1 + 3)   # begin per chain, (row, column) per sub-step, combine, refresh
     k = NSTEPS - STARTUP
-    adams = k if dim == 1 else 2 * k + 1     # 2D: col_begin, (row_mid, col_fused) x (k-1), row_mid, col_end
-    if dim == 2 and path == "cluster":
-        adams = 1
-    return init + startup + (1 if mixed else 0) + adams
+    adams = 1 if path == "cluster" else groups * (2 * k + 1)   # col_begin, then (row, column) per step
+    return 2 + startup + (1 if mixed else 0) + adams
 
 
 # DRAM bytes per point-step of the 2D step operator (k_row_mid + k_col_fused_ip)
@@ -282,7 +275,7 @@ def run_gpu(args, ws, rank, local):
     tb = TRAFFIC_BYTES_PER_POINT_STEP.get((args.precision, shape["path"]))
     traffic = None if tb is None else round(tb * B * points)
     kname = {"cluster": "k_step2d_cluster (one 16-CTA cluster per instance, a run of steps per launch)",
-             "passes": "k_row_mid + k_col_fused_ip" if args.precision == "mixed" else "k_row_mid + k_col_end (FP64)"}
+             "passes": "k_row32 + k_col_fused_ip" if args.precision == "mixed" else "k_row_mid + k_col_end (FP64)"}
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic, "traffic_unit": "bytes per step (all instances)",
                 "traffic_note": TRAFFIC_NOTE.get((args.precision, shape["path"])),
@@ -392,13 +385,17 @@ def fp64_variant(args, insts, stream, dev, mixed_value, oracle_err):
                     evs[i + 1].record(stream)
             stream.synchronize()
             t_step = float(np.mean([evs[i].elapsed_time(evs[i + 1]) / 1e3 / GROUP for i in range(NGROUPS)]))
-            ach = FP64_FLOPS_PER_POINT_STEP * B * M * M / t_step / 1e12
-            entry["roofline"] = {"bound": "alu", "achieved": round(ach, 4), "peak": round(peak, 4),
-                                 "unit": "TFLOP/s (FP64)", "frac": round(ach / peak, 4), "traffic": None,
-                                 "peak_source": peak_note,
+            # transforms, history and solve are 64-bit fixed point on the integer
+            # pipe, so the FP64 rate is no ceiling: given beside the HBM line
+            hpk, hsrc = hbm_peak()
+            gbs = ALGO_BYTES["fp64"] * B * M * M / t_step / 1e9
+            entry["roofline"] = {"bound": "hbm", "achieved": round(gbs, 1), "peak": hpk, "unit": "GB/s",
+                                 "frac": round(gbs / hpk, 4), "traffic": None, "peak_source": hsrc,
+                                 "algorithmic_bytes_per_point_step": ALGO_BYTES["fp64"],
                                  "kernel": "k_row_mid<double2,512> + k_col_end<double2,double2,512,1> (FP64 Adams step), "
                                            f"timed over groups of {GROUP} steps",
-                                 "algorithmic_flops_per_point_step": FP64_FLOPS_PER_POINT_STEP,
+                                 "fp64_equivalent": fp64_equivalent(
+                                     FP64_FLOPS_PER_POINT_STEP * B * M * M / t_step / 1e12, peak, peak_note),
                                  "step_ms": round(t_step * 1e3, 4)}
             entry["rel_l2_vs_oracle"] = oracle_err.get("fp64_gpu") if oracle_err else None
         prob.close()
@@ -506,6 +503,14 @@ def fp64_peak(dev) -> tuple:
         best = t if best is None else min(best, t)
     del a, b
     return 2.0 * n ** 3 / best / 1e12, "measured in this run: cuBLAS float64 GEMM 4096^3, best of 3"
+
+
+def fp64_equivalent(achieved: float, peak: float, note: str) -> dict:
+    """The algorithm's FP64 flops per second beside the GPU's FP64 rate.  Above 1
+    is possible: the kernels do this arithmetic in 64-bit fixed point on the
+    integer pipe."""
+    return {"achieved": round(achieved, 4), "fp64_rate": round(peak, 4), "unit": "TFLOP/s (FP64)",
+            "ratio": round(achieved / peak, 4), "rate_source": note}
 
 
 GOLDEN_512 = os.path.join(ROOT, "tests", "golden", "periodic_2d_wells_512.npz")
@@ -620,11 +625,13 @@ def run_free(args, ws, rank, local):
               "step_ms_p50": round(float(np.percentile(dts, 50)) * 1e3, 4),
               "step_ms_p99": round(float(np.percentile(dts, 99)) * 1e3, 4)}
     if prec == "fp64":
-        peak64, src64 = fp64_peak(dev)
-        roofline = {"bound": "alu", "achieved": round(achieved, 4), "peak": round(peak64, 4), "unit": "TFLOP/s",
-                    "frac": round(achieved / peak64, 4), "traffic": traffic,
+        algo = free_algo_bytes(prec) * B
+        hpk, hsrc = hbm_peak()
+        roofline = {"bound": "hbm", "achieved": round(algo / t_step / 1e9, 1), "peak": hpk, "unit": "GB/s",
+                    "frac": round(algo / t_step / 1e9 / hpk, 4), "algorithmic_bytes_per_step": algo,
+                    "traffic": traffic,
                     "traffic_unit": "DRAM bytes per fused k_fs_row launch (ncu), per instance x instances",
-                    "peak_source": src64, "nominal_fp64_tflops": FP64_PEAK_TFLOPS, **timing}
+                    "peak_source": hsrc, "fp64_equivalent": fp64_equivalent(achieved, *fp64_peak(dev)), **timing}
     else:
         # FP32 transforms: both ceilings, the nearer one reported as the bound
         algo = free_algo_bytes(prec) * B
@@ -686,7 +693,7 @@ def run_free(args, ws, rank, local):
 def free_launches_per_solve() -> int:
     L = ORDER // 2
     sub = sum(2 ** c for c in range(L))
-    startup = STARTUP * (L + sub * 3 + 2 + 2)   # copy_slot per chain, sub-steps, 2 combines, refresh (2)
+    startup = STARTUP * (L + sub * 2 + 2 + 2)   # begin per chain, (grid, row) per sub-step, 2 combines, refresh (2)
     init = 4
     k = FS_NSTEPS - STARTUP
     return init + startup + 2 * k + 1
@@ -729,7 +736,7 @@ def profile_run(args):
     torch.cuda.synchronize()
     prob.check_finite()
     print(json.dumps({"profile_adams": args.profile_adams, "batch": len(insts), "precision": args.precision,
-                      "launches_before_adams": launches_per_solve(2, args.precision == "mixed")
+                      "launches_before_adams": launches_per_solve(args.precision == "mixed")
                       - (2 * (NSTEPS - STARTUP) + 1)}))
     prob.close()
     return 0
@@ -968,7 +975,7 @@ def run_batch1d(args, ws, rank, local):
                 "traffic_unit": "DRAM bytes per k_periodic1d_multi launch (ncu, default launch shape)",
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                 "kernel": ("k_periodic1d_multi (one persistent launch per Adams step for all 512 instances)" if fused
-                           else "k_periodic1d<float2,float2,N> per member size, on parallel streams (tuner's "
+                           else "k_run1d32<N> (and four-step passes) per member size, on parallel streams (tuner's "
                                 "choice over the fused launch)") + ", timed per step over 100 steps",
                 "algorithmic_bytes_per_point_step": B1_ALGO_BYTES,
                 "step_ms_p50": round(float(np.percentile(dts, 50)) * 1e3, 4),
@@ -1024,12 +1031,23 @@ def run_batch1d(args, ws, rank, local):
                 errs=errs, f64_one_at_a_time=f64_points / f64_time if f64_time else None)
 
 
-def batch1d_launches(shape_members: int) -> int:
-    """Launches of one 1000-step batch solve: per member init + start-up
-    (7 x (4 copies + 15 sub-steps + combine + refresh)) + change of frame,
-    then one fused launch per Adams step."""
-    per_member = 1 + STARTUP * (4 + 15 + 1 + 1) + 1
-    return shape_members * per_member + (B1_NSTEPS - STARTUP)
+def batch1d_launches(sizes, nsteps: int, fused: bool, passes_from=None) -> int:
+    """Launches of one batch solve: per member init, start-up and change of
+    frame, then its Adams steps.  One CTA per instance (n <= 8192): a start-up
+    step is its chains, the combination and the refresh, and all Adams steps one
+    launch (fused mode: one launch per step for these members together).
+    Four-step members: the pass launches of launches_per_solve."""
+    L, k = ORDER // 2, nsteps - STARTUP
+    sub = sum(2 ** c for c in range(L))
+    total = k if fused else 0
+    for n in sizes:
+        if passes_from and n >= passes_from:
+            total += 2 + STARTUP * (L + 2 * sub + 1 + 3) + 1 + 2 * k + 1
+        elif n <= 8192:
+            total += 1 + STARTUP * 3 + 1 + (0 if fused else 1)
+        else:                                    # one CTA, a launch per sub-step and step
+            total += 2 + STARTUP * (L + sub + 1 + 1) + 1 + (0 if fused else k)
+    return total
 
 
 def batch1d_oracle_sample(nadams: int = 20):
@@ -1131,7 +1149,8 @@ def main_batch1d(args, ws, rank, local):
             "time_to_solution_s": {"p50": res["t_solve"], "p99": res["t_solve"],
                                    "note": "all instances of the batch finish together"},
             "roofline": res["roofline"], "cpu_baseline": cpu, "e2e": res["e2e"], "clocks": res["clocks"],
-            "gpu_launches": batch1d_launches(len(res["sizes"])) * args.steps,
+            "gpu_launches": batch1d_launches(res["sizes"], B1_NSTEPS, res["shape"].get("mode", "fused") == "fused",
+                                             args.passes_from) * args.steps,
         }
         print(json.dumps(line))
     if ws > 1:
@@ -1146,9 +1165,6 @@ EX_METRIC = ("point-steps/s (Example 1 moving periodic Gaussian well, V0=300, be
 # per point-step: state in/out 32, 7 ring reads 56, 1 ring write 8; the V row
 # (one shared table per speed) is read once per step for all instances
 EX_ALGO_BYTES = 16 + 7 * 8 + 16 + 8
-# DRAM bytes of one k_periodic1d<float2,float2,512> Adams-step launch over 2048
-# instances (ncu, profiles/example1_moving_well_512_mixed.md); per step x 3 speeds
-EX_LAUNCH_TRAFFIC = 77.75232e6 + 5.611776e6
 
 
 def example1_oracle_sample(nadams: int = 400):
@@ -1248,12 +1264,11 @@ def run_example1(args, ws, rank, local):
     achieved = EX_ALGO_BYTES * points / t_step / 1e9
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4),
-                "traffic": EX_LAUNCH_TRAFFIC * len(probs) * B / 2048 if shape.get("mode") == "streams" else None,
-                "traffic_unit": "DRAM bytes per Adams step (ncu launch of 2048 instances, scaled by instances)",
+                "traffic": None,
                 "peak_source": peak_src,
                 "kernel": ("k_periodic1d_multi (one persistent launch per Adams step for all instances of the three "
                            "speeds)" if shape.get("mode", "fused") == "fused" else
-                           "k_periodic1d<float2,float2,512> per speed on parallel streams (tuner's choice over the "
+                           "k_run1d32<512> per speed on parallel streams (tuner's choice over the "
                            "fused launch)") + ", timed per step over 100 steps",
                 "algorithmic_bytes_per_point_step": EX_ALGO_BYTES,
                 "step_ms_p50": round(float(np.percentile(dts, 50)) * 1e3, 4),
@@ -1375,7 +1390,8 @@ def main_example1(args, ws, rank, local):
                        "parallelism": f"replicas x{ws}"},
             "rel_l2_vs_fp64": res["errs"], "fp64_dt_error_c30": res["err_dt"],
             "roofline": res["roofline"], "cpu_baseline": cpu, "e2e": res["e2e"], "clocks": res["clocks"],
-            "gpu_launches": (3 * (1 + STARTUP * (4 + 15 + 1 + 1) + 1) + (EX_NSTEPS - STARTUP)) * args.steps,
+            "gpu_launches": batch1d_launches([EX_M] * 3, EX_NSTEPS,
+                                             res["shape"].get("mode", "fused") == "fused") * args.steps,
         }
         print(json.dumps(line))
     if ws > 1:
@@ -1530,12 +1546,12 @@ def oracle_sample_3d(nadams: int = 1):
 
 def launches_per_solve_3d(mixed: bool, groups: int) -> int:
     """Kernel launches of one tdse_step(NSTEPS3) call on a 3D context: one
-    unfused application of the step operator is 5 kernels (column pass,
-    axis-1 pass, row pass, axis-1 pass, column pass); each Adams step of a
-    group chain is 4 (row pass, axis-1, fused column pass, axis-1)."""
+    application of the step operator by itself is 5 kernels (column pass, axis-1
+    pass, row pass, axis-1 pass, column pass); a sub-step or Adams step within a
+    chain is 4, its end sharing the column pass with the next begin."""
     L = ORDER // 2
     sub = sum(2 ** c for c in range(L))
-    startup = STARTUP * (L + sub * 5 + 1 + 5)
+    startup = STARTUP * (L + sub * 4 + 1 + 5)   # begin per chain, (axis 1, row, axis 1, column) per sub-step
     k = NSTEPS3 - STARTUP
     adams = groups * (2 + (k - 1) * 4 + 3)
     return 4 + startup + (1 if mixed else 0) + adams
@@ -1638,12 +1654,13 @@ def main_periodic3d(args, ws, rank, local):
                 "kernel": "3D Adams step operator: column pass (axis 0), axis-1 passes, row pass (axis 2), "
                           f"timed over groups of {GROUP} steps"}
     else:
-        peak, src = fp64_peak(dev)
+        peak, src = hbm_peak()
+        gbs = ALGO_BYTES["fp64"] * B * P3 / t_step / 1e9
         fl = 6 * 35 + (6 * 18 + 7 * 4 + 4 + 18) + 21 + 4 + 6   # six 128-point transforms per point, 3-axis phases
         ach = fl * B * P3 / t_step / 1e12
-        roof = {"bound": "alu", "achieved": round(ach, 4), "peak": round(peak, 4), "unit": "TFLOP/s (FP64)",
-                "frac": round(ach / peak, 4), "traffic": None, "peak_source": src,
-                "algorithmic_flops_per_point_step": fl,
+        roof = {"bound": "hbm", "achieved": round(gbs, 1), "peak": peak, "unit": "GB/s", "frac": round(gbs / peak, 4),
+                "traffic": None, "peak_source": src, "algorithmic_bytes_per_point_step": ALGO_BYTES["fp64"],
+                "fp64_equivalent": fp64_equivalent(ach, *fp64_peak(dev)),
                 "kernel": f"3D FP64 Adams step operator, timed over groups of {GROUP} steps"}
     roof["step_ms_p50"] = round(float(np.percentile(dts, 50)) * 1e3, 4)
     roof["step_ms_p99"] = round(float(np.percentile(dts, 99)) * 1e3, 4)
@@ -1914,9 +1931,13 @@ def main_free3d(args, ws, rank, local):
               "algorithmic_flops_per_step": flops, "modes_per_axis": N,
               "step_ms_p50": round(float(np.percentile(dts, 50)) * 1e3, 4)}
     if prec == "fp64":
-        peak, src = fp64_peak(dev)
-        roofline = {"bound": "alu", "achieved": round(achieved, 4), "peak": round(peak, 4), "unit": "TFLOP/s",
-                    "frac": round(achieved / peak, 4), "traffic": None, "peak_source": src, **timing}
+        algo = free3d_algo_bytes(N, 16)
+        hpk, hsrc = hbm_peak()
+        gbs = algo / t_step / 1e9
+        roofline = {"bound": "hbm", "achieved": round(gbs, 1), "peak": hpk, "unit": "GB/s",
+                    "frac": round(gbs / hpk, 4), "traffic": None, "peak_source": hsrc,
+                    "algorithmic_bytes_per_step": algo, "fp64_equivalent": fp64_equivalent(achieved, *fp64_peak(dev)),
+                    **timing}
     else:
         # FP32 transforms: both ceilings, the nearer one reported as the bound
         algo = free3d_algo_bytes(N, 8)
@@ -2053,8 +2074,8 @@ def main():
             else res["oracle_err"],
             "fp64_variant": res["fp64"],
             "roofline": res["roofline"], "cpu_baseline": cpu, "e2e": res["e2e"], "clocks": res["clocks"],
-            "gpu_launches": launches_per_solve(2, args.precision == "mixed",
-                                               res["roofline"]["launch_shape"]["path"]) * args.steps,
+            "gpu_launches": launches_per_solve(args.precision == "mixed", res["roofline"]["launch_shape"]["path"],
+                                               res["roofline"]["launch_shape"].get("groups", 1)) * args.steps,
         }
         print(json.dumps(line))
     if ws > 1:

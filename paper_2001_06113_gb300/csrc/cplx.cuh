@@ -1,4 +1,6 @@
-// Complex arithmetic on double2/float2 and a shared-memory Stockham FFT.
+// Complex arithmetic on double2/float2 and a shared-memory Stockham FFT (FP32
+// values as written below; FP64 values through the same passes in 64-bit fixed
+// point, fx.cuh).
 //
 // The FFT computes, for each of L interleaved sequences of length N,
 //     forward:  X_k = sum_j x_j e^{-2 pi i j k / N}

@@ -1,4 +1,6 @@
 // 1D periodic step: one CTA per instance, the whole transform in shared memory.
+// (FP64 solves of n <= 1024 and mixed runs of n <= 8192 take run1d64.cu and
+// run1d32.cu instead: a run of steps per launch.)
 //
 // MODE_STEP fuses, for an instance of N modes, in one launch:
 //   history sum + phase (eq. uadamsk, lab frame or interaction picture) -> W

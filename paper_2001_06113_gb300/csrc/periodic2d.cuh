@@ -1,10 +1,11 @@
 // 2D periodic step as shared-memory pass kernels over [B][n0][n1]
 // (row-major, axis 1 contiguous):
 //
-//   col_begin (axis 0, 8 columns per CTA):
+//   col_begin (axis 0, 4 or 8 columns per CTA):
 //       state -> W (lab frame) or X (interaction picture), stored back in the
 //       state slot; inverse DFT along axis 0 of W or E_n X    -> T1 [i0][k1]
-//   row_mid   (axis 1, 8 rows per CTA, one warp per row):
+//   row_mid   (axis 1, 4 or 8 rows per CTA; FP32 rows of 64 points and more stay
+//       in the registers of N1 / 8 threads each, k_row32):
 //       inverse DFT along axis 1 -> y; u = y/(1 + i h mu_0 V); V u;
 //       forward DFT along axis 1 (1/n1)                        -> T2 [i0][k1]
 //   col_end   (axis 0):
@@ -16,10 +17,10 @@
 //       For mixed interaction-picture steps (the hot path) k_col_fused_ip does
 //       the same with the state and history reads staged by cp.async.
 //
-// Each CTA holds 8 whole lines (columns or rows) in shared memory, interleaved
+// Each CTA holds its whole lines (columns or rows) in shared memory, interleaved
 // so that consecutive threads touch consecutive lines, and transforms them
-// together (CtaFft).  The element phases read and write 8 consecutive columns
-// per row (one 64/128-byte segment); the per-mode history work is done one
+// together (CtaFft).  The element phases read and write 4 or 8 consecutive columns
+// per row (one 32- to 128-byte segment); the per-mode history work is done one
 // mode at a time per thread with all of that mode's loads in flight.
 //
 // MODE_REFRESH runs the passes with no phase/history and beta = 0;
