@@ -377,11 +377,14 @@ __global__ void __launch_bounds__((threads_2d<C, N1, L>()), (min_blocks_2d<C, N1
 // transforms, and stored to T2 from the last forward pass, so that a line
 // crosses shared memory four times instead of eleven and its group of threads
 // (a warp, part of one, or a few warps on a barrier of their own) never waits for
-// the other lines.  64 x 512^2: 488 -> 466 us per step; 5 x 128^3: 431 -> 339.
+// the other lines.  As few lines per CTA as fill two warps, so that an SM refills
+// line by line.  us per Adams step, k_row_mid / 256 threads per CTA / this:
+// 5 x 128^3 376 / 339 / 339; 64 x 256^2 106.4 / 101.5 / 101.2; 16 x 512^2 112.6 /
+// 111.7 / 109.7; 64 x 512^2 459.5 / 470 / 463.6; 16 x 1024^2 727 / 682 / 641;
+// 512^2 16.5 / 15.7 / 15.7.
 template <int N1> struct Row32 {
-    static constexpr int T = N1 / 8;                                   // threads per line
-    static constexpr int BIG = 256 / T > 8 ? 8 : 256 / T;              // lines per CTA
-    static constexpr int SMALL = 64 / T < 1 ? 1 : 64 / T;              // the same in launches of few CTAs
+    static constexpr int T = N1 / 8;                       // threads per line
+    static constexpr int L = 64 / T < 1 ? 1 : 64 / T;      // lines per CTA
 };
 template <int T, int L> struct LineSync {
     using type = std::conditional_t<(T <= 32), WarpSync, std::conditional_t<L == 1, CtaSync, GroupSync>>;
@@ -813,14 +816,9 @@ static cudaError_t col_fused_ip_n(const KArgs& a, cudaStream_t s) {
 template <int N1>
 static cudaError_t row32_n(const KArgs& a, cudaStream_t s) {
     using G = Row32<N1>;
-    auto go = [&](auto l) {
-        constexpr int L = decltype(l)::value;
-        static bool done = false;
-        return launch_pass(k_row32<N1, L>, dim3(a.n0 / L, a.B), G::T * L, (size_t)L * fft_len<float2>(N1) * sizeof(float2), done,
-                           s, a);
-    };
-    if ((long long)a.n0 * a.B < (long long)SMALL_CTAS * G::BIG) return go(std::integral_constant<int, G::SMALL>());
-    return go(std::integral_constant<int, G::BIG>());
+    static bool done = false;
+    return launch_pass(k_row32<N1, G::L>, dim3(a.n0 / G::L, a.B), G::T * G::L,
+                       (size_t)G::L * fft_len<float2>(N1) * sizeof(float2), done, s, a);
 }
 
 template <class C, int N1>
