@@ -119,10 +119,12 @@ __global__ void __launch_bounds__(Run1D32<N>::T, Run1D32<N>::MINB) k_run1d32(con
         FI::run(in, mid, buf, tw, twl, tid, sync);
         if constexpr (FI::NPASS == 1) sync();
         // The next step's weights: past the transform's barriers every thread has
-        // left the step before, the last to read their buffer.
+        // left the step before, the last to read their buffer.  The forward
+        // transform's barriers publish them (n = 8 has none: one of its own).
         if (n < last)
             for (int i = tid; i < CL_TAB / 4; i += T)
                 wsm[(n + 1) & 1][i] = __ldg(reinterpret_cast<const float4*>(wtab) + (size_t)(n + 1) * (CL_TAB / 4) + i);
+        if constexpr (FW::NPASS == 1) sync();
         const double vfac = tfac[8 * (size_t)n];
         const float fh = (float)vfac, fl = (float)(vfac - (double)fh);
         const float2* V = V0f + (g.vtable ? (size_t)(8 * g.S_eff + (n - g.S_eff)) * N : 0);
