@@ -662,8 +662,7 @@ static tdse_status set_field(tdse_ctx* c, int instance, tdse_field_fn A, void* u
     if (c->fs) {
         double dphi[3] = {0.0, 0.0, 0.0};
         fs_largest_dphi(c, phi.data(), dphi);
-        const tdse_status st = fs_field_range(c, lo, hi, dphi, s);
-        if (st != TDSE_OK) return st;
+        fs_field_range(c, lo, hi, dphi);
     }
     for (int b = lo; b < hi; ++b) {
         TDSE_CK(c, cudaMemcpyAsync(c->P<double>(c->off.phi) + (size_t)b * c->d * c->ntf, phi.data(),
@@ -690,8 +689,7 @@ tdse_status tdse_set_pulse(tdse_ctx* c, int instance, double A0, double omega, d
     const double d2[3] = {dir[0], c->d >= 2 ? dir[1] : 0.0, c->d == 3 ? dir[2] : 0.0};
     if (c->fs) {
         const double dphi[3] = {A0 * c->cfg.dt * d2[0], A0 * c->cfg.dt * d2[1], A0 * c->cfg.dt * d2[2]};
-        const tdse_status st = fs_field_range(c, lo, hi, dphi, s);
-        if (st != TDSE_OK) return st;
+        fs_field_range(c, lo, hi, dphi);
     }
     for (int b = lo; b < hi; ++b) {
         TDSE_CK(c, launch_pulse_phi(c->P<double>(c->off.phi) + (size_t)b * c->d * c->ntf, c->ntf, c->d,

@@ -157,7 +157,7 @@ inline size_t vrow(const tdse_ctx* c, int tf) {
 tdse_status fs_create(tdse_ctx* c);
 tdse_status fs_bind(tdse_ctx* c, cudaStream_t s);
 tdse_status fs_upload_tables(tdse_ctx* c, cudaStream_t s);
-tdse_status fs_field_range(tdse_ctx* c, int lo, int hi, const double* dphi, cudaStream_t s);
+void fs_field_range(tdse_ctx* c, int lo, int hi, const double* dphi);
 tdse_status fs_loaded_field_range(tdse_ctx* c, const char* flags, cudaStream_t s);
 void fs_largest_dphi(const tdse_ctx* c, const double* phi, double* dphi);
 tdse_status fs_build_phase_tables(tdse_ctx* c, int b, cudaStream_t s);

@@ -7,8 +7,11 @@ namespace {
 
 // P[iv][m] = exp(-i zeta_m^2 s + i zeta_m (phi(t1) - phi(t0))), s = t1 - t0
 // (eq. uhatxirecur with zeta for k), one instance.
-__global__ void k_fs_phase(int4* P, float2* Pf, double scale, const double2* zeta, int N, const int2* iv, int n_int, const double* phi,
-                           double dt8) {
+// The scale goes to the device with the tables, so that a captured launch leaves
+// both or neither as it found them.
+__global__ void k_fs_phase(int4* P, float2* Pf, int* g_out, int g, double scale, const double2* zeta, int N, const int2* iv,
+                           int n_int, const double* phi, double dt8) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *g_out = g;
     for (int it = blockIdx.y; it < n_int; it += gridDim.y) {
         const int2 q = iv[it];
         const double s = (double)(q.y - q.x) * dt8;
@@ -117,11 +120,11 @@ cudaError_t launch_fs_phys(const FsArgs& a, int from_usrc, int f32, cudaStream_t
 }
 cudaError_t launch_fs_mid(const FsArgs& a, int dir, int f32, cudaStream_t s) { return run(a, 3, dir, f32, s); }
 
-cudaError_t launch_fs_phase(int4* P, float2* Pf, int g, const double2* zeta, int N, const int2* intervals, int n_int,
+cudaError_t launch_fs_phase(int4* P, float2* Pf, int* g_out, int g, const double2* zeta, int N, const int2* intervals, int n_int,
                             const double* phi, double dt, cudaStream_t s) {
     if (n_int <= 0) return cudaSuccess;
     const unsigned gy = n_int < 65535 ? (unsigned)n_int : 65535u;
-    k_fs_phase<<<dim3((N + 255) / 256, gy), 256, 0, s>>>(P, Pf, ldexp(1.0, -(1 + g)), zeta, N, intervals, n_int, phi,
+    k_fs_phase<<<dim3((N + 255) / 256, gy), 256, 0, s>>>(P, Pf, g_out, g, ldexp(1.0, -(1 + g)), zeta, N, intervals, n_int, phi,
                                                             dt / 8.0);
     return cudaGetLastError();
 }

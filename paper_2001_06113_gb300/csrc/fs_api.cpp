@@ -783,16 +783,14 @@ tdse_status fs_bind(tdse_ctx* c, cudaStream_t s) {
 // The one-step phase of an axis has modulus at most e^{H |dphi|}; over the
 // history and all axes at most e^{7 H sum |dphi|}.  Its fixed-point factors
 // hold moduli below 2^(1 + g): g of instances [lo, hi) for a field that changes
-// by at most dphi per step (their phase tables are built after this).
-tdse_status fs_field_range(tdse_ctx* c, int lo, int hi, const double* dphi, cudaStream_t s) {
+// by at most dphi per step (their phase tables are built after this, and take g
+// to the device).
+void fs_field_range(tdse_ctx* c, int lo, int hi, const double* dphi) {
     FsState& F = c->F;
     double growth = 0.0;
     for (int x = 0; x < c->d; ++x) growth += 7.0 * F.ax[x].H * std::fabs(dphi[x]);
     const int g = std::max(0, (int)std::ceil(std::min(growth / M_LN2, 25.0) - 1.0));
     for (int b = lo; b < hi; ++b) F.g[b] = g;
-    TDSE_CK(c, cudaMemcpyAsync(c->P<int>(F.off.g) + lo, F.g.data() + lo, (size_t)(hi - lo) * sizeof(int),
-                               cudaMemcpyHostToDevice, s));    // pageable: taken before the call returns
-    return TDSE_OK;
 }
 
 // Largest change of phi per step and axis (the sum of the |changes| of its
@@ -823,11 +821,9 @@ tdse_status fs_loaded_field_range(tdse_ctx* c, const char* flags, cudaStream_t s
             TDSE_CK(c, cudaStreamSynchronize(s));
             fs_largest_dphi(c, phi.data(), dphi);
         }
-        const tdse_status st = fs_field_range(c, b, b + 1, dphi, s);
-        if (st != TDSE_OK) return st;
+        fs_field_range(c, b, b + 1, dphi);
         if (g) F.g[b] = g - 1;
     }
-    TDSE_CK(c, cudaMemcpyAsync(c->P<int>(F.off.g), F.g.data(), (size_t)c->B * sizeof(int), cudaMemcpyHostToDevice, s));
     return TDSE_OK;
 }
 
@@ -838,8 +834,8 @@ tdse_status fs_build_phase_tables(tdse_ctx* c, int b, cudaStream_t s) {
         const FsAxisHost& A = F.ax[x];
         const size_t at = (size_t)b * c->n_int * A.N;
         const double* phi = c->P<double>(F.off.phi) + ((size_t)b * c->d + x) * c->ntf;
-        TDSE_CK(c, launch_fs_phase(c->P<int4>(F.off.P[x]) + at, F.f32 ? c->P<float2>(F.off.P_f[x]) + at : nullptr, F.g[b],
-                                   c->P<double2>(F.off.zeta[x]), A.N, iv, c->n_int, phi, c->cfg.dt, s));
+        TDSE_CK(c, launch_fs_phase(c->P<int4>(F.off.P[x]) + at, F.f32 ? c->P<float2>(F.off.P_f[x]) + at : nullptr,
+                                   c->P<int>(F.off.g) + b, F.g[b], c->P<double2>(F.off.zeta[x]), A.N, iv, c->n_int, phi, c->cfg.dt, s));
     }
     return TDSE_OK;
 }

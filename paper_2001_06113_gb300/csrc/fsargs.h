@@ -147,9 +147,9 @@ cudaError_t launch_fs_res_decide(const double* sums, int B, double hm0, double t
 cudaError_t launch_fs_res_apply(const int* flags, int B, size_t NM, size_t NX, double2* uhat, const double2* Wc,
                                 float2* ring, size_t rstride, const double2* R64, double2* u, const double2* u64,
                                 cudaStream_t s);
-// P[iv][m] of one instance and axis (times 2^-(1 + g); and in FP32, unscaled, if
-// Pf): zeta [N] complex, phi_axis [ntf] = that component of phi at t = m dt / 8.
-cudaError_t launch_fs_phase(int4* P, float2* Pf, int g, const double2* zeta, int N, const int2* intervals, int n_int,
+// P[iv][m] of one instance and axis (times 2^-(1 + g), g to *g_out; and in FP32,
+// unscaled, if Pf): zeta [N] complex, phi_axis [ntf] = that component of phi at t = m dt / 8.
+cudaError_t launch_fs_phase(int4* P, float2* Pf, int* g_out, int g, const double2* zeta, int N, const int2* intervals, int n_int,
                             const double* phi_axis, double dt, cudaStream_t s);
 
 }  // namespace tdse
