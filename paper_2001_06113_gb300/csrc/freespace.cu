@@ -23,7 +23,8 @@ __global__ void k_fs_phase(int4* P, float2* Pf, int* g_out, int g, double scale,
             double sn, cs;
             sincos(im, &sn, &cs);
             const double e = exp(re);
-            P[(size_t)it * N + m] = fx_factor(scale * (e * cs), scale * (e * sn));
+            if (g < FS_WIDE) P[(size_t)it * N + m] = fx_factor(scale * (e * cs), scale * (e * sn));
+            else reinterpret_cast<double2*>(P)[(size_t)it * N + m] = make_double2(e * cs, e * sn);
             if (Pf) Pf[(size_t)it * N + m] = make_float2((float)(e * cs), (float)(e * sn));
         }
     }

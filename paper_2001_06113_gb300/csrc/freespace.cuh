@@ -538,13 +538,28 @@ struct Line {
 // ---------------------------------------------------------------- mode update
 // One-step phases are factors in units of 2^-(60 - g) (|p| < 2^(1 + g); g of the
 // instance, 0 unless its field moves the contour phases by more than a factor
-// of 2 over the history, see fs_api.cpp).
+// of 2 over the history, see fs_api.cpp); from g = FS_WIDE on they and the history
+// sum are FP64 (WIDE below).  A CTA takes one form or the other for the whole of
+// its modes, the FP64 one in functions of their own: a branch per mode cost the
+// fixed-point form 0.4 to 2.8 %.
 __device__ __forceinline__ longlong2 pmul(longlong2 v, int4 p, int g) {
     longlong2 r = fx_mul<false, 4>(v, p);
     if (g) r = make_longlong2((long long)((unsigned long long)r.x << g), (long long)((unsigned long long)r.y << g));
     return r;
 }
-__device__ __forceinline__ int4 pmul(int4 a, int4 b, int g) { return fx_as_factor(pmul(fx_value(a), b, g)); }
+__device__ __forceinline__ double2 wide_phase(int4 p) {
+    return make_double2(__hiloint2double(p.y, p.x), __hiloint2double(p.w, p.z));
+}
+__device__ __forceinline__ int4 wide_bits(double2 v) {
+    return make_int4(__double2loint(v.x), __double2hiint(v.x), __double2loint(v.y), __double2hiint(v.y));
+}
+template <bool WIDE> __device__ __forceinline__ int4 phase_one(int g) {
+    return WIDE ? wide_bits(make_double2(1.0, 0.0)) : make_int4(1 << (28 - g), 0, 0, 0);
+}
+template <bool WIDE> __device__ __forceinline__ int4 phase_mul(int4 a, int4 b, int g) {
+    if constexpr (WIDE) return wide_bits(cmul(wide_phase(a), wide_phase(b)));
+    else return fx_as_factor(pmul(fx_value(a), b, g));
+}
 
 __device__ __forceinline__ float2 to_c(double2 v, float2) { return make_float2(fx_to_float(v.x), fx_to_float(v.y)); }
 __device__ __forceinline__ double2 to_c(double2 v, double2) { return v; }
@@ -579,7 +594,8 @@ template <class N> struct RowPtr {
 // History sum of eq. uadamsk in Horner form with separable phases p_i = a_i b_i
 // (a_i of the row, b_i of the mode; 1D: a_i = 1):  S_j = c_j R_j + b_j S_{j+1},
 // c_j = mu_j a_1 .. a_{j-1}, so that S_1 = sum_j mu_j p_1 .. p_{j-1} R_j.
-// F32: in FP32; F64: in fixed point, the R_j sharing an exponent.
+// F32: in FP32; F64: in fixed point, the R_j sharing an exponent (WIDE: in FP64).
+template <bool WIDE>
 __device__ __forceinline__ float2 history(const FsArgs& a, int g, const int4* c, const float2 (&r)[FS_MAX_HIST],
                                           const float2* const (&pc)[FS_MAX_HIST], int m) {
     float2 S = make_float2(0.f, 0.f);
@@ -594,8 +610,20 @@ __device__ __forceinline__ float2 history(const FsArgs& a, int g, const int4* c,
     }
     return S;
 }
+template <bool WIDE>
 __device__ __forceinline__ double2 history(const FsArgs& a, int g, const int4* c, const double2 (&r)[FS_MAX_HIST],
                                            const int4* const (&pc)[FS_MAX_HIST], int m) {
+    if constexpr (WIDE) {
+        double2 S = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int j = FS_MAX_HIST; j >= 1; --j) {
+            if (j <= a.nhist) {
+                if (j < FS_MAX_HIST && j < a.nhist) S = cmul(S, wide_phase(__ldg(pc[j] + m)));
+                S = S + cmul(wide_phase(c[j]), r[j - 1]);
+            }
+        }
+        return S;
+    } else {
     unsigned mr = 0;
 #pragma unroll
     for (int j = 0; j < FS_MAX_HIST; ++j) mr = max(mr, fx_hi(r[j]));
@@ -609,6 +637,7 @@ __device__ __forceinline__ double2 history(const FsArgs& a, int g, const int4* c
         }
     }
     return fx_to(S, mr >= 0x7ff00000u ? FX_NAN : E - 1022 - S0);
+    }
 }
 
 template <> struct PhaseTab<NumF32> {
@@ -623,11 +652,11 @@ template <> struct PhaseTab<NumF64> {
 // Row factors of a begin, by the last warp of the CTA into sm.c (the caller's
 // next barrier publishes them): c[0] = a_0, c[j] = mu_j a_1 .. a_{j-1}; phase(i)
 // is the row's factor a_i.  Lane i holds a_i, a scan over the lanes the products.
-template <class N, class Sm, class Ph>
+template <class N, bool WIDE, class Sm, class Ph>
 __device__ __forceinline__ void row_factors(const FsArgs& a, int g, Sm& sm, int T, Ph phase) {
     const int lane = (int)threadIdx.x - (T - 32);
     if (lane < 0) return;
-    const int4 one = make_int4(1 << (28 - g), 0, 0, 0);
+    const int4 one = phase_one<WIDE>(g);
     const int nh = min(a.nhist, FS_MAX_HIST);
     int4 A = lane == 0 || lane < nh ? phase(lane) : one;
     if (lane == 0) {
@@ -638,16 +667,19 @@ __device__ __forceinline__ void row_factors(const FsArgs& a, int g, Sm& sm, int 
     for (int o = 1; o < 8; o <<= 1) {
         const int4 B = make_int4(__shfl_up_sync(0xffffffffu, A.x, o), __shfl_up_sync(0xffffffffu, A.y, o),
                                  __shfl_up_sync(0xffffffffu, A.z, o), __shfl_up_sync(0xffffffffu, A.w, o));
-        const int4 P = pmul(A, B, g);
+        const int4 P = phase_mul<WIDE>(A, B, g);
         if (lane >= o) A = P;
     }
     const int j = lane + 1;                            // A = a_1 .. a_{j-1}
     if (j > nh) return;
     const longlong2 v = fx_value(A);
     if constexpr (N::FX) {
-        sm.c[j] = fx_as_factor(make_longlong2(fx_mul_real<4>(v.x, a.mu_w[j]), fx_mul_real<4>(v.y, a.mu_w[j])));
+        if constexpr (WIDE) sm.c[j] = wide_bits(cscale(wide_phase(A), a.mu[j]));
+        else sm.c[j] = fx_as_factor(make_longlong2(fx_mul_real<4>(v.x, a.mu_w[j]), fx_mul_real<4>(v.y, a.mu_w[j])));
     } else {
-        const double2 d = fx_to(v, g - 60);
+        double2 d;
+        if constexpr (WIDE) d = wide_phase(A);
+        else d = fx_to(v, g - 60);
         sm.c[j] = make_int4(__float_as_int((float)(a.mu[j] * d.x)), __float_as_int((float)(a.mu[j] * d.y)), 0, 0);
     }
 }
@@ -675,7 +707,7 @@ __device__ __forceinline__ RowPtr<N> row_ptr(const FsArgs& a, bool end, const do
 // mu_0 F and u^ - i h S are FP64 fused multiply-adds (4 of them: their 256
 // cycles of the FP64 pipe run beside the integer work of other warps), the
 // phase product p_0 X, 8 more in FP64, is done in fixed point.
-template <class N>
+template <class N, bool WIDE>
 __device__ __forceinline__ double2 update_mode(const FsArgs& a, int g, const int4* c, bool end, bool begin, int m,
                                                typename N::C F, const RowPtr<N>& p) {
     using C = typename N::C;
@@ -697,11 +729,16 @@ __device__ __forceinline__ double2 update_mode(const FsArgs& a, int g, const int
         }
         if (p.first_is_new) r[0] = F;
     }
-    const double2 X = add_minus_i(u, a.h, widen(history(a, g, c, r, p.pc, m)));
-    const unsigned mx = fx_hi(X);
-    const int E = fx_exponent(mx);
-    const longlong2 v = pmul(pmul(fx_from(X, 59, E), c[0], g), b0, g);
-    const double2 W = fx_to(v, mx >= 0x7ff00000u ? FX_NAN : E - 1022 - 59);
+    const double2 X = add_minus_i(u, a.h, widen(history<WIDE>(a, g, c, r, p.pc, m)));
+    double2 W;
+    if constexpr (!WIDE) {
+        const unsigned mx = fx_hi(X);
+        const int E = fx_exponent(mx);
+        const longlong2 v = pmul(pmul(fx_from(X, 59, E), c[0], g), b0, g);
+        W = fx_to(v, mx >= 0x7ff00000u ? FX_NAN : E - 1022 - 59);
+    } else {
+        W = cmul(cmul(X, wide_phase(c[0])), wide_phase(b0));
+    }
     p.uh[m] = W;
     return W;
 }
@@ -751,6 +788,75 @@ __device__ __forceinline__ void each_mode(const FsAxis& ax, typename Ln::Sm& sm,
     }
 }
 
+// What locates the modes of a row (row_ptr's arguments).
+template <class N> struct RowArgs {
+    const double2* src;
+    double2* uh;
+    typename N::C* ring;
+    size_t slot_stride;
+    const int4* P;
+    const typename PhaseTab<N>::type* Pc;
+};
+
+// Every mode of this thread through update_mode (end and / or begin); returns
+// the largest fx_hi of its inputs of the inverse transform (FP64).
+template <class N, class Ln, bool WIDE>
+__device__ __forceinline__ unsigned update_modes(const FsArgs& a, const FsAxis& ax, typename Ln::Sm& sm, int g, bool end,
+                                                 bool begin, int xe, const RowArgs<N>& r) {
+    using C = typename N::C;
+    const RowPtr<N> p = row_ptr<N>(a, end, r.src, r.uh, r.ring, r.slot_stride, r.P, r.Pc, ax.N);
+    unsigned mx = 0;
+    each_mode<N, Ln>(ax, sm, end, xe, [&](int m, C F, C* at) {
+        const double2 W = update_mode<N, WIDE>(a, g, sm.c, end, begin, m, F, p);
+        if (begin) {
+            *at = to_c(W, C());
+            if constexpr (N::FX) mx = max(mx, fx_hi(*at));
+        }
+    });
+    return mx;
+}
+// Row k0 of instance b along the last axis (1D: the only row).
+template <class N> __device__ __forceinline__ RowArgs<N> row_args(const FsArgs& a, int b, int k0) {
+    const int d = a.d, Nl = a.ax[d - 1].N;
+    const size_t nrows = d == 1 ? 1 : (d == 2 ? (size_t)a.ax[0].N : (size_t)a.ax[0].N * a.ax[1].N);
+    const size_t NPm = nrows * Nl, at = (size_t)b * NPm + (size_t)k0 * Nl, ph = (size_t)b * a.n_int * Nl;
+    RowArgs<N> r;
+    r.uh = a.uhat + at;
+    r.src = a.uhat_src ? a.uhat_src + at : r.uh;
+    r.ring = reinterpret_cast<typename N::C*>(a.ring) + (size_t)b * a.ring_slots * NPm + (size_t)k0 * Nl;
+    r.slot_stride = NPm;
+    r.P = a.ax[d - 1].P + ph;
+    r.Pc = PhaseTab<N>::get(a.ax[d - 1]) + ph;
+    return r;
+}
+// (Few arguments: what the call keeps alive counts against the registers of the
+// fixed-point form.)
+template <class N, class Ln>
+__device__ __noinline__ unsigned update_modes_wide(const FsArgs& a, int flags, int xe) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    const int b = a.d == 1 ? blockIdx.x : blockIdx.y, k0 = a.d == 1 ? 0 : blockIdx.x;
+    return update_modes<N, Ln, true>(a, a.ax[a.d - 1], *reinterpret_cast<typename Ln::Sm*>(sm_raw), FS_WIDE, flags & FS_ROW_END,
+                                     flags & FS_ROW_BEGIN, xe, row_args<N>(a, b, k0));
+}
+
+// Row factor a_i of interval a.interval[i] of row k0 (1D: 1): P0 (2D), P0 P1 of axes 0 and 1 (3D).
+template <bool WIDE> __device__ __forceinline__ int4 row_phase(const FsArgs& a, int g, int b, int k0, int i) {
+    if (a.d == 1) return phase_one<WIDE>(g);
+    const int iv = a.interval[i], N0 = a.ax[0].N;
+    const int4* P0 = a.ax[0].P + (size_t)b * a.n_int * N0;
+    if (a.d == 2) return __ldg(&P0[(size_t)iv * N0 + k0]);
+    const int NA = a.ax[1].N, i0 = k0 / NA, i1 = k0 - i0 * NA;
+    const int4* PA = a.ax[1].P + (size_t)b * a.n_int * NA;
+    return phase_mul<WIDE>(__ldg(&P0[(size_t)iv * N0 + i0]), __ldg(&PA[(size_t)iv * NA + i1]), g);
+}
+template <class N, class Ln>
+__device__ __noinline__ void row_factors_wide(const FsArgs& a) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    const int b = a.d == 1 ? blockIdx.x : blockIdx.y, k0 = a.d == 1 ? 0 : blockIdx.x;
+    row_factors<N, true>(a, FS_WIDE, *reinterpret_cast<typename Ln::Sm*>(sm_raw), Ln::G::T,
+                         [&](int i) { return row_phase<true>(a, FS_WIDE, b, k0, i); });
+}
+
 template <class N, int M, int R>
 __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) k_fs_1d(const __grid_constant__ FsArgs a, int mode) {
     using Ln = Line<N, M, R>;
@@ -780,18 +886,12 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
         each_mode<N, Ln>(ax, sm, true, xe, [&](int m, C F, C*) { store_fwd(a, (size_t)b * a.fdst_bstride + m, F); });
         return;
     }
-    double2* uh = a.uhat + (size_t)b * Nm;
-    C* ring = reinterpret_cast<C*>(a.ring) + (size_t)b * a.ring_slots * Nm;
-    const int4* P = ax.P + (size_t)b * a.n_int * Nm;
-    const auto* Pc = PhaseTab<N>::get(ax) + (size_t)b * a.n_int * Nm;
-    row_factors<N>(a, g, sm, G::T, [&](int) { return make_int4(1 << (28 - g), 0, 0, 0); });    // 1
+    if (g < FS_WIDE) row_factors<N, false>(a, g, sm, G::T, [&](int) { return phase_one<false>(g); });
+    else row_factors_wide<N, Ln>(a);
     __syncthreads();
-    unsigned mx = 0;
-    const RowPtr<N> rp = row_ptr<N>(a, false, uh, uh, ring, (size_t)Nm, P, Pc, Nm);
-    each_mode<N, Ln>(ax, sm, false, 0, [&](int m, C F, C* at) {
-        *at = to_c(update_mode<N>(a, g, sm.c, false, true, m, F, rp), C());
-        if constexpr (N::FX) mx = max(mx, fx_hi(*at));
-    });
+    const RowArgs<N> rp = row_args<N>(a, b, 0);
+    const unsigned mx = g < FS_WIDE ? update_modes<N, Ln, false>(a, ax, sm, g, false, true, 0, rp)
+                                    : update_modes_wide<N, Ln>(a, FS_ROW_BEGIN, 0);
     C y[G::FPT];
     Ln::inverse(sm, mx, y, ax);
     const double hm0 = a.h * a.mu[0];
@@ -809,9 +909,7 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
     __syncthreads();                 // every thread has read its y
     const auto E = Ln::put_grid(f, sm, ax);
     Ln::forward(sm, ax, E, xe);
-    each_mode<N, Ln>(ax, sm, true, xe, [&](int m, C F, C*) {
-        update_mode<N>(a, g, sm.c, true, false, m, F, rp);
-    });
+    update_modes<N, Ln, false>(a, ax, sm, g, true, false, xe, rp);      // (no phases)
 }
 
 template <class N, int M, int R>
@@ -826,31 +924,22 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
     const int k0 = blockIdx.x, b = blockIdx.y;           // k0: the row (k0 N1 + k1 in 3D)
     const int N0 = a.ax[0].N, N1 = ax.N, g = __ldg(&a.g[b]);
     const int nrows = d3 ? N0 * a.ax[1].N : N0;
-    const size_t NPm = (size_t)nrows * N1;
-    double2* urow = a.uhat + (size_t)b * NPm + (size_t)k0 * N1;
-    const double2* usrc = a.uhat_src ? a.uhat_src + (size_t)b * NPm + (size_t)k0 * N1 : urow;
+    const RowArgs<N> rp = row_args<N>(a, b, k0);
     C* zrow = reinterpret_cast<C*>(a.Z) + ((size_t)b * nrows + k0) * M;
     const bool end = flags & FS_ROW_END, begin = flags & FS_ROW_BEGIN;
-    if (begin) {   // phase of the row over interval iv: P0 (2D), P0 P1 of axes 0 and 1 (3D)
-        const int4* P0 = a.ax[0].P + (size_t)b * a.n_int * N0;
-        row_factors<N>(a, g, sm, G::T, [&](int i) -> int4 {
-            const int iv = a.interval[i];
-            if (!d3) return __ldg(&P0[(size_t)iv * N0 + k0]);
-            const int NA = a.ax[1].N, i0 = k0 / NA, i1 = k0 - i0 * NA;
-            const int4* PA = a.ax[1].P + (size_t)b * a.n_int * NA;
-            return pmul(__ldg(&P0[(size_t)iv * N0 + i0]), __ldg(&PA[(size_t)iv * NA + i1]), g);
-        });
+    if (begin) {
+        if (g < FS_WIDE) row_factors<N, false>(a, g, sm, G::T, [&](int i) { return row_phase<false>(a, g, b, k0, i); });
+        else row_factors_wide<N, Ln>(a);
     }
     // the row's state and history on their way to the L2 while the transform runs
     if (begin) {
-        const C* ring0 = reinterpret_cast<const C*>(a.ring) + (size_t)b * a.ring_slots * NPm + (size_t)k0 * N1;
         for (int off = (int)threadIdx.x * 128; off < N1 * 16; off += G::T * 128) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(usrc) + off));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(rp.src) + off));
             if (off < N1 * (int)sizeof(C))
                 for (int j = 0; j < a.nhist; ++j)
                     if (!(end && a.hist_slot[j] == a.out_slot))
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(
-                            reinterpret_cast<const char*>(ring0 + (size_t)a.hist_slot[j] * NPm) + off));
+                            reinterpret_cast<const char*>(rp.ring + (size_t)a.hist_slot[j] * rp.slot_stride) + off));
         }
     }
     int xe = 0;
@@ -871,18 +960,8 @@ __global__ void __launch_bounds__((Geo<M, R>::T), (min_blocks<N, Geo<M, R>>())) 
     } else {
         __syncthreads();             // sm.c
     }
-    const int4* P1 = ax.P + (size_t)b * a.n_int * N1;
-    const auto* P1c = PhaseTab<N>::get(ax) + (size_t)b * a.n_int * N1;
-    C* ring = reinterpret_cast<C*>(a.ring) + (size_t)b * a.ring_slots * NPm + (size_t)k0 * N1;
-    unsigned mx = 0;
-    const RowPtr<N> rp = row_ptr<N>(a, end, usrc, urow, ring, NPm, P1, P1c, N1);
-    each_mode<N, Ln>(ax, sm, end, xe, [&](int m, C F, C* at) {
-        const double2 W = update_mode<N>(a, g, sm.c, end, begin, m, F, rp);
-        if (begin) {
-            *at = to_c(W, C());
-            if constexpr (N::FX) mx = max(mx, fx_hi(*at));
-        }
-    });
+    const unsigned mx = g < FS_WIDE ? update_modes<N, Ln, false>(a, ax, sm, g, end, begin, xe, rp)
+                                    : update_modes_wide<N, Ln>(a, flags, xe);
     if (!begin) return;
     C y[G::FPT];
     Ln::inverse(sm, mx, y, ax);

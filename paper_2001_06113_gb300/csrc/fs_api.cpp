@@ -782,14 +782,15 @@ tdse_status fs_bind(tdse_ctx* c, cudaStream_t s) {
 
 // The one-step phase of an axis has modulus at most e^{H |dphi|}; over the
 // history and all axes at most e^{7 H sum |dphi|}.  Its fixed-point factors
-// hold moduli below 2^(1 + g): g of instances [lo, hi) for a field that changes
+// hold moduli below 2^(1 + g), g < FS_WIDE; beyond that it is held in FP64: g of instances [lo, hi) for a field that changes
 // by at most dphi per step (their phase tables are built after this, and take g
 // to the device).
 void fs_field_range(tdse_ctx* c, int lo, int hi, const double* dphi) {
     FsState& F = c->F;
     double growth = 0.0;
     for (int x = 0; x < c->d; ++x) growth += 7.0 * F.ax[x].H * std::fabs(dphi[x]);
-    const int g = std::max(0, (int)std::ceil(std::min(growth / M_LN2, 25.0) - 1.0));
+    const double x = growth / M_LN2 - 1.0;
+    const int g = x <= FS_WIDE - 1 ? std::max(0, (int)std::ceil(x)) : FS_WIDE;      // (a NaN: FS_WIDE)
     for (int b = lo; b < hi; ++b) F.g[b] = g;
 }
 
@@ -822,7 +823,7 @@ tdse_status fs_loaded_field_range(tdse_ctx* c, const char* flags, cudaStream_t s
             fs_largest_dphi(c, phi.data(), dphi);
         }
         fs_field_range(c, b, b + 1, dphi);
-        if (g) F.g[b] = g - 1;
+        if (g) F.g[b] = std::min(g - 1, FS_WIDE);
     }
     return TDSE_OK;
 }

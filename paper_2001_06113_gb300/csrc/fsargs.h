@@ -27,6 +27,10 @@ namespace tdse {
 constexpr int FS_MAX_ND = 128;    // dense (Alpert + Gauss) modes per axis
 constexpr int FS_MAX_HIST = 7;
 constexpr int FS_MAX_NT = 64;     // terms of the Chebyshev interpolant of the C-type transforms
+// From this scale on (FsArgs::g) an instance's phases are FP64 values: every unit
+// of g takes a bit of the 58 that the fixed-point history sum holds, and below
+// 53 it would hold less than an FP64 sum.
+constexpr int FS_WIDE = 5;
 
 struct FsAxis {
     int M;        // physical points
@@ -51,6 +55,7 @@ struct FsAxis {
     const int4* Fd;     // [ND][M]    forward dense: (2/M) e^{-i zeta_d x_j}
     const int4* tw;        // [M]        e^{-2 pi i m / M}, fixed-point factors (fx.cuh)
     const int4* P;      // [B][n_int][N] one-step phases e^{-i zeta^2 s + i zeta (phi(t1) - phi(t0))}
+                        // (instances of g >= FS_WIDE: FP64 pairs in place of the factors, unscaled)
     // FP32 copies for the FP32-transform variant (TDSE_MIXED), same layouts
     const float2* preI_f;
     const float2* postI_f;
@@ -147,8 +152,8 @@ cudaError_t launch_fs_res_decide(const double* sums, int B, double hm0, double t
 cudaError_t launch_fs_res_apply(const int* flags, int B, size_t NM, size_t NX, double2* uhat, const double2* Wc,
                                 float2* ring, size_t rstride, const double2* R64, double2* u, const double2* u64,
                                 cudaStream_t s);
-// P[iv][m] of one instance and axis (times 2^-(1 + g), g to *g_out; and in FP32,
-// unscaled, if Pf): zeta [N] complex, phi_axis [ntf] = that component of phi at t = m dt / 8.
+// P[iv][m] of one instance and axis (g < FS_WIDE: factors, times 2^-(1 + g), else
+// FP64 pairs; g to *g_out; and in FP32, unscaled, if Pf): zeta [N] complex, phi_axis [ntf] = that component of phi at t = m dt / 8.
 cudaError_t launch_fs_phase(int4* P, float2* Pf, int* g_out, int g, const double2* zeta, int N, const int2* intervals, int n_int,
                             const double* phi_axis, double dt, cudaStream_t s);
 
