@@ -417,11 +417,54 @@ struct FxPass {
         }
         dft_r<R, INV>(v);
     }
+    // A pass divides by its radix whether or not its sums grew: an input in few
+    // places (a smooth state's modes on a fine grid, a narrow state) would lose
+    // log2(N / radix(0)) of its 59 bits.  Up to N = 1024 what is left is no less than
+    // FP64 gives; longer lines are scaled up before each middle pass by what their
+    // largest component leaves free (2^s, taken off the results' exponent).
+    static constexpr bool rescales(int S) { return N >= 2048 && S > 0 && S < Plan::NPASS - 1; }
+    FX_HD static unsigned magnitude(longlong2 v) {
+        const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
+        const unsigned a = (unsigned)(x ^ (x >> 31)), b = (unsigned)(y ^ (y >> 31));
+        return a > b ? a : b;
+    }
+    FX_HD static int headroom(unsigned mag) {       // components below 2^62 after v 2^s
+#ifdef __CUDA_ARCH__
+        const int z = __clz((int)mag);
+#else
+        const int z = mag ? __builtin_clz(mag) : 32;
+#endif
+        return z > 2 ? z - 2 : 0;
+    }
+    FX_HD static longlong2 up(longlong2 v, int s) {
+        return make_longlong2((long long)((unsigned long long)v.x << s), (long long)((unsigned long long)v.y << s));
+    }
     // exponent of the results for block exponent E (of the largest high word mx)
     FX_HD static int out_exp(unsigned mx, int E, int lg) {
         return mx >= 0x7ff00000u ? FX_NAN : E - 1022 - S0 + GAIN + lg;
     }
 };
+
+// v 2^s for the block's common headroom s, which is returned; with the barrier that a
+// pass needs between its loads and its stores.
+template <class Fx, int T, int PER, int R, class Sync>
+__device__ __forceinline__ int fx_rescale(longlong2 (&v)[PER][R], const Sync& sync) {
+    __shared__ unsigned mx[T / 32];
+    unsigned m = 0;
+#pragma unroll
+    for (int p = 0; p < PER; ++p)
+#pragma unroll
+        for (int r = 0; r < R; ++r) m = max(m, Fx::magnitude(v[p][r]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) mx[threadIdx.x >> 5] = m;
+    sync();
+    const int s = Fx::headroom(__reduce_max_sync(0xffffffffu, mx[(threadIdx.x & 31) % (T / 32)]));
+#pragma unroll
+    for (int p = 0; p < PER; ++p)
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[p][r] = Fx::up(v[p][r], s);
+    return s;
+}
 
 template <int N, int L, int LS, int T, bool INV>
 struct CtaFft<double2, N, L, LS, T, INV> {
@@ -440,7 +483,12 @@ struct CtaFft<double2, N, L, LS, T, INV> {
                     for (int r = 0; r < R; ++r) v[p][r] = buf[(it / L + r * NB) * LS + it % L];
                 }
             }
-            __syncthreads();
+            if constexpr (Fx::rescales(S)) {
+                static_assert(ITEMS % T == 0, "every value is set");
+                X -= fx_rescale<Fx, T>(v, CtaSync{});
+            } else {
+                __syncthreads();
+            }
             store<S, PER, R, Ns>(buf, tw, v, X);
             __syncthreads();
             pass<S + 1>(buf, tw, X);
@@ -509,8 +557,9 @@ struct Fft<double2, N, L, PS, T, INV> : FftShape<N, L, T, INV> {
     using Shape::RF;
     using Shape::RL;
 
+    // (returns the power of two by which the values were scaled up on the way)
     template <int S, class Sync>
-    __device__ static __forceinline__ void mids(longlong2* buf, const int4* __restrict__ tw, int tid, const Sync& sync) {
+    __device__ static __forceinline__ int mids(longlong2* buf, const int4* __restrict__ tw, int tid, const Sync& sync) {
         if constexpr (S <= NPASS - 2) {
             constexpr int R = Plan::radix(S), Ns = Plan::ns(S), NB = N / R, PER = (NB * L + T - 1) / T;
             longlong2 v[PER][R];
@@ -522,7 +571,13 @@ struct Fft<double2, N, L, PS, T, INV> : FftShape<N, L, T, INV> {
                     for (int r = 0; r < R; ++r) v[p][r] = buf[(j + r * NB) * PS + line];
                 }
             }
-            sync();
+            int s = 0;
+            if constexpr (Fx::rescales(S)) {
+                static_assert(NB * L % T == 0, "every value is set");
+                s = fx_rescale<Fx, T>(v, sync);
+            } else {
+                sync();
+            }
 #pragma unroll
             for (int p = 0; p < PER; ++p) {
                 int j, line;
@@ -534,8 +589,9 @@ struct Fft<double2, N, L, PS, T, INV> : FftShape<N, L, T, INV> {
                 }
             }
             sync();
-            mids<S + 1>(buf, tw, tid, sync);
+            return s + mids<S + 1>(buf, tw, tid, sync);
         }
+        return 0;
     }
     // Block exponent of a transform from this thread's largest high word; every
     // thread of the group calls it.
@@ -561,9 +617,9 @@ struct Fft<double2, N, L, PS, T, INV> : FftShape<N, L, T, INV> {
     }
     template <class Sync>
     __device__ static __forceinline__ void middle(double2* buf, const int4* __restrict__ tw, const int4*, int tid,
-                                                  const Sync& sync) {
+                                                  const Sync& sync, Scale& sc) {
         sync();
-        mids<1>(reinterpret_cast<longlong2*>(buf), tw, tid, sync);
+        sc.X -= mids<1>(reinterpret_cast<longlong2*>(buf), tw, tid, sync);
     }
     __device__ static __forceinline__ bool last_item(int p, double2 (&x)[RL], const double2* dbuf,
                                                      const int4* __restrict__ tw, const int4*, int tid, int& j,
@@ -595,7 +651,7 @@ struct Fft<double2, N, L, PS, T, INV> : FftShape<N, L, T, INV> {
                 for (int r = 0; r < RF; ++r) mx = max(mx, fx_hi(in[p][r]));
             }
         }
-        const Scale sc = scale_of(mx, lg);
+        Scale sc = scale_of(mx, lg);
         if constexpr (NPASS == 1) {
 #pragma unroll
             for (int p = 0; p < PF; ++p) {
@@ -609,7 +665,7 @@ struct Fft<double2, N, L, PS, T, INV> : FftShape<N, L, T, INV> {
         } else {
 #pragma unroll
             for (int p = 0; p < PF; ++p) first_item(p, in[p], buf, tid, sc);
-            middle(buf, tw, twl, tid, sync);
+            middle(buf, tw, twl, tid, sync, sc);
 #pragma unroll
             for (int p = 0; p < PL; ++p) {
                 int j;

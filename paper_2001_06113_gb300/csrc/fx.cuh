@@ -15,11 +15,13 @@
 // keeps that bound; the power of two is put back into the exponent when the
 // results are rounded to FP64.  Quantisation of the input is below 2^-58 of
 // the block's largest component, each product is rounded at 2^-59.5 / R of
-// the full scale: the transform's error is below that of the FP64 butterflies
-// it takes the place of (n = 512: 7e-17 against 3.7e-16 relative;
-// tests/test_fx_cpu.py compares both with long double).  Measured: 100 steps of
-// 4 x 512^2 in FP64 90.4 -> 51.4 ms, 60 steps of the 256^2 free-space workload
-// 328 -> 216 ms.
+// the full scale.  Lines of 2048 points and more are scaled up again before each
+// middle pass (FxPass::rescales).  Relative L2 error of a transform, FP64 passes in
+// brackets: input spread over the line 7e-17 (4e-16) at any n; one nonzero value
+// 7.5e-17 (3e-16) at n = 512, 1.6e-16 (3.5e-16) at 1024, 9e-17 (4e-16) at 8192, where
+// without the scaling it was 1.4e-15 (tests/test_fx_cpu.py, test_fx_long_cpu.py compare
+// both with long double).  Measured: 100 steps of 4 x 512^2 in FP64 90.4 -> 51.4 ms,
+// 60 steps of the 256^2 free-space workload 328 -> 216 ms.
 //
 // A table factor w (|w| <= 1) is an int4 {ch, cl, sh, sl}: cos = ch 2^32 + cl in
 // units of 2^-61, cl signed (likewise sin), so that signed 32-bit

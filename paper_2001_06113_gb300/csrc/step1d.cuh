@@ -213,7 +213,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
                     }
                 }
             }
-            const auto sc = FI::scale_of(mx, 0);
+            auto sc = FI::scale_of(mx, 0);
 #pragma unroll 1
             for (int p = 0; p < PB; ++p) {
                 int j, line;
@@ -224,7 +224,7 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
                 }
                 FI::first_item(p, x, buf, tid, sc);
             }
-            FI::middle(buf, tw, twl, tid, sync);
+            FI::middle(buf, tw, twl, tid, sync, sc);
             C mid[FI::PL][FI::RL];
 #pragma unroll
             for (int p = 0; p < FI::PL; ++p) {
@@ -238,10 +238,10 @@ __device__ __forceinline__ void step1d(const KArgs& a, const int b, const int ti
             for (int p = 0; p < FI::PL; ++p)
 #pragma unroll
                 for (int r = 0; r < FI::RL; ++r) mx = max(mx, fx_hi(mid[p][r]));
-            const auto sw = FW::scale_of(mx, -ilog2(N));
+            auto sw = FW::scale_of(mx, -ilog2(N));
 #pragma unroll
             for (int p = 0; p < FW::PF; ++p) FW::first_item(p, mid[p], buf, tid, sw);
-            FW::middle(buf, tw, twl, tid, sync);
+            FW::middle(buf, tw, twl, tid, sync, sw);
 #pragma unroll 1
             for (int p = 0; p < FW::PL; ++p) {
                 C o[FW::RL];
