@@ -94,6 +94,7 @@ __device__ __forceinline__ void core(const double2 (&W)[Run1D64<N>::PER], const 
     for (int p = 0; p < G::PER; ++p) {
         const double beta = hmu0 * V[p], qx = V[p] * recip_ge1(fma(beta, beta, 1.0));
         q[p] = make_double2(qx, -beta * qx);
+        if (N < G::T && tid + p * G::T >= N) continue;      // n = 8, 16: threads without a mode of their own
         mw = max(mw, fx_hi(W[p]));
         mq = max(mq, fx_hi(q[p]));
     }
