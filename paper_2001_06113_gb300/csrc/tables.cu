@@ -249,9 +249,9 @@ __global__ void k_to_interaction(float4* state, float2* ring, int ring_slots, co
 
 // The same in 2D and 3D, where conj(E) is a product of one factor per axis.
 // Factors of the steps to convert: tab[b][q][n0 + n1 (+ n2)], q = 0 the state's
-// step in FP64, q = 1 + slot the ring's in double-float with the ring dither on
-// axis 0 (exact phases per mode instead took 10.9 ms of FP64 sines for 64 x
-// 512^2, 7.0 ms for 5 x 128^3).
+// step in FP64, q = 1 + slot the ring's as fixed-point factors (fx.cuh: 61 bits, and
+// products on the integer pipe) with the ring dither on axis 0 (exact phases per
+// mode instead took 10.9 ms of FP64 sines for 64 x 512^2, 7.0 ms for 5 x 128^3).
 __global__ void k_interaction_tables(double2* tab, const double* phi, int ntf, int n0, int n1, int n2, double dt, int n,
                                      Steps8 steps, int nslots) {
     const int q = blockIdx.x, b = blockIdx.y, d = n2 > 0 ? 3 : 2, len = n0 + n1 + n2;
@@ -267,7 +267,7 @@ __global__ void k_interaction_tables(double2* tab, const double* phi, int ntf, i
         double2 e = make_double2(c, -s);        // conj(E)
         if (q > 0) {
             if (ax == 0) e = cmul(make_double2(steps.z[q - 1][0], steps.z[q - 1][1]), e);
-            *reinterpret_cast<float4*>(&row[j]) = d_to_ffc(e);
+            *reinterpret_cast<int4*>(&row[j]) = fx_factor(e.x, e.y);
         } else {
             row[j] = e;
         }
@@ -297,11 +297,14 @@ __global__ void k_to_interaction_sep(float4* state, float2* ring, int ring_slots
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             if (q < nslots && steps.s[q] >= 0) {
-                const float4* t = reinterpret_cast<const float4*>(t0 + (size_t)(q + 1) * len);
-                float4 w = ffc_mul(__ldg(&t[m0]), __ldg(&t[n0 + m1]));
-                if (n2 > 0) w = ffc_mul(w, __ldg(&t[n0 + n1 + m2]));
-                const float4 p = ffc_mul(w, make_float4(r[q].x, r[q].y, 0.f, 0.f));
-                ring[((size_t)b * ring_slots + q) * NP + idx] = make_float2(p.x, p.y);
+                const int4* t = reinterpret_cast<const int4*>(t0 + (size_t)(q + 1) * len);
+                int4 w = fx_as_factor(fx_mul<false, 3>(fx_value(__ldg(&t[m0])), __ldg(&t[n0 + m1])));
+                if (n2 > 0) w = fx_as_factor(fx_mul<false, 3>(fx_value(w), __ldg(&t[n0 + n1 + m2])));
+                const double2 R = make_double2(fx_widen(r[q].x), fx_widen(r[q].y));
+                const unsigned mx = fx_hi(R);
+                const int E = fx_exponent(mx);
+                const double2 p = fx_to(fx_mul<false, 3>(fx_from(R, 59, E), w), mx >= 0x7ff00000u ? FX_NAN : E - 1022 - 59);
+                ring[((size_t)b * ring_slots + q) * NP + idx] = make_float2(fx_to_float(p.x), fx_to_float(p.y));
             }
         }
     }
