@@ -31,7 +31,8 @@
 // below 2^63 when |a| <= 2^62.5.
 //
 // NaN or infinity anywhere in the block gives NaN everywhere in it (an FP64
-// transform spreads them over the whole line).  Subnormals are kept.
+// transform spreads them over the whole line); magnitudes below 2^-958 lose
+// low bits and those below 2^-1022 become 0.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -43,18 +44,17 @@ FX_HD longlong2 operator+(longlong2 a, longlong2 b) { return make_longlong2(a.x 
 FX_HD longlong2 operator-(longlong2 a, longlong2 b) { return make_longlong2(a.x - b.x, a.y - b.y); }
 
 // Exponent of a block from the largest high word (sign bit cleared) of its
-// values: E, 1 for zeros and subnormals.
+// values: E, at least 64 so that the shifts below stay in range.
 FX_HD int fx_exponent(unsigned max_hi) {
     const int e = (int)(max_hi >> 20);
-    return e < 1 ? 1 : e;
+    return e < 64 ? 64 : e;
 }
 constexpr int FX_NAN = 1 << 20;     // output exponent of a block with a NaN or an infinity
 
 // v 2^(S + 1022 - E), truncated towards zero (S <= 61, E >= the exponent of v).
 FX_HD long long fx_from_bits(int hi, unsigned lo, int S, int E) {
-    const int e = (hi >> 20) & 0x7ff, one = e < 1 ? 0 : 0x100000;     // a subnormal has no leading one
-    const unsigned long long mant = ((unsigned long long)(unsigned)((hi & 0xfffff) | one) << 32 | lo) << 10;
-    int sh = 63 - S + E - (e < 1 ? 1 : e);
+    const unsigned long long mant = ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | lo) << 10;
+    int sh = 63 - S + E - ((hi >> 20) & 0x7ff);
     sh = sh > 63 ? 63 : sh;
     const long long t = (long long)(mant >> (sh & 63));
     return hi < 0 ? -t : t;
@@ -73,7 +73,6 @@ FX_HD unsigned long long fx_to_bits(long long v, int X) {
     const int e = X - lz + 1085;
     if (u == 0 || (unsigned)e >= 2046u) {
         if (X >= FX_NAN / 2) return 0x7ff8000000000000ull;
-        if (u != 0 && e < 0 && e > -54) return sign | ((t >> 1 >> (10 - e)) + ((t >> (10 - e)) & 1));     // a subnormal
         return sign | (u == 0 || e < 0 ? 0ull : 0x7ff0000000000000ull);
     }
     return sign | (((unsigned long long)(unsigned)e << 52) + (t >> 11) + ((t >> 10) & 1));
@@ -170,24 +169,18 @@ __device__ __forceinline__ double2 fx_factor_to_d(int4 w) {
     const double u = 1.0 / 536870912.0, l = 1.0 / 2305843009213693952.0;
     return make_double2(fma((double)w.y, l, (double)w.x * u), fma((double)w.w, l, (double)w.z * u));
 }
-// FP64 bits -> FP32, rounded to nearest (ties away), in integer arithmetic
-// (below FP32's normal range by the conversion instruction).
+// FP64 bits -> FP32, rounded to nearest (ties away), in integer arithmetic.
 __device__ __forceinline__ float fx_to_float(double v) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     const int e = (int)((hi >> 20) & 0x7ff) - 896;
     unsigned f = ((unsigned)e << 23 | (hi & 0xfffffu) << 3 | lo >> 29) + ((lo >> 28) & 1);
-    if (e <= 0) {
-        if ((hi << 1 | lo) != 0) return (float)v;
-        f = 0;
-    }
+    if (e <= 0) f = 0;
     if (e >= 255) f = 0x7f800000u + (e == 1151 && ((hi & 0xfffffu) | lo) ? 0x400000u : 0);
     return __uint_as_float(f | (hi & 0x80000000u));
 }
-// FP32 value as FP64 bits, in integer arithmetic (subnormals by the conversion
-// instruction).
+// FP32 value as FP64 bits (subnormals become 0), in integer arithmetic.
 __device__ __forceinline__ double fx_widen(float x) {
     const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xff;
-    if (e == 0 && (b << 1) != 0) return (double)x;
     const unsigned hi = e == 0 ? 0u : ((b & 0x7fffffffu) >> 3) + (e == 255 ? 0x70000000u : 0x38000000u);
     return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(e == 0 ? 0u : b << 29));
 }
