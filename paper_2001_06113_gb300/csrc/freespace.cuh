@@ -561,10 +561,10 @@ template <bool WIDE> __device__ __forceinline__ int4 phase_mul(int4 a, int4 b, i
     else return fx_as_factor(pmul(fx_value(a), b, g));
 }
 
-__device__ __forceinline__ float2 to_c(double2 v, float2) { return make_float2(fx_to_float(v.x), fx_to_float(v.y)); }
+__device__ __forceinline__ float2 to_c(double2 v, float2) { return fx_to_float(v); }
 __device__ __forceinline__ double2 to_c(double2 v, double2) { return v; }
 
-__device__ __forceinline__ double2 widen(float2 x) { return make_double2(fx_widen(x.x), fx_widen(x.y)); }
+__device__ __forceinline__ double2 widen(float2 x) { return fx_widen(x); }
 __device__ __forceinline__ double2 widen(double2 x) { return x; }
 // v * (-i c) added to u
 __device__ __forceinline__ double2 add_minus_i(double2 u, double c, double2 v) {

@@ -169,20 +169,29 @@ __device__ __forceinline__ double2 fx_factor_to_d(int4 w) {
     const double u = 1.0 / 536870912.0, l = 1.0 / 2305843009213693952.0;
     return make_double2(fma((double)w.y, l, (double)w.x * u), fma((double)w.w, l, (double)w.z * u));
 }
-// FP64 bits -> FP32, rounded to nearest (ties away), in integer arithmetic.
-__device__ __forceinline__ float fx_to_float(double v) {
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+// FP64 -> FP32, rounded to nearest (ties away), in integer arithmetic; a pair with
+// a value below FP32's normal range by the conversion instruction.
+__device__ __forceinline__ float fx_to_float(unsigned hi, unsigned lo) {
     const int e = (int)((hi >> 20) & 0x7ff) - 896;
     unsigned f = ((unsigned)e << 23 | (hi & 0xfffffu) << 3 | lo >> 29) + ((lo >> 28) & 1);
-    if (e <= 0) f = 0;
     if (e >= 255) f = 0x7f800000u + (e == 1151 && ((hi & 0xfffffu) | lo) ? 0x400000u : 0);
     return __uint_as_float(f | (hi & 0x80000000u));
 }
-// FP32 value as FP64 bits (subnormals become 0), in integer arithmetic.
-__device__ __forceinline__ double fx_widen(float x) {
-    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xff;
-    const unsigned hi = e == 0 ? 0u : ((b & 0x7fffffffu) >> 3) + (e == 255 ? 0x70000000u : 0x38000000u);
-    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(e == 0 ? 0u : b << 29));
+__device__ __forceinline__ float2 fx_to_float(double2 v) {
+    const unsigned a = (unsigned)__double2hiint(v.x), b = (unsigned)__double2hiint(v.y);
+    if (min(a << 1, b << 1) < 0x70200000u) return make_float2((float)v.x, (float)v.y);      // below 2^-126
+    return make_float2(fx_to_float(a, (unsigned)__double2loint(v.x)), fx_to_float(b, (unsigned)__double2loint(v.y)));
+}
+// FP32 -> FP64 in integer arithmetic; a pair with a zero or a subnormal by the
+// conversion instruction.
+__device__ __forceinline__ double2 fx_widen(float2 v) {
+    const unsigned a = __float_as_uint(v.x), b = __float_as_uint(v.y);
+    if (min(a << 1, b << 1) < 0x1000000u) return make_double2((double)v.x, (double)v.y);
+    auto one = [](unsigned x) {
+        const unsigned hi = ((x & 0x7fffffffu) >> 3) + ((x & 0x7f800000u) == 0x7f800000u ? 0x70000000u : 0x38000000u);
+        return __hiloint2double((int)(hi | (x & 0x80000000u)), (int)(x << 29));
+    };
+    return make_double2(one(a), one(b));
 }
 // Largest value of v over the T threads of a CTA (all of them call it).
 template <int T>

@@ -161,6 +161,12 @@ __global__ void k_split_float(float2* hilo, const double* src, size_t n) {
 
 struct Coef4 { double c[4]; };
 
+// FP64 -> double-float, the conversions in integer arithmetic.
+__device__ __forceinline__ float4 ff_split(double2 v) {
+    const float2 h = fx_to_float(v), l = fx_to_float(v - fx_widen(h));
+    return make_float4(h.x, h.y, l.x, l.y);
+}
+
 // Double-float states: FP64 sums of products with the FP32 parts (4 fused
 // multiply-adds per chain instead of conversions and sums of each pair: the
 // FP64 pipe bounds it; 5 x 128^3: 0.76 -> 0.37 ms).
@@ -174,14 +180,14 @@ __global__ void k_combine_ff(float4* state, const float4* chains, size_t stride,
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             if (c < L) {
-                re = fma(co.c[c], fx_widen(v[c].x), re);
-                im = fma(co.c[c], fx_widen(v[c].y), im);
-                re = fma(co.c[c], fx_widen(v[c].z), re);
-                im = fma(co.c[c], fx_widen(v[c].w), im);
+                const double2 hi = fx_widen(make_float2(v[c].x, v[c].y)), lo = fx_widen(make_float2(v[c].z, v[c].w));
+                re = fma(co.c[c], hi.x, re);
+                im = fma(co.c[c], hi.y, im);
+                re = fma(co.c[c], lo.x, re);
+                im = fma(co.c[c], lo.y, im);
             }
         }
-        const float rh = fx_to_float(re), ih = fx_to_float(im);
-        state[i] = make_float4(rh, ih, fx_to_float(re - fx_widen(rh)), fx_to_float(im - fx_widen(ih)));
+        state[i] = ff_split(make_double2(re, im));
     }
 }
 
@@ -291,20 +297,18 @@ __global__ void k_to_interaction_sep(float4* state, float2* ring, int ring_slots
         const float4 x = *sv;
         double2 e = cmul(__ldg(&t0[m0]), __ldg(&t0[n0 + m1]));
         if (n2 > 0) e = cmul(e, __ldg(&t0[n0 + n1 + m2]));
-        const double2 v = cmul(e, make_double2(fx_widen(x.x) + fx_widen(x.z), fx_widen(x.y) + fx_widen(x.w)));
-        const float vh = fx_to_float(v.x), wh = fx_to_float(v.y);
-        *sv = make_float4(vh, wh, fx_to_float(v.x - fx_widen(vh)), fx_to_float(v.y - fx_widen(wh)));
+        *sv = ff_split(cmul(e, fx_widen(make_float2(x.x, x.y)) + fx_widen(make_float2(x.z, x.w))));
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             if (q < nslots && steps.s[q] >= 0) {
                 const int4* t = reinterpret_cast<const int4*>(t0 + (size_t)(q + 1) * len);
                 int4 w = fx_as_factor(fx_mul<false, 3>(fx_value(__ldg(&t[m0])), __ldg(&t[n0 + m1])));
                 if (n2 > 0) w = fx_as_factor(fx_mul<false, 3>(fx_value(w), __ldg(&t[n0 + n1 + m2])));
-                const double2 R = make_double2(fx_widen(r[q].x), fx_widen(r[q].y));
+                const double2 R = fx_widen(r[q]);
                 const unsigned mx = fx_hi(R);
                 const int E = fx_exponent(mx);
                 const double2 p = fx_to(fx_mul<false, 3>(fx_from(R, 59, E), w), mx >= 0x7ff00000u ? FX_NAN : E - 1022 - 59);
-                ring[((size_t)b * ring_slots + q) * NP + idx] = make_float2(fx_to_float(p.x), fx_to_float(p.y));
+                ring[((size_t)b * ring_slots + q) * NP + idx] = fx_to_float(p);
             }
         }
     }
