@@ -749,7 +749,7 @@ __device__ __forceinline__ float2 implicit_solve(float2 y, float c) {
     return make_float2((y.x + c * y.y) / den, (y.y - c * y.x) / den);
 }
 __device__ __forceinline__ double2 implicit_solve(double2 y, double c) {
-    const double q = recip_ge1(fma(c, c, 1.0));
+    const double q = recip_any(fma(c, c, 1.0));
     return make_double2(fma(c, y.y, y.x) * q, fma(-c, y.x, y.y) * q);
 }
 

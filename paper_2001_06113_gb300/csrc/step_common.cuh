@@ -287,14 +287,19 @@ __device__ __forceinline__ double2 horner_W64(const KArgs& a, double2 uh, const 
     return fx_horner(uh, r, a.nhist, a.mu_w, a.h_w, a.h_e, [&](int j) { return ph.w64(j); });
 }
 
-// 1/d for 1 <= d: the hardware's estimate and one step of Halley's third-order
-// iteration (e = 1 - d r, r (1 + e + e^2)): 2^-20 -> below 2^-53 in 3 FP64
-// instructions (an FP64 division takes about ten).
+// 1/d for 1 <= d < 2^1022: the hardware's estimate r, e = 1 - d r, and one step of
+// Halley's third-order iteration r (1 + e + e^2), which cubes the estimate's error
+// (below 2^-18 leaves 2^-54) in 3 FP64 instructions where an FP64 division takes about
+// ten.  (Beyond, where the estimate is flushed to 0: 0, and NaN at infinity.)
 __device__ __forceinline__ double recip_ge1(double d) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
     const double e = fma(-d, r, 1.0);
     return fma(r, fma(e, e, e), r);
+}
+// The same up to infinity.
+__device__ __forceinline__ double recip_any(double d) {
+    return (unsigned)__double2hiint(d) >= 0x7fd00000u ? 1.0 / d : recip_ge1(d);
 }
 
 // u = y / (1 + i beta), beta = h mu_0 V, returns V u with V = Vhi + Vlo.

@@ -1,7 +1,7 @@
 // Device functions of csrc/step_common.cuh and csrc/fx.cuh against CUDA's own
 // division and conversions.  `fx_device recip`: 1/d of recip_ge1, prints the largest
 // error in ulps of 1.0 / d over random d in 1..2^1022, the largest relative error
-// of the estimate that it starts from, and the number of wrong results of recip_ge1
+// of the estimate that it starts from, and the number of wrong results of recip_any
 // beyond (d up to infinity, NaN).  `fx_device float`: conversions between FP32 and FP64, prints
 // the number of results that are not nearest, for widening and for narrowing.
 #include <cmath>
@@ -48,8 +48,8 @@ __global__ void k_recip(Out* o, int n) {
         const double inf = __longlong_as_double(0x7ff0000000000000ll), nan = __longlong_as_double(0x7ff8000000000000ll);
         const double big[] = {0x1p1022, 0x1.5555555555555p1022, 0x1.fffffffffffffp1022, 0x1p1023, 0x1.fffffffffffffp1023, inf};
         for (double d : big)
-            if (recip_ge1(d) != 1.0 / d) atomicAdd(&o->wrong, 1);
-        if (recip_ge1(nan) == recip_ge1(nan) || recip_ge1(-nan) == recip_ge1(-nan)) atomicAdd(&o->wrong, 1);
+            if (recip_any(d) != 1.0 / d) atomicAdd(&o->wrong, 1);
+        if (recip_any(nan) == recip_any(nan) || recip_any(-nan) == recip_any(-nan)) atomicAdd(&o->wrong, 1);
     }
 }
 

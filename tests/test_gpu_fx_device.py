@@ -22,6 +22,15 @@ def exe(tmp_path_factory):
     return out
 
 
+def test_reciprocal_of_the_implicit_solve(exe):
+    """One step of Halley's iteration cubes the estimate's error e: with e below
+    2^-18 the result is off by 2^-54 and a rounding, one ulp of 1.0 / d at most."""
+    ulps, estimate, wrong = subprocess.run([exe, "recip"], capture_output=True, text=True, check=True).stdout.split()
+    assert float(estimate) <= 2.0 ** -18
+    assert float(ulps) <= 1.0
+    assert int(wrong) == 0
+
+
 def test_conversions_round_to_nearest(exe):
     """FP32 -> FP64 exact, FP64 -> FP32 to nearest, over subnormals, infinities and NaN."""
     assert subprocess.run([exe, "float"], capture_output=True, text=True, check=True).stdout.split() == ["0", "0"]
