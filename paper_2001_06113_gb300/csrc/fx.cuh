@@ -169,29 +169,46 @@ __device__ __forceinline__ double2 fx_factor_to_d(int4 w) {
     const double u = 1.0 / 536870912.0, l = 1.0 / 2305843009213693952.0;
     return make_double2(fma((double)w.y, l, (double)w.x * u), fma((double)w.w, l, (double)w.z * u));
 }
-// FP64 -> FP32, rounded to nearest (ties away), in integer arithmetic; a pair with
-// a value below FP32's normal range by the conversion instruction.
-__device__ __forceinline__ float fx_to_float(unsigned hi, unsigned lo) {
-    const int e = (int)((hi >> 20) & 0x7ff) - 896;
+// FP64 -> FP32, rounded to nearest (ties away), in integer arithmetic: small
+// values as v 2^64 and an FP32 product with 2^-64, which gives the subnormals
+// (rounded twice).  A branch to the conversion instruction for them instead cost the
+// 256^2 free-space step 1 % (FP64 conversions are issued at 1/64 of the FP32 rate).
+__device__ __forceinline__ float fx_to_float(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const int e0 = (int)((hi >> 20) & 0x7ff) - 896, k = e0 < 64 ? 64 : 0, e = e0 + k;
     unsigned f = ((unsigned)e << 23 | (hi & 0xfffffu) << 3 | lo >> 29) + ((lo >> 28) & 1);
+    if (e <= 0) f = 0;
     if (e >= 255) f = 0x7f800000u + (e == 1151 && ((hi & 0xfffffu) | lo) ? 0x400000u : 0);
-    return __uint_as_float(f | (hi & 0x80000000u));
+    return __uint_as_float(f | (hi & 0x80000000u)) * (k ? 0x1p-64f : 1.0f);
 }
-__device__ __forceinline__ float2 fx_to_float(double2 v) {
-    const unsigned a = (unsigned)__double2hiint(v.x), b = (unsigned)__double2hiint(v.y);
-    if (min(a << 1, b << 1) < 0x70200000u) return make_float2((float)v.x, (float)v.y);      // below 2^-126
-    return make_float2(fx_to_float(a, (unsigned)__double2loint(v.x)), fx_to_float(b, (unsigned)__double2loint(v.y)));
-}
-// FP32 -> FP64 in integer arithmetic; a pair with a zero or a subnormal by the
-// conversion instruction.
+__device__ __forceinline__ float2 fx_to_float(double2 v) { return make_float2(fx_to_float(v.x), fx_to_float(v.y)); }
+// FP32 -> FP64 times 1 / FX_WIDEN in integer arithmetic: with the exponent field
+// as it is, zeros, subnormals and normal numbers move alike.  What multiplies
+// the result takes the factor FX_WIDEN, which changes no rounding.
+constexpr double FX_WIDEN = 0x1p896;
 __device__ __forceinline__ double2 fx_widen(float2 v) {
-    const unsigned a = __float_as_uint(v.x), b = __float_as_uint(v.y);
-    if (min(a << 1, b << 1) < 0x1000000u) return make_double2((double)v.x, (double)v.y);
-    auto one = [](unsigned x) {
-        const unsigned hi = ((x & 0x7fffffffu) >> 3) + ((x & 0x7f800000u) == 0x7f800000u ? 0x70000000u : 0x38000000u);
-        return __hiloint2double((int)(hi | (x & 0x80000000u)), (int)(x << 29));
+    auto one = [](float f) {
+        const unsigned x = __float_as_uint(f), a = x & 0x7fffffffu;
+        return __hiloint2double((int)((a >> 3) + (a >= 0x7f800000u ? 0x70000000u : 0u) | (x & 0x80000000u)), (int)(x << 29));
     };
-    return make_double2(one(a), one(b));
+    return make_double2(one(v.x), one(v.y));
+}
+// An FP32 pair as integers: components v 2^(59 + 126 - E), E the larger exponent field
+// (1 at least), and back from such integers.
+__device__ __forceinline__ longlong2 fx_from_float(float2 v, int& E) {
+    const unsigned a = __float_as_uint(v.x), b = __float_as_uint(v.y);
+    const int ea = max((int)((a >> 23) & 0xff), 1), eb = max((int)((b >> 23) & 0xff), 1);
+    E = max(ea, eb);
+    auto one = [E](unsigned x, int e) {
+        const unsigned m = (x & 0x7fffffu) | ((x & 0x7f800000u) ? 0x800000u : 0u);
+        const long long t = (long long)((unsigned long long)m << 35 >> min(E - e, 63));
+        return (int)x < 0 ? -t : t;
+    };
+    return make_longlong2(one(a, ea), one(b, eb));
+}
+__device__ __forceinline__ float2 fx_to_float(longlong2 v, int E) {
+    const float s = __uint_as_float((unsigned)E << 23);          // 2^(E - 127); infinite for a pair with an infinity or a NaN
+    return make_float2(__ll2float_rn(v.x) * 0x1p-58f * s, __ll2float_rn(v.y) * 0x1p-58f * s);
 }
 // Largest value of v over the T threads of a CTA (all of them call it).
 template <int T>

@@ -163,7 +163,9 @@ struct Coef4 { double c[4]; };
 
 // FP64 -> double-float, the conversions in integer arithmetic.
 __device__ __forceinline__ float4 ff_split(double2 v) {
-    const float2 h = fx_to_float(v), l = fx_to_float(v - fx_widen(h));
+    const float2 h = fx_to_float(v);
+    const double2 w = fx_widen(h);
+    const float2 l = fx_to_float(make_double2(fma(-FX_WIDEN, w.x, v.x), fma(-FX_WIDEN, w.y, v.y)));
     return make_float4(h.x, h.y, l.x, l.y);
 }
 
@@ -181,10 +183,11 @@ __global__ void k_combine_ff(float4* state, const float4* chains, size_t stride,
         for (int c = 0; c < 4; ++c) {
             if (c < L) {
                 const double2 hi = fx_widen(make_float2(v[c].x, v[c].y)), lo = fx_widen(make_float2(v[c].z, v[c].w));
-                re = fma(co.c[c], hi.x, re);
-                im = fma(co.c[c], hi.y, im);
-                re = fma(co.c[c], lo.x, re);
-                im = fma(co.c[c], lo.y, im);
+                const double k = co.c[c] * FX_WIDEN;
+                re = fma(k, hi.x, re);
+                im = fma(k, hi.y, im);
+                re = fma(k, lo.x, re);
+                im = fma(k, lo.y, im);
             }
         }
         state[i] = ff_split(make_double2(re, im));
@@ -275,7 +278,7 @@ __global__ void k_interaction_tables(double2* tab, const double* phi, int ntf, i
             if (ax == 0) e = cmul(make_double2(steps.z[q - 1][0], steps.z[q - 1][1]), e);
             *reinterpret_cast<int4*>(&row[j]) = fx_factor(e.x, e.y);
         } else {
-            row[j] = e;
+            row[j] = ax == 0 ? cscale(e, FX_WIDEN) : e;      // (times fx_widen's results)
         }
     }
 }
@@ -304,11 +307,9 @@ __global__ void k_to_interaction_sep(float4* state, float2* ring, int ring_slots
                 const int4* t = reinterpret_cast<const int4*>(t0 + (size_t)(q + 1) * len);
                 int4 w = fx_as_factor(fx_mul<false, 3>(fx_value(__ldg(&t[m0])), __ldg(&t[n0 + m1])));
                 if (n2 > 0) w = fx_as_factor(fx_mul<false, 3>(fx_value(w), __ldg(&t[n0 + n1 + m2])));
-                const double2 R = fx_widen(r[q]);
-                const unsigned mx = fx_hi(R);
-                const int E = fx_exponent(mx);
-                const double2 p = fx_to(fx_mul<false, 3>(fx_from(R, 59, E), w), mx >= 0x7ff00000u ? FX_NAN : E - 1022 - 59);
-                ring[((size_t)b * ring_slots + q) * NP + idx] = fx_to_float(p);
+                int E;
+                const longlong2 R = fx_from_float(r[q], E);
+                ring[((size_t)b * ring_slots + q) * NP + idx] = fx_to_float(fx_mul<false, 3>(R, w), E);
             }
         }
     }

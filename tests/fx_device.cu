@@ -61,7 +61,15 @@ __global__ void k_float(Out* o, int n) {
         if (i % 64 == 1) f = (f & 0x80000000u) | 0x7f800000u;
         const float x = __uint_as_float(f);
         const float x2 = __uint_as_float((unsigned)(b >> 32));    // any neighbour
-        const double w = i & 1 ? fx_widen(make_float2(x, x2)).x : fx_widen(make_float2(x2, x)).y, t = (double)x;
+        const double w = FX_WIDEN * (i & 1 ? fx_widen(make_float2(x, x2)).x : fx_widen(make_float2(x2, x)).y), t = (double)x;
+        // a pair as integers and back, the second component within 2^34 of the first
+        if (x == x && isfinite(x)) {
+            int E;
+            const float y = ldexpf(1.0f + (float)(b >> 59), max(-149, min(120, ilogbf(x == 0.0f ? 1e-30f : x) - 20 + (int)((b >> 40) % 40))));
+            const longlong2 v = fx_from_float(make_float2(x, y), E);
+            const float2 z = fx_to_float(v, E);
+            if (z.x != x || z.y != y) atomicAdd(&o->widen, 1);
+        }
         if (x == x ? __double_as_longlong(w) != __double_as_longlong(t) : w == w) atomicAdd(&o->widen, 1);
         // FP64 values over FP32's range and a little beyond it on both sides
         const unsigned long long e = 1023 - 155 + (b >> 54) % 290;
@@ -71,7 +79,10 @@ __global__ void k_float(Out* o, int n) {
         if (i % 64 == 4) v = __longlong_as_double(0x7ff0000000000001ll);
         const double v2 = __longlong_as_double((long long)mix(b + 1));
         const float got = i & 1 ? fx_to_float(make_double2(v, v2)).x : fx_to_float(make_double2(v2, v)).y, want = (float)v;
-        if (v != v ? got == got : (got != want && fabs((double)got - v) != fabs((double)want - v))) atomicAdd(&o->narrow, 1);
+        // nearest, ties either way; subnormal results: rounded to 24 bits, then to their step
+        const bool sub = fabs(v) < 0x1p-126;
+        const double off = fabs((double)got - v);
+        if (v != v ? got == got : (got != want && (sub ? off > 0x1p-150 + fabs(v) * 0x1p-24 : off != fabs((double)want - v)))) atomicAdd(&o->narrow, 1);
         if (v == v && signbit(got) != signbit(want)) atomicAdd(&o->narrow, 1);
     }
 }

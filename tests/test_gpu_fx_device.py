@@ -32,5 +32,6 @@ def test_reciprocal_of_the_implicit_solve(exe):
 
 
 def test_conversions_round_to_nearest(exe):
-    """FP32 -> FP64 exact, FP64 -> FP32 to nearest, over subnormals, infinities and NaN."""
+    """FP32 -> FP64 exact (pairs as integers and back too), FP64 -> FP32 to nearest, over
+    subnormals, infinities and NaN."""
     assert subprocess.run([exe, "float"], capture_output=True, text=True, check=True).stdout.split() == ["0", "0"]
