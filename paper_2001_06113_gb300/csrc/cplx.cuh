@@ -484,7 +484,7 @@ struct CtaFft<double2, N, L, LS, T, INV> {
                 }
             }
             if constexpr (Fx::rescales(S)) {
-                static_assert(ITEMS % T == 0, "every value is set");
+                static_assert(ITEMS % T == 0 && L == 1, "every value is set, one line");
                 X -= fx_rescale<Fx, T>(v, CtaSync{});
             } else {
                 __syncthreads();
@@ -529,7 +529,8 @@ struct CtaFft<double2, N, L, LS, T, INV> {
                 }
             }
         }
-        mx = fx_cta_max<T>(mx);                 // its barrier also orders the loads above before the stores below
+        static_assert(T % L == 0, "a thread keeps its line");
+        mx = fx_line_max<T, L>(mx);             // its barrier also orders the loads above before the stores below
         if constexpr (T <= 32) __syncwarp();
         const int E = fx_exponent(mx), X = Fx::out_exp(mx, E, lg);
         longlong2 v[PER][R];

@@ -7,14 +7,14 @@
 // with its twiddles is 84 FP64 instructions = 5376 cycles, and about 375
 // cycles in the form below.
 //
-// A transform takes FP64 inputs, finds the largest exponent E of the block of
-// lines, and holds x 2^(S + 1022 - E), S = 62 - log2(first radix), as 64-bit
+// A transform takes FP64 inputs, finds the largest exponent E of the line, and
+// holds x 2^(S + 1022 - E), S = 62 - log2(first radix), as 64-bit
 // integers: components below 2^S, so that after the first butterfly the
 // modulus is at most 2^62.5.  Every later pass of radix R multiplies by the
 // twiddle and by 1/R in the same 128-bit product and adds up R terms, which
 // keeps that bound; the power of two is put back into the exponent when the
 // results are rounded to FP64.  Quantisation of the input is below 2^-58 of
-// the block's largest component, each product is rounded at 2^-59.5 / R of
+// the line's largest component, each product is rounded at 2^-59.5 / R of
 // the full scale.  Lines of 2048 points and more are scaled up again before each
 // middle pass (FxPass::rescales).  Relative L2 error of a transform, FP64 passes in
 // brackets: input spread over the line 7e-17 (4e-16) at any n; one nonzero value
@@ -30,9 +30,11 @@
 // and for complex factors the four cross products of one component stay
 // below 2^63 when |a| <= 2^62.5.
 //
-// NaN or infinity anywhere in the block gives NaN everywhere in it (an FP64
-// transform spreads them over the whole line); magnitudes below 2^-958 lose
-// low bits and those below 2^-1022 become 0.
+// NaN or infinity anywhere in a line gives NaN everywhere in it (an FP64
+// transform spreads them over the whole line).  A line is held to 2^-1017 at best:
+// magnitudes below 2^-958 lose low bits and those below 2^-1022 become 0.  (Keeping
+// them costs three more instructions in every conversion: 4 x 512^2 in FP64 31.6 ->
+// 33.9 ms.)
 #pragma once
 #include <cuda_runtime.h>
 
@@ -221,6 +223,33 @@ __device__ __forceinline__ unsigned fx_cta_max(unsigned v) {
         v = __reduce_max_sync(0xffffffffu, mx[(threadIdx.x & 31) % (T / 32)]);
     }
     return v;
+}
+// The same per line, L lines interleaved over the threads (thread t works on line t % L).
+template <int T, int L>
+__device__ __forceinline__ unsigned fx_line_max(unsigned v) {
+    static_assert(L <= 32 && 32 % L == 0 && T % 32 == 0, "a warp holds whole sets of lines");
+    if constexpr (L == 1) {
+        return fx_cta_max<T>(v);
+    } else {
+        auto fold = [](unsigned x) {
+#pragma unroll
+            for (int o = 16; o >= L; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
+            return x;
+        };
+        v = fold(v);
+        if constexpr (T > 32) {
+            __shared__ unsigned mx[T / 32 * L];
+            const int lane = threadIdx.x & 31;
+            if (lane < L) mx[(threadIdx.x >> 5) * L + lane] = v;
+            __syncthreads();
+            v = 0;
+#pragma unroll
+            for (int w = 0; w < T / 32; w += 32 / L)
+                if (w + lane / L < T / 32) v = max(v, mx[(w + lane / L) * L + lane % L]);
+            v = fold(v);
+        }
+        return v;
+    }
 }
 #endif  // __CUDACC__
 
