@@ -50,6 +50,7 @@
 #include <type_traits>
 
 #include "cplx.cuh"
+#include "device_once.h"
 #include "fsargs.h"
 #include "step_common.cuh"
 
@@ -1096,12 +1097,11 @@ template <class N, int M, int R>
 cudaError_t launch_mr(const FsArgs& a, int which, int flag, cudaStream_t s) {
     using G = Geo<M, R>;
     constexpr size_t sm = sizeof(Smem<N, G>);
-    static bool done[4] = {false, false, false, false};
+    static DeviceOnce once[4];
     cudaError_t e = cudaSuccess;
     auto ready = [&](auto kernel) {
-        if (!done[which]) e = prepare(kernel, sm);
-        done[which] = e == cudaSuccess;
-        return done[which];
+        e = once[which]([&] { return prepare(kernel, sm); });
+        return e == cudaSuccess;
     };
     if (which == 0) {
         if (!ready(k_fs_1d<N, M, R>)) return e;

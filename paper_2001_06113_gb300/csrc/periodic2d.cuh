@@ -31,6 +31,7 @@
 #pragma once
 #include <type_traits>
 
+#include "device_once.h"
 #include "step_common.cuh"
 
 namespace tdse {
@@ -743,16 +744,14 @@ __global__ void __launch_bounds__((threads_2d<float2, N0, L>()), (min_blocks_2d<
 // 6.6 (with the smaller CTAs); 4 x 512^2 in FP64 as four chains 31.8 -> 34.3 if
 // they overlapped too.
 template <class K, class... A>
-static cudaError_t launch_pass(K kern, dim3 grid, int threads, size_t smem, bool& done, cudaStream_t s, const KArgs& a,
+static cudaError_t launch_pass(K kern, dim3 grid, int threads, size_t smem, DeviceOnce& once, cudaStream_t s, const KArgs& a,
                                const A&... more) {
-    cudaError_t e = cudaSuccess;
-    if (!done) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        done = true;
-    }
+    cudaError_t e = once([&] {
+        const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return r != cudaSuccess ? r
+                                : cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    });
+    if (e != cudaSuccess) return e;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -777,9 +776,9 @@ template <class C, class RT, int N0>
 static cudaError_t col_begin_n(const KArgs& a, cudaStream_t s) {
     return with_lanes<C>((long long)a.n1 * a.B, [&](auto l) {
         constexpr int L = decltype(l)::value;
-        static bool done = false;
+        static DeviceOnce once;
         return launch_pass(k_col_begin<C, RT, N0, L>, dim3(a.n1 / L, a.B), threads_2d<C, N0, L>(), (size_t)N0 * L * sizeof(C),
-                           done, s, a);
+                           once, s, a);
     });
 }
 
@@ -787,9 +786,9 @@ template <class C, class RT, int N0, bool FUSED>
 static cudaError_t col_end_n(const KArgs& a, cudaStream_t s) {
     return with_lanes<C>((long long)a.n1 * a.B, [&](auto l) {
         constexpr int L = decltype(l)::value;
-        static bool done = false;
+        static DeviceOnce once;
         return launch_pass(k_col_end<C, RT, N0, FUSED, L>, dim3(a.n1 / L, a.B), threads_2d<C, N0, L>(),
-                           (size_t)N0 * L * sizeof(C), done, s, a);
+                           (size_t)N0 * L * sizeof(C), once, s, a);
     });
 }
 
@@ -797,9 +796,9 @@ template <int N0>
 static cudaError_t col_chain_n(const KArgs& a, cudaStream_t s) {
     return with_lanes<float2>((long long)a.n1 * a.B, [&](auto l) {
         constexpr int L = decltype(l)::value;
-        static bool done = false;
+        static DeviceOnce once;
         return launch_pass(k_col_chain<N0, L>, dim3(a.n1 / L, a.B), threads_2d<float2, N0, L>(), (size_t)N0 * L * sizeof(float2),
-                           done, s, a);
+                           once, s, a);
     });
 }
 
@@ -808,17 +807,17 @@ static cudaError_t col_fused_ip_n(const KArgs& a, cudaStream_t s) {
     return with_lanes<float2>((long long)a.n1 * a.B, [&](auto l) {
         constexpr int L = decltype(l)::value, RC = chunk_rows<N0, L>(), NB = N0 > RC ? 2 : 1;
         const size_t smem = (size_t)N0 * L * sizeof(float2) + NB * (size_t)RC * L * (sizeof(float4) + (MAX_HIST - 1) * sizeof(float2));
-        static bool done = false;
-        return launch_pass(k_col_fused_ip<N0, VAR, L>, dim3(a.n1 / L, a.B), threads_2d<float2, N0, L>(), smem, done, s, a);
+        static DeviceOnce once;
+        return launch_pass(k_col_fused_ip<N0, VAR, L>, dim3(a.n1 / L, a.B), threads_2d<float2, N0, L>(), smem, once, s, a);
     });
 }
 
 template <int N1>
 static cudaError_t row32_n(const KArgs& a, cudaStream_t s) {
     using G = Row32<N1>;
-    static bool done = false;
+    static DeviceOnce once;
     return launch_pass(k_row32<N1, G::L>, dim3(a.n0 / G::L, a.B), G::T * G::L,
-                       (size_t)G::L * fft_len<float2>(N1) * sizeof(float2), done, s, a);
+                       (size_t)G::L * fft_len<float2>(N1) * sizeof(float2), once, s, a);
 }
 
 template <class C, int N1>
@@ -827,9 +826,9 @@ static cudaError_t row_mid_n(const KArgs& a, cudaStream_t s) {
     else
     return with_lanes<C>((long long)a.n0 * a.B, [&](auto l) {
         constexpr int L = decltype(l)::value;
-        static bool done = false;
+        static DeviceOnce once;
         return launch_pass(k_row_mid<C, N1, L>, dim3(a.n0 / L, a.B), threads_2d<C, N1, L>(), (size_t)N1 * (L + 1) * sizeof(C),
-                           done, s, a);
+                           once, s, a);
     });
 }
 
@@ -939,12 +938,12 @@ template <class C, int N1>
 static cudaError_t axis1_n(const KArgs& a, bool inv, void* X, cudaStream_t s) {
     return with_lanes<C>((long long)a.tn2 * a.tn0 * a.B, [&](auto l) {
         constexpr int L = decltype(l)::value;
-        static bool done_f = false, done_i = false;
+        static DeviceOnce once_f, once_i;
         const dim3 grid(a.tn2 / L, a.tn0, a.B);
         const size_t smem = (size_t)N1 * L * sizeof(C);
         C* x = static_cast<C*>(X);
-        return inv ? launch_pass(k_axis1<C, N1, true, L>, grid, threads_2d<C, N1, L>(), smem, done_i, s, a, x)
-                   : launch_pass(k_axis1<C, N1, false, L>, grid, threads_2d<C, N1, L>(), smem, done_f, s, a, x);
+        return inv ? launch_pass(k_axis1<C, N1, true, L>, grid, threads_2d<C, N1, L>(), smem, once_i, s, a, x)
+                   : launch_pass(k_axis1<C, N1, false, L>, grid, threads_2d<C, N1, L>(), smem, once_f, s, a, x);
     });
 }
 

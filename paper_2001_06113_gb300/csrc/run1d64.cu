@@ -16,6 +16,7 @@
 // Against one launch per step of the kernel that larger n use, 100 steps:
 // n = 128 x 1 9.1 -> 0.88 ms, 64 x 2048 25.1 -> 3.7, 512 x 1 10.0 -> 1.65,
 // 512 x 400 14.0 -> 5.1, 1024 x 1 11.5 -> 3.2, 1024 x 200 18.4 -> 6.3.
+#include "device_once.h"
 #include "step_common.cuh"
 
 namespace tdse {
@@ -287,13 +288,11 @@ __global__ void __launch_bounds__(Run1D64<N>::T, 1) k_run1d64(const __grid_const
 
 template <int N>
 cudaError_t go(const KArgs& a, const Run1DArgs& g, cudaStream_t s) {
-    static bool done = false;
-    if (!done) {
-        const cudaError_t e = cudaFuncSetAttribute(k_run1d64<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)Run1D64<N>::smem);
-        if (e != cudaSuccess) return e;
-        done = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = once([] {
+        return cudaFuncSetAttribute(k_run1d64<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Run1D64<N>::smem);
+    });
+    if (e != cudaSuccess) return e;
     k_run1d64<N><<<a.B, Run1D64<N>::T, Run1D64<N>::smem, s>>>(a, g);
     return cudaGetLastError();
 }
