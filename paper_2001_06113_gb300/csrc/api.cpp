@@ -148,7 +148,7 @@ static void plan_workspace(tdse_ctx* c) {
     if (c->four1d) {
         c->off.tw1d64 = take((size_t)c->n0 * 16);
         c->off.tw1d32 = take((size_t)c->n0 * 8);
-        c->off.tw1d32lo = take((size_t)c->n0 * 8);
+        take((size_t)c->n0 * 8);        // a table of older checkpoints, which keep their layout; nothing reads it
     }
     c->off.tw64_2 = take((size_t)(c->d == 3 ? c->n2 : 1) * 16);
     c->off.tw32_2 = take((size_t)(c->d == 3 ? c->n2 : 1) * 8);

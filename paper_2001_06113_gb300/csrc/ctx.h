@@ -77,7 +77,7 @@ struct tdse_ctx {
     struct {
         size_t uhat, ring, chain_uhat, chain_ring, aux, aux2, V0, V0f, tfac, phi, kin64, kinff, adv64, advff,
             q64, qff, e2d, k1lo, k1hi, a1d, tw64_0, tw32_0, tw64_1, tw32_1, tw32lo_0, tw32lo_1, tw64_2, tw32_2,
-            tw32lo_2, tw1d64, tw1d32, tw1d32lo, iv, tw128, res_sums,
+            tw32lo_2, tw1d64, tw1d32, iv, tw128, res_sums,
             res_rho, res_flags, res_ncorr, cl_tab, err, scratch, end, run_tab;
     } off{};
     // 2D mixed steps over CTA clusters (512^2): plan built at bind, used when

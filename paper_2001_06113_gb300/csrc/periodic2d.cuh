@@ -377,7 +377,7 @@ __global__ void __launch_bounds__((threads_2d<C, N1, L>()), (min_blocks_2d<C, N1
 // first inverse pass's inputs, through the implicit solve between the two
 // transforms, and stored to T2 from the last forward pass, so that a line
 // crosses shared memory four times instead of eleven and its group of threads
-// (a warp, part of one, or a few warps on a barrier of their own) never waits for
+// (part of a warp, or a CTA of its own) never waits for
 // the other lines.  As few lines per CTA as fill two warps, so that an SM refills
 // line by line.  us per Adams step, k_row_mid / 256 threads per CTA / this:
 // 5 x 128^3 376 / 339 / 339; 64 x 256^2 106.4 / 101.5 / 101.2; 16 x 512^2 112.6 /
@@ -386,13 +386,6 @@ __global__ void __launch_bounds__((threads_2d<C, N1, L>()), (min_blocks_2d<C, N1
 template <int N1> struct Row32 {
     static constexpr int T = N1 / 8;                       // threads per line
     static constexpr int L = 64 / T < 1 ? 1 : 64 / T;      // lines per CTA
-};
-template <int T, int L> struct LineSync {
-    using type = std::conditional_t<(T <= 32), WarpSync, std::conditional_t<L == 1, CtaSync, GroupSync>>;
-    static __device__ __forceinline__ type make(int line) {
-        if constexpr (std::is_same<type, GroupSync>::value) return GroupSync{1u + (unsigned)line, (unsigned)T};
-        else return type{};
-    }
 };
 template <int N1, int L>
 __global__ void __launch_bounds__((Row32<N1>::T * L), (1024 / (Row32<N1>::T * L) > 16 ? 16 : 1024 / (Row32<N1>::T * L)))
@@ -404,7 +397,8 @@ k_row32(const __grid_constant__ KArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int line = threadIdx.x / T, tid = threadIdx.x % T;
     float2* buf = reinterpret_cast<float2*>(smem_raw) + (size_t)line * fft_len<float2>(N1);
-    const auto sync = LineSync<T, L>::make(line);
+    static_assert(T <= 32 || L == 1, "a line is part of a warp, or alone in its CTA");
+    const std::conditional_t<(T <= 32), WarpSync, CtaSync> sync{};
     const int b = blockIdx.y, row = blockIdx.x * L + line;
     const size_t NP = (size_t)a.n0 * N1, base = (size_t)b * NP + (size_t)row * N1;
     const double vfac = a.tfac[(size_t)b * a.ntf + a.tf];
