@@ -219,6 +219,7 @@ static KArgs base_args(const tdse_ctx* c) {
     KArgs a{};
     a.B = c->B;
     a.overlap = 1;
+    a.beyond_l2 = (double)c->NP * c->B * 16.0 > 120e6;
     a.n0 = c->n0;
     a.n1 = c->n1;
     a.tn0 = c->n0;

@@ -30,6 +30,7 @@ struct KArgs {
     int overlap;              // pass kernels: may start while the launch before drains (one chain on the GPU;
                               // beside other chains its waiting CTAs would take their slots)
     int B;                    // instances in this launch
+    int beyond_l2;            // 2D: the intermediates of all instances exceed the L2
     int n0, n1;               // launch geometry: lines x line length (n1 = 1 for 1D); for 3D the
                               // column pass sees [n0][n1 n2] and the row pass [n0 n1][n2]
     int tn0, tn1, tn2;        // the grid per axis for the phase and E tables (tn2 = 0 below 3D)

@@ -381,7 +381,8 @@ __global__ void __launch_bounds__((threads_2d<C, N1, L>()), (min_blocks_2d<C, N1
 // the other lines.  As few lines per CTA as fill two warps, so that an SM refills
 // line by line.  us per Adams step, k_row_mid / 256 threads per CTA / this:
 // 5 x 128^3 376 / 339 / 339; 64 x 256^2 106.4 / 101.5 / 101.2; 16 x 512^2 112.6 /
-// 111.7 / 109.7; 64 x 512^2 459.5 / 470 / 463.6; 16 x 1024^2 727 / 682 / 641;
+// 111.7 / 109.7; 64 x 512^2 459.5 / 470 / 463.6 (takes k_row_mid, see row_mid_n); 16 x
+// 1024^2 727 / 682 / 641;
 // 512^2 16.5 / 15.7 / 15.7.
 template <int N1> struct Row32 {
     static constexpr int T = N1 / 8;                       // threads per line
@@ -816,14 +817,27 @@ static cudaError_t row32_n(const KArgs& a, cudaStream_t s) {
 
 template <class C, int N1>
 static cudaError_t row_mid_n(const KArgs& a, cudaStream_t s) {
-    if constexpr (is_f32<C>() && N1 >= 64) return row32_n<N1>(a, s);
-    else
-    return with_lanes<C>((long long)a.n0 * a.B, [&](auto l) {
-        constexpr int L = decltype(l)::value;
-        static DeviceOnce once;
-        return launch_pass(k_row_mid<C, N1, L>, dim3(a.n0 / L, a.B), threads_2d<C, N1, L>(), (size_t)N1 * (L + 1) * sizeof(C),
-                           once, s, a);
-    });
+    auto shared = [&] {
+        return with_lanes<C>((long long)a.n0 * a.B, [&](auto l) {
+            constexpr int L = decltype(l)::value;
+            static DeviceOnce once;
+            return launch_pass(k_row_mid<C, N1, L>, dim3(a.n0 / L, a.B), threads_2d<C, N1, L>(),
+                               (size_t)N1 * (L + 1) * sizeof(C), once, s, a);
+        });
+    };
+    // FP32 lines of 64 points and more in registers, with one exception (same bits):
+    // 512-point lines of 2D batches whose intermediates (16 B per point) are beyond the
+    // L2 (126 MB), where a row pass waits for HBM and the wide loads of the shared-memory
+    // pass do better.  us per Adams step, registers / shared memory: 64 x 512^2 (268 MB)
+    // 468.4 / 463.6, 64 x 256 x 512 (134 MB) 219.6 / 216.7, 512 x 64 x 512 493.8 / 491;
+    // within the L2 (100 MB) 24 x 512^2 159 / 170; n0 = 1024, x 32: 587 / 628; 3D lines equal.
+    if constexpr (is_f32<C>() && N1 == 512) {
+        return a.mode == MODE_STEP && a.beyond_l2 && a.tn2 == 0 && !a.flat1d && a.n0 <= 512 ? shared() : row32_n<N1>(a, s);
+    } else if constexpr (is_f32<C>() && N1 >= 64) {
+        return row32_n<N1>(a, s);
+    } else {
+        return shared();
+    }
 }
 
 #define TDSE_SWITCH_N(n, ...)                                \
