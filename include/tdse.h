@@ -377,6 +377,13 @@ tdse_status tdse_set_step_path(tdse_ctx* ctx, int path);
  * create the streams; take them before any stream capture. */
 tdse_status tdse_set_step_groups(tdse_ctx* ctx, int groups);
 
+/* Pass kernels (2D, 3D, four-step 1D): whether a pass of a context's own step
+ * chain may start while the pass before it drains (on by default; the same
+ * results).  Off is the better choice for TDSE_FP64 contexts that step beside
+ * others on streams of their own: the waiting CTAs hold slots that the others'
+ * passes could use.  A batch stepped in groups never overlaps. */
+tdse_status tdse_set_overlap(tdse_ctx* ctx, int on);
+
 /* 1D periodic TDSE_MIXED contexts of n <= 16384 (one CTA per instance):
  * launch shape of the step kernel.  Shape 0 (default): n/8 threads per
  * instance (32..1024); shape 1: for n = 8192 1024 threads (8 points each),

@@ -336,6 +336,12 @@ class Problem:
         parallel streams (same results; default 4)."""
         _check(self._lib.tdse_set_step_groups(self._ctx, int(groups)), self._ctx)
 
+    def set_overlap(self, on: bool):
+        """2D, 3D and four-step passes: whether a pass may start while the one
+        before it drains (default on, same results; off for FP64 problems that
+        step beside others on streams of their own)."""
+        _check(self._lib.tdse_set_overlap(self._ctx, int(bool(on))), self._ctx)
+
     def set_shape_1d(self, shape: int):
         """1D mixed contexts: launch shape of the step kernel (0: n/8 threads per
         instance, at most 512 below n = 16384; 1: 1024 threads for n = 8192, half

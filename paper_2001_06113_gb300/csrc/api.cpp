@@ -218,7 +218,7 @@ static std::vector<float> weight_table(const tdse_ctx* c) {
 static KArgs base_args(const tdse_ctx* c) {
     KArgs a{};
     a.B = c->B;
-    a.overlap = 1;
+    a.overlap = c->overlap;
     a.beyond_l2 = (double)c->NP * c->B * 16.0 > 120e6;
     a.n0 = c->n0;
     a.n1 = c->n1;
@@ -1355,6 +1355,12 @@ tdse_status tdse_set_step_path(tdse_ctx* c, int path) {
         return c->fail(TDSE_EUNSUPPORTED, "cluster step path: 2D periodic TDSE_MIXED 512 x 512 on a device that runs "
                                           "16-CTA clusters, after tdse_bind_workspace");
     c->step_path = path;
+    return TDSE_OK;
+}
+
+tdse_status tdse_set_overlap(tdse_ctx* c, int on) {
+    if (!c) return TDSE_EINVAL;
+    c->overlap = on ? 1 : 0;
     return TDSE_OK;
 }
 

@@ -91,6 +91,7 @@ struct tdse_ctx {
     // 64 x 512^2 mixed workload, 0.495 ms per step with one chain, 0.46 with
     // 2..16 groups.
     int step_groups = 4;
+    int overlap = 1;            // tdse_set_overlap
     std::vector<cudaStream_t> group_streams;
     std::vector<cudaEvent_t> group_join;
     cudaEvent_t group_fork = nullptr;

@@ -27,8 +27,8 @@ constexpr int E1D_NLO = 32;    // 1D absolute kinetic phase: e^{-i k^2 n dt} = K
 
 struct KArgs {
     int mode;
-    int overlap;              // pass kernels: may start while the launch before drains (one chain on the GPU;
-                              // beside other chains its waiting CTAs would take their slots)
+    int overlap;              // pass kernels: may start while the launch before drains (tdse_set_overlap; not for
+                              // the groups of a batch, see launch_pass)
     int B;                    // instances in this launch
     int beyond_l2;            // 2D: the intermediates of all instances exceed the L2
     int n0, n1;               // launch geometry: lines x line length (n1 = 1 for 1D); for 3D the

@@ -736,8 +736,12 @@ __global__ void __launch_bounds__((threads_2d<float2, N0, L>()), (min_blocks_2d<
 // Launch of a pass; with a.overlap it may start while the launch before it
 // drains (wait_previous: no pass reads anything of its predecessor before).
 // 128 x 256, one instance, 400 mixed steps 8.7 -> 5.3 ms, 1D 65536 points 10.1 ->
-// 6.6 (with the smaller CTAs); 4 x 512^2 in FP64 as four chains 31.8 -> 34.3 if
-// they overlapped too.
+// 6.6 (with the smaller CTAs).  Beside other chains the waiting CTAs take slots:
+// 4 x 512^2 in FP64 as four chains of one context 31.8 -> 34.3 ms, so groups do not
+// overlap.  Contexts on streams of their own, with / without, ms: mixed 16 x (128 x 256)
+// 13.9 / 16.2, 4 x 1024^2 24.85 / 24.8, 16 x 65536 points 17.2 / 17.7, 64 x 65536 59.0 / 58.6;
+// FP64 one 512^2 9.05 / 9.41, two 14.8 / 12.1, 8 x 256^2 19.1 / 17.9, 8 x 128^2 14.2 / 14.6:
+// on unless the caller says otherwise.
 template <class K, class... A>
 static cudaError_t launch_pass(K kern, dim3 grid, int threads, size_t smem, DeviceOnce& once, cudaStream_t s, const KArgs& a,
                                const A&... more) {
