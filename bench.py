@@ -189,13 +189,13 @@ def launches_per_solve(mixed: bool, path: str = "passes", groups: int = 1) -> in
 
 
 # DRAM bytes per point-step of the 2D step operator (k_row_mid + k_col_fused_ip)
-# from the ncu capture of the 512^2 mixed workload at batch 8 (summarised under
-# profiles/); traffic scales with the number of instances.  None = not captured
-# for the current kernels.
+# from an ncu capture of the 512^2 mixed workload at batch 8 with these kernels
+# (summarised under profiles/); traffic scales with the number of instances.
+# Batches whose intermediates fit the L2 take k_row32 instead (not captured).
 TRAFFIC_BYTES_PER_POINT_STEP = {("mixed", "passes"): 72.143 + 16.105}
 TRAFFIC_NOTE = {("mixed", "passes"): "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_col_fused_ip<512> + "
                 "k_row_mid<float2,512>, batch 8 in 4 groups (2 instances per launch), scaled by points: reads "
-                "72.1 + 16.1 B per point-step (re-taken on the current kernels); the state, history and intermediate writes (40 B) stayed in L2 "
+                "72.1 + 16.1 B per point-step; the state, history and intermediate writes (40 B) stayed in L2 "
                 "within that capture (profiles/step2d_512x512_mixed_fused.md)"}
 
 
@@ -272,13 +272,14 @@ def run_gpu(args, ws, rank, local):
     peak, peak_src = hbm_peak()
     achieved = algo / t_step / 1e9
     shape = prob.describe_steps()
-    tb = TRAFFIC_BYTES_PER_POINT_STEP.get((args.precision, shape["path"]))
+    row_mid = 16 * B * points > 120e6        # intermediates beyond the L2: the shared-memory row pass
+    tb = TRAFFIC_BYTES_PER_POINT_STEP.get((args.precision, shape["path"])) if row_mid else None
     traffic = None if tb is None else round(tb * B * points)
     kname = {"cluster": "k_step2d_cluster (one 16-CTA cluster per instance, a run of steps per launch)",
-             "passes": "k_row32 + k_col_fused_ip" if args.precision == "mixed" else "k_row_mid + k_col_end (FP64)"}
+             "passes": ("k_row_mid" if row_mid else "k_row32") + " + k_col_fused_ip" if args.precision == "mixed" else "k_row_mid + k_col_end (FP64)"}
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic, "traffic_unit": "bytes per step (all instances)",
-                "traffic_note": TRAFFIC_NOTE.get((args.precision, shape["path"])),
+                "traffic_note": TRAFFIC_NOTE.get((args.precision, shape["path"])) if row_mid else None,
                 "peak_source": peak_src,
                 "kernel": f"2D Adams step operator: {kname[shape['path']]}, timed over groups of {GROUP} steps",
                 "launch_shape": shape,
