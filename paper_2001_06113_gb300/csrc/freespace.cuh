@@ -567,7 +567,7 @@ __device__ __forceinline__ double2 to_c(double2 v, double2) { return v; }
 
 __device__ __forceinline__ double2 widen(float2 x) { return fx_widen(x); }
 __device__ __forceinline__ double2 widen(double2 x) { return x; }
-template <class C> constexpr double widen_factor() { return std::is_same<C, float2>::value ? FX_WIDEN : 1.0; }
+template <class C> constexpr int widens() { return std::is_same<C, float2>::value ? 1 : 0; }     // index of up_h, up_hmu0
 // v * (-i c) added to u
 __device__ __forceinline__ double2 add_minus_i(double2 u, double c, double2 v) {
     return make_double2(fma(c, v.y, u.x), fma(-c, v.x, u.y));
@@ -724,14 +724,14 @@ __device__ __forceinline__ double2 update_mode(const FsArgs& a, int g, const int
     }
     if (end) {
         p.out[m] = F;
-        u = add_minus_i(u, a.h * a.mu[0] * widen_factor<C>(), widen(F));
+        u = add_minus_i(u, a.up_hmu0[widens<C>()], widen(F));
         if (!begin) {
             p.uh[m] = u;
             return u;
         }
         if (p.first_is_new) r[0] = F;
     }
-    const double2 X = add_minus_i(u, a.h * widen_factor<C>(), widen(history<WIDE>(a, g, c, r, p.pc, m)));
+    const double2 X = add_minus_i(u, a.up_h[widens<C>()], widen(history<WIDE>(a, g, c, r, p.pc, m)));
     double2 W;
     if constexpr (!WIDE) {
         const unsigned mx = fx_hi(X);

@@ -359,6 +359,11 @@ void set_weights(FsArgs& a, double h, const double* mu, int n) {
     auto factor = [](double x, int2& w) { fx_limbs(std::llround(std::ldexp(x, 61)), w.x, w.y); };
     a.nhist = n;
     a.h = h;
+    const double f[2] = {1.0, FX_WIDEN};
+    for (int i = 0; i < 2; ++i) {
+        a.up_h[i] = h * f[i];
+        a.up_hmu0[i] = h * mu[0] * f[i];
+    }
     for (int j = 0; j <= n; ++j) {
         a.mu[j] = mu[j];
         factor(0.5 * mu[j], a.mu_w[j]);

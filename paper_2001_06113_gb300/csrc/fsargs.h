@@ -95,6 +95,7 @@ struct FsArgs {
     int nhist;             // history terms j = 1..nhist
     double h;              // step size
     double mu[FS_MAX_HIST + 1];
+    double up_h[2], up_hmu0[2];   // h and h mu_0 for the mode update; [1]: times FX_WIDEN (FP32 transforms)
     int2 mu_w[FS_MAX_HIST + 1];   // mu_j / 2 as fixed-point factors
     const int* g;          // [B] extra powers of two in the scale of P (0 unless the phases' moduli are large)
     int hist_slot[FS_MAX_HIST];   // ring slot of lag j (index j-1)

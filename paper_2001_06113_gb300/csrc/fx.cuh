@@ -147,6 +147,9 @@ FX_HD int4 fx_ldg(const int4* p) {
 #endif
 }
 
+// Factor of fx_widen's results.
+constexpr double FX_WIDEN = 0x1p896;
+
 // ---- device side
 #ifdef __CUDACC__
 __device__ __forceinline__ unsigned fx_hi(double2 v) {
@@ -187,7 +190,6 @@ __device__ __forceinline__ float2 fx_to_float(double2 v) { return make_float2(fx
 // FP32 -> FP64 times 1 / FX_WIDEN in integer arithmetic: with the exponent field
 // as it is, zeros, subnormals and normal numbers move alike.  What multiplies
 // the result takes the factor FX_WIDEN, which changes no rounding.
-constexpr double FX_WIDEN = 0x1p896;
 __device__ __forceinline__ double2 fx_widen(float2 v) {
     auto one = [](float f) {
         const unsigned x = __float_as_uint(f), a = x & 0x7fffffffu;
