@@ -6,12 +6,13 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-def test_pulse_set_in_a_captured_graph():
+@pytest.mark.parametrize("A0", [150.0, 400.0])       # scale 3; FP64 phases
+def test_pulse_set_in_a_captured_graph(A0):
     import torch
     import synth
     from paper_2001_06113_gb300 import Problem
     n, H = 6, 2.0
-    strong = synth.free_bump_gaussians((64,), seed=2, dt=1e-3, nsteps=n, A0=150.0)
+    strong = synth.free_bump_gaussians((64,), seed=2, dt=1e-3, nsteps=n, A0=A0)
     q = strong.pulse
 
     def solve(p):
@@ -86,3 +87,37 @@ def test_strong_field_matches_oracle(d, M, H, r, g, precision):
         assert rel(got_u, u) <= tol_u
     flags = len(blob) - struct.unpack_from("<Q", blob, 88)[0] - 4      # two instances, two bytes each
     assert (blob[flags] >> 1) - 1 == 0 and (blob[flags + 2] >> 1) - 1 == g
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_fp64_phases_alone_in_a_batch_and_resumed(precision):
+    import synth
+    from paper_2001_06113_gb300 import Problem
+    n = 8
+    weak, strong = (synth.free_bump_gaussians((64,), seed=s, dt=1e-3, nsteps=n, A0=a) for s, a in ((1, 1.0), (2, 400.0)))
+
+    def problem(batch=1):
+        return Problem((64,), 1e-3, n, order=4, batch=batch, bc="free", nu=(512,), H=2.0, precision=precision)
+
+    def setup(p, inst, i=-1):
+        q = inst.pulse
+        p.set_potential(inst.V0, instance=i)
+        p.set_pulse(q.A0, q.omega, q.T_pulse, q.direction, instance=i)
+        p.set_initial(inst.u0, instance=i)
+
+    with problem(2) as p:
+        setup(p, weak, 0)
+        setup(p, strong, 1)
+        p.step(n)
+        both = p.read_u()
+    for i, inst in enumerate((weak, strong)):
+        with problem() as p:
+            setup(p, inst)
+            p.step(5)
+            blob = p.save()
+            p.step(3)
+            assert np.array_equal(p.read_u(0), both[i])
+        with problem() as p:
+            p.load(blob)
+            p.step(3)
+            assert np.array_equal(p.read_u(0), both[i])
